@@ -78,7 +78,8 @@ typedef struct {
   double tol;          /* natural-residual tolerance of each step, > 0 */
   int nu1, nu2;        /* pre/post projected smoothing sweeps of the V-cycle, >= 0, nu1+nu2 >= 1 */
   int max_cycles;      /* V-cycle cap per step, >= 1 */
-  int coarse_min;      /* coarsen while both cell counts are even and min/2 >= coarse_min (>= 1) */
+  int coarse_min;      /* coarsen (W, H) to ((W + 1)/2, (H + 1)/2) while the smaller of the two stays >= coarse_min
+                          (>= 1) and the level is not yet mass-dominated (8 tau eps > 4 h^2 on its cells of side h) */
   int precision;       /* AC_FP64: every array and operation of the solve in FP64.
                           AC_MIXED: FP64 state u and its update; right-hand side, colour
                           means, energy and residual r = b - S u of the defect correction in

@@ -209,8 +209,22 @@ constexpr double kTiledFreeFraction = 0.25;
 #endif
 constexpr int kCoarseSweeps = AC_COARSE_SWEEPS;
 static_assert(kCoarseSweeps >= 2 && kCoarseSweeps % 2 == 0, "coarse sweeps: an even count >= 2");
-constexpr int kCoarsestSweeps = 20;  // sweeps of the one-block coarsest solve
-constexpr int64_t kCoarsestBlockNodes = 1 << 14;
+// Level k (cell side h = 2^k) is mass-dominated when 8 tau eps <= kMassRatio
+// h^2.  On cells of side h the Galerkin operator is about h^2 (consistent
+// mass) + tau eps A with A <= 8, so its condition number is at most a small
+// multiple of 1 + kMassRatio there and kDominatedSweeps Gauss-Seidel sweeps
+// are as good as any coarser grid: cycles per solve with all levels / up to
+// this rule's at 4096^2 N = 8 (eps 3) 12 / 12, 1024^2 N = 4 11 / 11,
+// 1001 x 751 13 / 12; one level less (8 tau eps = 16 h^2) takes 22, 25 and 28.
+// The levels below cost launches and the serial one-block tail: 1024^2, N = 4
+// 3.73 ms a step with all levels, 2.21 ms with two coarse levels (eps 2).
+constexpr double kMassRatio = 4.0;
+bool mass_dominated(double te, int level) { return 8.0 * te <= kMassRatio * std::ldexp(1.0, 2 * level); }
+// Sweeps on the coarsest level, in the tail and in tile launches (a pair
+// each); a hierarchy that ends early (coarse_min, a tuned depth) leaves a
+// system that is not mass-dominated.
+constexpr int kDominatedTailSweeps = 6, kDominatedSweeps = 4, kCoarsestSweeps = 20;
+bool ends_dominated(const Solve &S) { return mass_dominated(S.lv[0].g.te, S.depth - 1); }
 // AC_MIXED: inner FP32 solve to max(0.9 tol, 1e-5 rho_outer) ...  The inner
 // natural residual and the outer one agree to about 0.1% at tol 1e-6 (float
 // rounding of S delta against rho), so 0.9 tol still passes the outer check
@@ -600,19 +614,16 @@ int coarse_vcycle(ac_ctx *ctx, Solve &S, int k, void **res) {
       a.op[l] = S.lv[k + l].op;
       ops += 4.0 * (double)S.lv[k + l].n * ns;
     }
-    AC_RUNB(AC_PROF_COARSE, ops + 2 * lk, o->coarse_tail(a, L.r, L.v, kCoarseSweeps, kCoarsestSweeps, smem, S.coarse_gs, ctx->s));
+    AC_RUNB(AC_PROF_COARSE, ops + 2 * lk, o->coarse_tail(a, L.r, L.v, kCoarseSweeps,
+                                                      ends_dominated(S) ? kDominatedTailSweeps : kCoarsestSweeps, smem, S.coarse_gs, ctx->s));
     *res = L.v;
     return AC_OK;
   }
   if (k == S.depth - 1) {
-    if (L.n <= kCoarsestBlockNodes) {
-      AC_CUDA(cudaMemsetAsync(L.v, 0, (size_t)L.n * ctx->N * o->elem, ctx->s));
-      AC_RUNB(AC_PROF_COARSE, 6 * lk, o->coarse_solve(L.op, L.r, L.v, L.g, kCoarsestSweeps, ctx->s));
-      *res = L.v;
-    } else {
-      AC_RUNB(AC_PROF_COARSE, pair0 + (kCoarseSweeps - 1) * pair,
-              o->coarse_smooth(L.op, L.r, L.v, L.t, L.g, 2 * kCoarseSweeps, true, res, nullptr, S.coarse_gs, ctx->s));
-    }
+    // the coarsest level (a Gauss-Seidel sweep is worth two of l1-Jacobi)
+    const int sweeps = !ends_dominated(S) ? kCoarsestSweeps : S.coarse_gs ? kDominatedSweeps : 2 * kDominatedSweeps;
+    AC_RUNB(AC_PROF_COARSE, pair0 + (sweeps / 2 - 1) * pair,
+            o->coarse_smooth(L.op, L.r, L.v, L.t, L.g, sweeps, true, res, nullptr, S.coarse_gs, ctx->s));
     return AC_OK;
   }
   Level &C = S.lv[k + 1];
@@ -1469,9 +1480,18 @@ int ac_create(ac_ctx **out, const ac_params *p) {
   int W = p->width, H = p->height;
   ctx->g0 = make_geo(W, H, te);
   S.lv.push_back(Level{ctx->g0, (int64_t)(W + 1) * (H + 1)});
-  while (W % 2 == 0 && H % 2 == 0 && (W < H ? W : H) / 2 >= p->coarse_min) {
-    W /= 2;
-    H /= 2;
+  // An odd side W coarsens to (W + 1) / 2 cells: the last coarse nodes then
+  // lie one fine cell outside the grid and act through the fine nodes under
+  // their hats that are inside (every kernel drops the others, and stored
+  // couplings to them are 0), so P'SP stays positive definite.  Halving even
+  // sides only left 1001 x 751, N = 5 without a coarse level: 90 cycles of
+  // plain sweeps to 1e-12 in 6.08 ms, against 13 cycles in 3.68 ms.
+  // Coarsening stops at the first level whose system the mass dominates
+  // (kMassRatio): a few sweeps solve that one.
+  while ((W < H ? W : H) >= 2 && ((W < H ? W : H) + 1) / 2 >= p->coarse_min &&
+         !mass_dominated(te, (int)S.lv.size() - 1)) {
+    W = (W + 1) / 2;
+    H = (H + 1) / 2;
     Level L;
     L.g = make_geo(W, H, te);
     L.n = (int64_t)(W + 1) * (H + 1);

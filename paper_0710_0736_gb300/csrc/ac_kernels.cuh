@@ -2028,59 +2028,6 @@ __global__ void __launch_bounds__(GS ? kGsThreads : kJ2Threads, pair_min_blocks(
   });
 }
 
-// Whole-level Gauss-Seidel in one block for small coarsest grids: `sweeps`
-// passes over 3 colours ((x + y) % 3 is a valid colouring of the 7-point
-// E, W, N, S, NE, SW pattern) with a barrier between colours.
-template <typename T, int N>
-__global__ void __launch_bounds__(1024) k_coarse_solve_block(const T *__restrict__ op, const T *__restrict__ r,
-                                                             T *__restrict__ v, Geo g, int sweeps) {
-  const int64_t nc = (int64_t)g.Wn * (g.H + 1);
-  for (int s = 0; s < sweeps; ++s)
-    for (int color = 0; color < 3; ++color) {
-      for (int64_t k = threadIdx.x; k < nc; k += blockDim.x) {
-        const int x = (int)(k % g.Wn), y = (int)(k / g.Wn);
-        if ((x + y) % 3 != color) continue;
-#pragma unroll
-        for (int i = 0; i < N; ++i) {
-          const T d = op[i * nc + k];
-          v[i * nc + k] = d > T(0) ? (r[i * nc + k] - op_offdiag<T, N>(op, v, g, nc, x, y, i)) / d : T(0);
-        }
-      }
-      __syncthreads();
-    }
-}
-
-// The same Gauss-Seidel for coarsest grids that fit in shared memory: the
-// operator, right-hand side and iterate are staged on chip and each thread
-// updates (node, phase) items of the current colour.  Dynamic shared memory:
-// 6 N nc values of T.
-template <typename T, int N>
-__global__ void __launch_bounds__(1024) k_coarse_solve_smem(const T *__restrict__ op, const T *__restrict__ r,
-                                                            T *__restrict__ v, Geo g, int sweeps) {
-  extern __shared__ unsigned char smem_raw[];
-  T *sop = reinterpret_cast<T *>(smem_raw);
-  const int nc = g.Wn * (g.H + 1);
-  T *sr = sop + 4 * N * nc, *sv = sr + N * nc;
-  for (int t = threadIdx.x; t < 4 * N * nc; t += blockDim.x) sop[t] = op[t];
-  for (int t = threadIdx.x; t < N * nc; t += blockDim.x) {
-    sr[t] = r[t];
-    sv[t] = T(0);
-  }
-  __syncthreads();
-  for (int s = 0; s < sweeps; ++s)
-    for (int color = 0; color < 3; ++color) {
-      for (int t = threadIdx.x; t < N * nc; t += blockDim.x) {
-        const int i = t / nc, k = t - i * nc;
-        const int x = k % g.Wn, y = k / g.Wn;
-        if ((x + y) % 3 != color) continue;
-        const T d = sop[i * nc + k];
-        sv[t] = d > T(0) ? (sr[t] - op_offdiag<T, N>(sop, sv, g, nc, x, y, i)) / d : T(0);
-      }
-      __syncthreads();
-    }
-  for (int t = threadIdx.x; t < N * nc; t += blockDim.x) v[t] = sv[t];
-}
-
 // ---------------------------------------------------------------------------
 // The bottom of the coarse V-cycle in one launch.  Below some level k0 the
 // levels are small (at most a few thousand nodes) and each of their kernels

@@ -164,17 +164,6 @@ struct SolverLaunch {
                               bool gs, cudaStream_t s) {
     return gs ? coarse_pre_resid_t<true>(op, r, v, t, g, L, s) : coarse_pre_resid_t<false>(op, r, v, t, g, L, s);
   }
-  static int coarse_solve(const void *op, const void *r, void *v, const Geo &g, int sweeps, cudaStream_t s) {
-    const int64_t nc = (int64_t)g.Wn * (g.H + 1);
-    const size_t smem = (size_t)6 * N * nc * sizeof(T);
-    if (smem <= 48 * 1024) {
-      const int threads = (int)std::min<int64_t>(1024, ((N * nc + 31) / 32) * 32);
-      k_coarse_solve_smem<T, N><<<1, threads, smem, s>>>((const T *)op, (const T *)r, (T *)v, g, sweeps);
-    } else {
-      k_coarse_solve_block<T, N><<<1, 1024, 0, s>>>((const T *)op, (const T *)r, (T *)v, g, sweeps);
-    }
-    return 1;
-  }
   static int coarse_resid(const void *op, const void *r, const void *v, const Geo &g, void *t, const LevelLists *Lv,
                           cudaStream_t s) {
     if (Lv) {
@@ -244,7 +233,7 @@ struct SolverLaunch {
   }
   static SolverOps table() {
     return SolverOps{(int)sizeof(T), smooth,       resid,        restrict0,   galerkin0,   galerkin,   coarse_smooth,
-                     coarse_solve,   coarse_resid, coarse_pre_resid, restrict_, prolong_add, coarse_tail,
+                     coarse_resid, coarse_pre_resid, restrict_, prolong_add, coarse_tail,
                      line_search};
   }
 };

@@ -79,7 +79,6 @@ struct SolverOps {
   // 3-colour Gauss-Seidel on shared-memory tiles, else l1-Jacobi
   int (*coarse_smooth)(const void *op, const void *r, void *v, void *tmp, const Geo &g, int sweeps, bool zero_start,
                        void **out, const LevelLists *L, bool gs, cudaStream_t s);
-  int (*coarse_solve)(const void *op, const void *r, void *v, const Geo &g, int sweeps, cudaStream_t s);
   int (*coarse_resid)(const void *op, const void *r, const void *v, const Geo &g, void *t, const LevelLists *L,
                       cudaStream_t s);
   // one pair of smoothing sweeps from v = 0, then t = r - S v
