@@ -560,7 +560,9 @@ int tail_level(const Solve &S, size_t *smem) {
   size_t bytes = 0;
   int k0 = S.depth;
   for (int k = S.depth - 1; k >= 1; --k) {
-    const size_t b = bytes + (size_t)ac::kTailArrays * (size_t)S.lv[k].n * (size_t)S.o->elem;
+    const ac::Geo &g = S.lv[k].g;
+    if ((int64_t)(g.W + ac::kTailFrame) * (g.H + ac::kTailFrame) > (int64_t)ac::kTailSmemBytes) break;
+    const size_t b = bytes + (size_t)ac::kTailArrays * (size_t)ac::tail_nodes_framed(g.W, g.H) * (size_t)S.o->elem;
     if (b > ac::kTailSmemBytes || S.depth - k > ac::kTailMaxLevels) break;
     bytes = b;
     k0 = k;
@@ -711,7 +713,10 @@ int enqueue_correction(ac_ctx *ctx, Solve &S) {
   if (tiled_end(S) > 1) AC_CUDA(cudaMemsetAsync(S.list_counts, 0, 2 * S.lv.size() * sizeof(int), ctx->s));
   AC_RUNB(AC_PROF_TRANSFER, bm.n + 4 * l1,
           o->galerkin0(S.mask, g0, L1.g, S.tab0, L1.op, level_lists(S, 1), L1.lists.dirty, ctx->s));
-  for (int k = 1; k + 1 < S.depth; ++k)
+  // (the float tail forms those below its first level itself)
+  size_t tail_smem = 0;
+  const int k0 = tail_level(S, &tail_smem), top = o->elem == 4 && k0 < S.depth - 1 ? k0 : S.depth - 1;
+  for (int k = 1; k < top; ++k)
     AC_RUNB(AC_PROF_TRANSFER, 4.0 * (double)(S.lv[k].n + S.lv[k + 1].n) * bm.ns,
             o->galerkin(S.lv[k].op, S.lv[k].g, S.lv[k + 1].g, S.lv[k + 1].op, level_lists(S, k), level_lists(S, k + 1),
                         ctx->s));

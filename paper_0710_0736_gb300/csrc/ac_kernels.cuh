@@ -2031,192 +2031,261 @@ __global__ void __launch_bounds__(GS ? kGsThreads : kJ2Threads, pair_min_blocks(
 // ---------------------------------------------------------------------------
 // The bottom of the coarse V-cycle in one launch.  Below some level k0 the
 // levels are small (at most a few thousand nodes) and each of their kernels
-// is latency-bound, about 7 us for tiny grids.  One block per phase stages
-// the operators of levels k0 .. depth-1 and r of level k0 in shared memory
-// and runs the same cycle there: kCoarseSweeps l1-Jacobi sweeps from zero,
-// residual, restriction, ..., Gauss-Seidel on the coarsest level,
-// prolongation and kCoarseSweeps l1-Jacobi sweeps back up.  v of level k0
-// is written once.  Only W, H of each level and its operator are needed.
+// would be latency-bound.  One block per phase stages r and the operator of
+// level k0 in shared memory, forms the coarser levels' operators there
+// (float; FP64 blocks load them, see k_coarse_tail) and runs the same cycle:
+// kCoarseSweeps sweeps from zero, residual, restriction, ..., Gauss-Seidel on
+// the coarsest level, prolongation and kCoarseSweeps sweeps back up.  v of
+// level k0 is written once.  Only W, H of each level and its operator are
+// needed.
+//
+// The block is bound by the latency of its serial chain of colour passes
+// (shared-memory loads, six multiply-adds, a barrier), so a pass must do
+// nothing else: every array has a frame of zeros around the level (one node
+// west and south, two east and north, which an odd side's hats reach), so no
+// sum tests its range; the reciprocal diagonal is staged (0 on dead rows,
+// which then keep v = 0); and a thread walks its nodes of a colour -- node x
+// of row y has colour (x + y) mod 3, so they are x = 3 j + m, j < W / 3 + 1
+// -- by additions.  With a modulo and a division per node, a test per
+// neighbour and a third of the threads at work in a pass the same cycle took
+// 89 us on 65^2 + 33^2 nodes (float) and 109 us on 33^2 + 17^2 (FP64).
 // ---------------------------------------------------------------------------
 constexpr int kTailThreads = 1024;
 
-// Shared-memory view of one level of one phase.
+// Shared-memory view of one level of one phase: the arrays point at node
+// (0, 0), rows are P apart.
 template <typename T>
 struct TailLevel {
-  int W, H, Wn, n;
-  T *C, *E, *Nn, *NE, *r, *v, *t;
+  int W, H, P;
+  T *C, *I, *E, *Nn, *NE, *r, *v, *t;  // I = 1 / C (0 on dead rows)
 };
+
+// A thread's nodes of one colour on one level: item (row, j), stepped by the
+// block's threads.
+struct TailWalk {
+  int row, j, drow, dj, J;
+  __device__ __forceinline__ TailWalk(int W) {
+    J = W / 3 + 1;
+    row = (int)threadIdx.x / J;
+    j = (int)threadIdx.x - row * J;
+    drow = (int)blockDim.x / J;
+    dj = (int)blockDim.x - drow * J;
+  }
+};
+
+template <typename T, class F>
+__device__ __forceinline__ void tail_colour(const TailLevel<T> &L, const TailWalk &w, int colour, F &&update) {
+  int row = w.row, j = w.j;
+  while (row <= L.H) {
+    const int x = 3 * j + (colour + 2 * row) % 3;  // x + row = colour (mod 3)
+    if (x <= L.W) update(row * L.P + x);
+    row += w.drow;
+    j += w.dj;
+    if (j >= w.J) {
+      j -= w.J;
+      ++row;
+    }
+  }
+}
+
+// Every node of the level, body(k, x, y).
+template <typename T, class F>
+__device__ __forceinline__ void tail_nodes(const TailLevel<T> &L, F &&body) {
+  const int Wn = L.W + 1;
+  int y = (int)threadIdx.x / Wn, x = (int)threadIdx.x - y * Wn;
+  const int dy = (int)blockDim.x / Wn, dx = (int)blockDim.x - dy * Wn;
+  while (y <= L.H) {
+    body(y * L.P + x, x, y);
+    y += dy;
+    x += dx;
+    if (x >= Wn) {
+      x -= Wn;
+      ++y;
+    }
+  }
+}
 
 // sum over the six off-diagonal neighbours (E, W, N, S, NE, SW) of S_Km v_m
 template <typename T>
-__device__ __forceinline__ T tail_offdiag(const TailLevel<T> &L, const T *v, int k, int x, int y, T &l1) {
-  T s = T(0), c;
-  if (x < L.W) { c = L.E[k]; s += c * v[k + 1]; l1 += fabs(c); }
-  if (x > 0) { c = L.E[k - 1]; s += c * v[k - 1]; l1 += fabs(c); }
-  if (y < L.H) { c = L.Nn[k]; s += c * v[k + L.Wn]; l1 += fabs(c); }
-  if (y > 0) { c = L.Nn[k - L.Wn]; s += c * v[k - L.Wn]; l1 += fabs(c); }
-  if (x < L.W && y < L.H) { c = L.NE[k]; s += c * v[k + L.Wn + 1]; l1 += fabs(c); }
-  if (x > 0 && y > 0) { c = L.NE[k - L.Wn - 1]; s += c * v[k - L.Wn - 1]; l1 += fabs(c); }
+__device__ __forceinline__ T tail_offdiag(const TailLevel<T> &L, const T *v, int k) {
+  T s = L.E[k] * v[k + 1];
+  s += L.E[k - 1] * v[k - 1];
+  s += L.Nn[k] * v[k + L.P];
+  s += L.Nn[k - L.P] * v[k - L.P];
+  s += L.NE[k] * v[k + L.P + 1];
+  s += L.NE[k - L.P - 1] * v[k - L.P - 1];
   return s;
+}
+
+// `sweeps` Gauss-Seidel sweeps on v in place, the colours forward (0, 1, 2)
+// in even sweeps and backward in odd ones (as the tiles of k_coarse_pair).
+// The colour that ends one sweep starts the next: its second pass would
+// repeat the first one's values, and is left out.
+template <typename T>
+__device__ __forceinline__ void tail_sgs(const TailLevel<T> &L, int sweeps) {
+  const TailWalk w(L.W);
+  for (int s = 0; s < sweeps; ++s)
+    for (int q = s > 0 ? 1 : 0; q < 3; ++q) {
+      tail_colour(L, w, (s & 1) ? 2 - q : q,
+                  [&](int k) { L.v[k] = (L.r[k] - tail_offdiag(L, L.v, k)) * L.I[k]; });
+      __syncthreads();
+    }
 }
 
 // one l1-Jacobi sweep vout = vin + (r - S vin) / l1 (vin = 0 when null);
 // rows with a zero diagonal give 0
 template <typename T>
 __device__ __forceinline__ void tail_jacobi(const TailLevel<T> &L, const T *vin, T *vout) {
-  for (int k = threadIdx.x; k < L.n; k += blockDim.x) {
+  tail_nodes(L, [&](int k, int, int) {
     const T d = L.C[k];
     if (!(d > T(0))) {
       vout[k] = T(0);
-      continue;
+      return;
     }
-    const int x = k % L.Wn, y = k / L.Wn;
-    T l1 = fabs(d), sv = T(0);
-    if (vin) {
-      sv = d * vin[k] + tail_offdiag(L, vin, k, x, y, l1);
-    } else {
-      if (x < L.W) l1 += fabs(L.E[k]);
-      if (x > 0) l1 += fabs(L.E[k - 1]);
-      if (y < L.H) l1 += fabs(L.Nn[k]);
-      if (y > 0) l1 += fabs(L.Nn[k - L.Wn]);
-      if (x < L.W && y < L.H) l1 += fabs(L.NE[k]);
-      if (x > 0 && y > 0) l1 += fabs(L.NE[k - L.Wn - 1]);
-    }
+    T l1 = fabs(d);
+    l1 += fabs(L.E[k]);
+    l1 += fabs(L.E[k - 1]);
+    l1 += fabs(L.Nn[k]);
+    l1 += fabs(L.Nn[k - L.P]);
+    l1 += fabs(L.NE[k]);
+    l1 += fabs(L.NE[k - L.P - 1]);
+    const T sv = vin ? d * vin[k] + tail_offdiag(L, vin, k) : T(0);
     vout[k] = (vin ? vin[k] : T(0)) + (L.r[k] - sv) / l1;
-  }
+  });
 }
 
-// t = r - S v (0 on rows with a zero diagonal)
+// t = r - S v (0 on rows with a zero diagonal, where r, v and the couplings are 0)
 template <typename T>
 __device__ __forceinline__ void tail_resid(const TailLevel<T> &L) {
-  for (int k = threadIdx.x; k < L.n; k += blockDim.x) {
-    const T d = L.C[k];
-    if (!(d > T(0))) {
-      L.t[k] = T(0);
-      continue;
-    }
-    const int x = k % L.Wn, y = k / L.Wn;
-    T l1 = T(0);
-    L.t[k] = L.r[k] - d * L.v[k] - tail_offdiag(L, L.v, k, x, y, l1);
-  }
+  tail_nodes(L, [&](int k, int, int) { L.t[k] = L.r[k] - L.C[k] * L.v[k] - tail_offdiag(L, L.v, k); });
 }
 
 // r_c = P' t (weights 1 at 2K, 1/2 at its E, W, N, S, NE, SW fine
-// neighbours; 0 on coarse rows with a zero diagonal)
+// neighbours; 0 on coarse rows with a zero diagonal, under which t = 0)
 template <typename T>
 __device__ __forceinline__ void tail_restrict(const TailLevel<T> &F, const TailLevel<T> &Cc) {
-  constexpr int dx[7] = {0, 1, -1, 0, 0, 1, -1};
-  constexpr int dy[7] = {0, 0, 0, 1, -1, 1, -1};
-  for (int K = threadIdx.x; K < Cc.n; K += blockDim.x) {
-    if (!(Cc.C[K] > T(0))) {
-      Cc.r[K] = T(0);
-      continue;
-    }
-    const int X = K % Cc.Wn, Y = K / Cc.Wn;
-    T acc = T(0);
-#pragma unroll
-    for (int s = 0; s < 7; ++s) {
-      const int ax = 2 * X + dx[s], ay = 2 * Y + dy[s];
-      if (ax < 0 || ax > F.W || ay < 0 || ay > F.H) continue;
-      acc += (s == 0 ? T(1) : T(0.5)) * F.t[ay * F.Wn + ax];
-    }
+  tail_nodes(Cc, [&](int K, int X, int Y) {
+    const T *t = F.t + 2 * Y * F.P + 2 * X;
+    T acc = t[0];
+    acc += T(0.5) * t[1];
+    acc += T(0.5) * t[-1];
+    acc += T(0.5) * t[F.P];
+    acc += T(0.5) * t[-F.P];
+    acc += T(0.5) * t[F.P + 1];
+    acc += T(0.5) * t[-F.P - 1];
     Cc.r[K] = acc;
-  }
+  });
 }
 
-// v_f += P v_c on rows with a nonzero diagonal (odd-odd fine nodes sit on
-// the coarse SW-NE diagonal)
+// v_f += P v_c (odd-odd fine nodes sit on the coarse SW-NE diagonal; dead
+// rows included: the sweep that follows returns them to 0, and until then
+// their couplings are 0)
 template <typename T>
 __device__ __forceinline__ void tail_prolong(const TailLevel<T> &F, const TailLevel<T> &Cc) {
-  for (int k = threadIdx.x; k < F.n; k += blockDim.x) {
-    if (!(F.C[k] > T(0))) continue;
-    const int x = k % F.Wn, y = k / F.Wn;
-    const int K0 = (y >> 1) * Cc.Wn + (x >> 1);
-    T p = Cc.v[K0];
-    if ((x & 1) || (y & 1)) p = T(0.5) * (p + Cc.v[K0 + (x & 1) + (y & 1) * Cc.Wn]);
+  tail_nodes(F, [&](int k, int x, int y) {
+    const T *c = Cc.v + (y >> 1) * Cc.P + (x >> 1);
+    T p = c[0];
+    if ((x & 1) || (y & 1)) p = T(0.5) * (p + c[(x & 1) + (y & 1) * Cc.P]);
     F.v[k] += p;
-  }
+  });
 }
 
-// Gauss-Seidel in three colours ((x + y) % 3 colours the 7-point pattern)
-// from v = 0 on the coarsest level
+// The operator of Cc from that of F, S_c = P' S_f P, both in shared memory:
+// galerkin_phase's sums, in its order, over the frame of zeros.  A hat's
+// fine nodes reach one node past the frame's first one only with weight 0.
 template <typename T>
-__device__ __forceinline__ void tail_gs(const TailLevel<T> &L, int sweeps) {
-  for (int k = threadIdx.x; k < L.n; k += blockDim.x) L.v[k] = T(0);
-  __syncthreads();
-  for (int s = 0; s < sweeps; ++s)
-    for (int color = 0; color < 3; ++color) {
-      for (int k = threadIdx.x; k < L.n; k += blockDim.x) {
-        const int x = k % L.Wn, y = k / L.Wn;
-        if ((x + y) % 3 != color) continue;
-        const T d = L.C[k];
-        T l1 = T(0);
-        L.v[k] = d > T(0) ? (L.r[k] - tail_offdiag(L, L.v, k, x, y, l1)) / d : T(0);
+__device__ __forceinline__ void tail_galerkin(const TailLevel<T> &F, const TailLevel<T> &Cc) {
+  constexpr int sx[7] = {0, 1, -1, 0, 0, 1, -1};
+  constexpr int sy[7] = {0, 0, 0, 1, -1, 1, -1};
+  constexpr int lx[4] = {0, 1, 0, 1};
+  constexpr int ly[4] = {0, 0, 1, 1};
+  tail_nodes(Cc, [&](int K, int X, int Y) {
+    T c4[4] = {T(0), T(0), T(0), T(0)};
+    const int a0 = 2 * Y * F.P + 2 * X;
+#pragma unroll
+    for (int s = 0; s < 7; ++s) {
+      const int a = a0 + sy[s] * F.P + sx[s];
+      const T pa = s == 0 ? T(1) : T(0.5);
+#pragma unroll
+      for (int o = 0; o < 7; ++o) {
+        T q[4];
+        bool any = false;
+#pragma unroll
+        for (int l = 0; l < 4; ++l) {
+          q[l] = hat_weight_t<T>(sx[s] + sx[o] - 2 * lx[l], sy[s] + sy[o] - 2 * ly[l]);
+          any |= q[l] != T(0);
+        }
+        if (!any) continue;
+        const T *p = o == 0 ? F.C : (o == 1 || o == 2) ? F.E : (o == 3 || o == 4) ? F.Nn : F.NE;
+        const T sab = pa * p[o == 2 ? a - 1 : o == 4 ? a - F.P : o == 6 ? a - F.P - 1 : a];
+#pragma unroll
+        for (int l = 0; l < 4; ++l)
+          if (q[l] != T(0)) c4[l] += sab * q[l];
       }
-      __syncthreads();
     }
+    Cc.C[K] = c4[0];
+    Cc.I[K] = c4[0] > T(0) ? rcp_t(c4[0]) : T(0);
+    Cc.E[K] = X < Cc.W ? c4[1] : T(0);
+    Cc.Nn[K] = Y < Cc.H ? c4[2] : T(0);
+    Cc.NE[K] = X < Cc.W && Y < Cc.H ? c4[3] : T(0);
+  });
 }
 
-// `sweeps` Gauss-Seidel sweeps on v in place, the colours forward (0, 1, 2)
-// in even sweeps and backward in odd ones (as the tiles of k_coarse_pair)
-template <typename T>
-__device__ __forceinline__ void tail_sgs(const TailLevel<T> &L, int sweeps) {
-  for (int s = 0; s < sweeps; ++s)
-    for (int q = 0; q < 3; ++q) {
-      const int color = (s & 1) ? 2 - q : q;
-      for (int k = threadIdx.x; k < L.n; k += blockDim.x) {
-        const int x = k % L.Wn, y = k / L.Wn;
-        if ((x + y) % 3 != color) continue;
-        const T d = L.C[k];
-        if (!(d > T(0))) continue;
-        T l1 = T(0);
-        L.v[k] = (L.r[k] - tail_offdiag(L, L.v, k, x, y, l1)) / d;
-      }
-      __syncthreads();
-    }
-}
-
-// one block per phase (blockIdx.x); dynamic shared memory
-// kTailArrays * sum_l n_l values of T.  GS: the levels' smoothing sweeps are
-// Gauss-Seidel (tail_sgs), else l1-Jacobi.
+// one block per phase (blockIdx.x); dynamic shared memory kTailArrays *
+// sum_l tail_nodes_framed(W_l, H_l) values of T.  GS: the levels' smoothing
+// sweeps are Gauss-Seidel (tail_sgs), else l1-Jacobi.  The float tail forms
+// the operators below level k0 itself; at GB300's FP64 rate one block would
+// take longer than k_galerkin's launches, so the FP64 tail loads them.
 template <typename T, int N, bool GS>
 __global__ void __launch_bounds__(kTailThreads) k_coarse_tail(TailArgs a, const T *__restrict__ r0, T *__restrict__ v0,
                                                               int coarse_sweeps, int coarsest_sweeps) {
-  extern __shared__ unsigned char smem_raw[];
-  T *base = reinterpret_cast<T *>(smem_raw);
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  T *const base = reinterpret_cast<T *>(smem_raw);
   const int i = blockIdx.x;
-  TailLevel<T> lv[kTailMaxLevels];
-  int off = 0;
-  for (int l = 0; l < a.levels; ++l) {
-    TailLevel<T> &L = lv[l];
-    L.W = a.W[l];
-    L.H = a.H[l];
-    L.Wn = L.W + 1;
-    L.n = L.Wn * (L.H + 1);
-    L.C = base + off;
-    L.E = L.C + L.n;
-    L.Nn = L.E + L.n;
-    L.NE = L.Nn + L.n;
-    L.r = L.NE + L.n;
-    L.v = L.r + L.n;
-    L.t = L.v + L.n;
-    off += kTailArrays * L.n;
-    const T *op = static_cast<const T *>(a.op[l]);
-    for (int k = threadIdx.x; k < L.n; k += blockDim.x) {
-      L.C[k] = op[(0 * N + i) * L.n + k];
-      L.E[k] = op[(1 * N + i) * L.n + k];
-      L.Nn[k] = op[(2 * N + i) * L.n + k];
-      L.NE[k] = op[(3 * N + i) * L.n + k];
-    }
+  __shared__ int s_off[kTailMaxLevels + 1];
+  if (threadIdx.x == 0) {
+    s_off[0] = 0;
+    for (int l = 0; l < a.levels; ++l) s_off[l + 1] = s_off[l] + kTailArrays * tail_nodes_framed(a.W[l], a.H[l]);
   }
-  for (int k = threadIdx.x; k < lv[0].n; k += blockDim.x) lv[0].r[k] = r0[(int64_t)i * lv[0].n + k];
   __syncthreads();
+  // the view of level l (pointers into the block's shared memory)
+  auto level = [&](int l) {
+    const int P = a.W[l] + kTailFrame, size = tail_nodes_framed(a.W[l], a.H[l]);
+    T *p = base + s_off[l] + P + 1;
+    return TailLevel<T>{a.W[l],       a.H[l],       P,
+                        p,            p + size,     p + 2 * size, p + 3 * size,
+                        p + 4 * size, p + 5 * size, p + 6 * size, p + 7 * size};
+  };
+  for (int k = threadIdx.x; k < s_off[a.levels]; k += blockDim.x) base[k] = T(0);
+  __syncthreads();
+  constexpr bool kForm = sizeof(T) == 4;  // operators below the first formed here
   const int last = a.levels - 1;
-  for (int l = 0; l < last; ++l) {
-    const TailLevel<T> &L = lv[l];
-    if constexpr (GS) {
-      for (int k = threadIdx.x; k < L.n; k += blockDim.x) L.v[k] = T(0);
+  for (int l = 0; l <= (kForm ? 0 : last); ++l) {
+    const TailLevel<T> L = level(l);
+    const int Wn = L.W + 1;
+    const int64_t n = (int64_t)Wn * (L.H + 1);
+    const T *op = static_cast<const T *>(a.op[l]) + i * n;
+    tail_nodes(L, [&](int k, int x, int y) {
+      const T *q = op + y * Wn + x;
+      const T c = q[0], e = q[N * n], nn = q[2 * N * n], ne = q[3 * N * n];
+      L.C[k] = c;
+      L.I[k] = c > T(0) ? rcp_t(c) : T(0);
+      L.E[k] = e;
+      L.Nn[k] = nn;
+      L.NE[k] = ne;
+      if (l == 0) L.r[k] = r0[i * n + y * Wn + x];
+    });
+  }
+  __syncthreads();
+  if constexpr (kForm)
+    for (int l = 0; l < last; ++l) {
+      const TailLevel<T> F = level(l), Cc = level(l + 1);
+      tail_galerkin(F, Cc);
       __syncthreads();
+    }
+  for (int l = 0; l < last; ++l) {
+    const TailLevel<T> L = level(l), Cc = level(l + 1);
+    if constexpr (GS) {
       tail_sgs(L, coarse_sweeps);
     } else {
       // coarse_sweeps (even) sweeps from zero, alternating t and v, ending in v
@@ -2230,13 +2299,16 @@ __global__ void __launch_bounds__(kTailThreads) k_coarse_tail(TailArgs a, const 
     }
     tail_resid(L);
     __syncthreads();
-    tail_restrict(L, lv[l + 1]);
+    tail_restrict(L, Cc);
     __syncthreads();
   }
-  tail_gs(lv[last], coarsest_sweeps);
+  {
+    const TailLevel<T> L = level(last);
+    tail_sgs(L, coarsest_sweeps);
+  }
   for (int l = last - 1; l >= 0; --l) {
-    const TailLevel<T> &L = lv[l];
-    tail_prolong(L, lv[l + 1]);
+    const TailLevel<T> L = level(l), Cc = level(l + 1);
+    tail_prolong(L, Cc);
     __syncthreads();
     if constexpr (GS) {
       tail_sgs(L, coarse_sweeps);
@@ -2250,7 +2322,9 @@ __global__ void __launch_bounds__(kTailThreads) k_coarse_tail(TailArgs a, const 
       }
     }
   }
-  for (int k = threadIdx.x; k < lv[0].n; k += blockDim.x) v0[(int64_t)i * lv[0].n + k] = lv[0].v[k];
+  const TailLevel<T> L = level(0);
+  const int64_t n = (int64_t)(L.W + 1) * (L.H + 1);
+  tail_nodes(L, [&](int k, int x, int y) { v0[i * n + y * (L.W + 1) + x] = L.v[k]; });
 }
 
 // t = r - S v on a coarse level, one thread per (node, phase) (interior

@@ -210,7 +210,11 @@ struct SolverLaunch {
     static const cudaError_t attr = cudaFuncSetAttribute(
         k_coarse_tail<T, N, GS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTailSmemBytes);
     (void)attr;
-    k_coarse_tail<T, N, GS><<<N, kTailThreads, smem, s>>>(a, (const T *)r0, (T *)v0, coarse_sweeps, coarsest_sweeps);
+    // one thread per node of a colour of the first level (a wider block only
+    // makes the barriers slower)
+    const int64_t third = (int64_t)(a.W[0] / 3 + 1) * (a.H[0] + 1);
+    const int threads = (int)std::min<int64_t>(kTailThreads, std::max<int64_t>(128, (third + 31) / 32 * 32));
+    k_coarse_tail<T, N, GS><<<N, threads, smem, s>>>(a, (const T *)r0, (T *)v0, coarse_sweeps, coarsest_sweeps);
     return 1;
   }
   static int coarse_tail(const TailArgs &a, const void *r0, void *v0, int coarse_sweeps, int coarsest_sweeps,

@@ -15,11 +15,13 @@ struct MaskDirty;
 constexpr int kMaxPartBlocks = 1024;
 
 // The bottom levels k0 .. k0 + levels - 1 of a coarse V-cycle, run by one
-// block per phase in shared memory (kTailArrays values per node: C, E, N,
-// NE, r, v, t); the last level is the coarsest.
+// block per phase in shared memory (kTailArrays values per node: C, 1/C, E,
+// N, NE, r, v, t, each array framed by zeros: one node west and south, two
+// east and north); the last level is the coarsest.
 constexpr int kTailMaxLevels = 8;
-constexpr int kTailArrays = 7;
-constexpr size_t kTailSmemBytes = 200 * 1024;  // shared memory cap of one block
+constexpr int kTailArrays = 8, kTailFrame = 4;  // kTailFrame: framed sides minus cells
+constexpr size_t kTailSmemBytes = 220 * 1024;   // shared memory cap of one block
+__host__ __device__ constexpr int tail_nodes_framed(int W, int H) { return (W + kTailFrame) * (H + kTailFrame); }
 struct TailArgs {
   int levels;
   int W[kTailMaxLevels], H[kTailMaxLevels];
