@@ -284,7 +284,8 @@ struct ac_ctx {
   double *u = nullptr, *b = nullptr, *mom = nullptr;
   float *r32 = nullptr, *u32 = nullptr;        // AC_MIXED: FP32 right-hand side and obstacle
   double *part = nullptr, *tot = nullptr, *c = nullptr, *c_tmp = nullptr, *energy = nullptr;
-  double *rho = nullptr, *omega = nullptr, *ls_part = nullptr, *ls_tot = nullptr;
+  double *rho = nullptr, *omega = nullptr, *ls_part = nullptr;
+  unsigned *ls_done = nullptr;                 // blocks of the line search that have stored their partials
   void *img = nullptr;  // device copy of a host image (allocated on demand)
   size_t img_bytes = 0;
   __nv_bfloat16 *img16 = nullptr;  // AC_MIXED: the image stored in bfloat16
@@ -687,8 +688,9 @@ int enqueue_smooth_resid(ac_ctx *ctx, Solve &S, bool later) {
                                   ? ac::MaskDirty{S.lv[1].lists.dirty, ac::tiles_x(S.lv[1].g), ac::tiles_y(S.lv[1].g)}
                                   : ac::MaskDirty{nullptr, 0, 0};
   AC_RUNB(AC_PROF_SMOOTH, sm_bytes, o->smooth(S.x, S.rhs, S.ob, corr, ctx->omega, g0, nsw, rt_zero,
-                                              fused ? S.mask : nullptr, dirty, ctx->s));
-  AC_CUDA(cudaMemsetAsync(ctx->rho, 0, 2 * sizeof(double), ctx->s));  // rho and the free-node count
+                                              fused ? S.mask : nullptr, dirty, ctx->rho, ctx->s));
+  // rho and the free-node count (a masked smoothing sequence has cleared them)
+  if (!fused) AC_CUDA(cudaMemsetAsync(ctx->rho, 0, 2 * sizeof(double), ctx->s));
   // residual at the visited nodes: x (their own and, for one colour, the
   // other colour's as neighbours), rhs, obstacle read, rt and the mask
   // byte written
@@ -730,7 +732,7 @@ int enqueue_correction(ac_ctx *ctx, Solve &S) {
   // written; curvature: d and the mask read
   const double ls_bytes = bm.n * (bm.ns * (3 + bm.ob) + 1) + l1 + bm.n * (bm.ns + 1);
   AC_RUNB(AC_PROF_LINESEARCH, ls_bytes,
-          o->line_search(S.x, S.ob, S.rt, v1, S.mask, g0, L1.g, S.d, ctx->ls_part, ctx->ls_tot, ctx->omega, ctx->s));
+          o->line_search(S.x, S.ob, S.rt, v1, S.mask, g0, L1.g, S.d, ctx->ls_part, ctx->ls_done, ctx->omega, ctx->s));
   return AC_OK;
 }
 
@@ -1536,7 +1538,7 @@ int ac_create(ac_ctx **out, const ac_params *p) {
     AC_ALLOC(ctx->rho, 2 * sizeof(double));  // rho and the free-node count of the fine residual
     AC_ALLOC(ctx->omega, 2 * sizeof(double));  // omega and its float rounding
     AC_ALLOC(ctx->ls_part, (size_t)2 * ls_blocks * sizeof(double));
-    AC_ALLOC(ctx->ls_tot, 2 * sizeof(double));
+    AC_ALLOC(ctx->ls_done, sizeof(unsigned));
     AC_ALLOC(S.list_counts, 2 * S.lv.size() * sizeof(int));
     for (size_t k = 1; k < S.lv.size(); ++k) {
       Level &L = S.lv[k];
@@ -1559,6 +1561,7 @@ int ac_create(ac_ctx **out, const ac_params *p) {
     AC_CUDA(cudaMallocHost(&ctx->h_scalars, 4 * sizeof(double)));
     AC_CUDA(cudaMemsetAsync(ctx->c, 0, (size_t)3 * N * sizeof(double), ctx->s));
     AC_CUDA(cudaMemsetAsync(ctx->omega, 0, 2 * sizeof(double), ctx->s));
+    AC_CUDA(cudaMemsetAsync(ctx->ls_done, 0, sizeof(unsigned), ctx->s));
     AC_CUDA(cudaMemsetAsync(S.rt, 0, fNs, ctx->s));  // second-colour slots stay 0 (see solve_mg)
     return AC_OK;
   };

@@ -868,8 +868,10 @@ __global__ void __launch_bounds__(kBlock) k_smooth_fine(T *__restrict__ x, const
                                                         const T *__restrict__ ob, const T *__restrict__ corr,
                                                         const double *__restrict__ omega, Geo g, int color,
                                                         T *__restrict__ rt, uint8_t *__restrict__ mask,
-                                                        MaskDirty dirty) {
+                                                        MaskDirty dirty, double *__restrict__ rho) {
   const int y = blockIdx.y;
+  // the residual that follows accumulates into rho and the free-node count
+  if (MASK && rho && blockIdx.x == 0 && y == 0 && threadIdx.x == 0) rho[0] = rho[1] = 0.0;
   const int xx = 2 * (blockIdx.x * blockDim.x + threadIdx.x) + ((y + color) & 1);
   if (xx > g.W) return;
   const int64_t n = fslot<T>(g, xx, y);
@@ -1726,7 +1728,8 @@ __device__ __forceinline__ void jacobi2_tile(const T *__restrict__ op, const T *
 // and blocks agree wherever their regions overlap only up to that boundary
 // information -- a smoother with overlapping blocks (every block's sweep is
 // Gauss-Seidel on its own region).  The second sweep runs the colours in
-// reverse (symmetric Gauss-Seidel).  Rows with a zero diagonal (no free fine
+// reverse (symmetric Gauss-Seidel), so the pass that ends the first sweep
+// counts for both.  Rows with a zero diagonal (no free fine
 // node of the phase under them) keep 0.
 
 // The blocks' work is spread over threads by horizontal triplets: a thread
@@ -1849,8 +1852,8 @@ __device__ __forceinline__ void gs_tile_body(const T *__restrict__ op, const T *
   __syncthreads();
   if (in1 & 4u) AC_GS_UPDATE(2);
   __syncthreads();
-  if (in2 & 4u) AC_GS_UPDATE(2);
-  __syncthreads();
+  // the second sweep starts on colour 2 again, whose neighbours have not
+  // changed since: the pass would repeat the values it finds
   if (in2 & 2u) AC_GS_UPDATE(1);
   __syncthreads();
   if (in2 & 1u) AC_GS_UPDATE(0);
@@ -2463,97 +2466,156 @@ __global__ void __launch_bounds__(kTileThreads) k_prolong_add_tiled(const T *__r
 //   d   = P(x + w) - x  (feasible direction: the constraint set is convex),
 //   omega = clamp(rt'd / d'Sd, 0, 1) minimises the step energy on [x, x + d].
 // k_ls_dir writes d and the block partials of rt'd; k_ls_curv the partials of
-// d'Sd; k_ls_finish computes omega; the next smoothing pass applies
-// x += omega d (see k_smooth_fine).
+// d'Sd, and omega; the next smoothing pass applies x += omega d (see
+// k_smooth_fine).
 // ---------------------------------------------------------------------------
-template <typename T, int N, int FORM>
-__global__ void __launch_bounds__(kBlock) k_ls_dir(const T *__restrict__ x, const T *__restrict__ ob,
-                                                   const T *__restrict__ rt, const T *__restrict__ v1,
-                                                   const uint8_t *__restrict__ mask, Geo gf, Geo gc,
-                                                   T *__restrict__ d, double *__restrict__ part) {
-  const int xx = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
-  T dot = T(0);
-  if (xx <= gf.W) {
-    const int64_t n = (int64_t)y * gf.Wn + xx, sl = fslot<T>(gf, xx, y);
-    const unsigned fr = mask[n];
-    T dn[N];
-    if (fr) {
-      T w[N], xk[N], r[N], o[N];
-      prolong_at<T, N>(v1, gc, xx, y, w);
-      T s = T(0);
-      int cnt = 0;
-#pragma unroll
-      for (int i = 0; i < N; ++i)
-        if ((fr >> i) & 1u) {
-          s += w[i];
-          ++cnt;
-        }
-      const T mean = s * rcp_small<T>(cnt);
-      ldn<T, N>(x + sl * N, xk);
-      if constexpr (FORM != kDirect) ldn<T, N>(ob + sl * N, o);
-#pragma unroll
-      for (int i = 0; i < N; ++i) w[i] = xk[i] + (((fr >> i) & 1u) ? w[i] - mean : T(0));
-      proj_box<T, N, FORM>(w, o);
-      ldn<T, N>(rt + sl * N, r);
-      T loc = T(0);
-#pragma unroll
-      for (int i = 0; i < N; ++i) {
-        dn[i] = w[i] - xk[i];
-        loc += r[i] * dn[i];
-      }
-      dot = loc;
-    } else {
-#pragma unroll
-      for (int i = 0; i < N; ++i) dn[i] = T(0);
-    }
-    stn<T, N>(d + sl * N, dn);
+// Both kernels give a block `chunks` runs of kBlock consecutive nodes (in row
+// order, so that no block hangs over the end of a row), few enough blocks
+// that one of them can add up all block partials (SolverLaunch::line_search);
+// a thread sums its nodes with a compensation, so a partial carries the
+// rounding of one block sum whatever the chunks.  The last block of k_ls_curv
+// to finish adds the partials of both up in a fixed order and sets omega: two
+// column sums and a one-thread kernel took 51 us at 4096^2 (69,649 partials
+// each, one SM reading them) and three of about twenty launches of a small
+// picture's cycle.
+template <typename T>
+struct NodeSum {
+  T s = T(0), c = T(0);
+  __device__ __forceinline__ void add(T v) {
+    const T t = s + v, z = t - s;
+    c += (s - (t - z)) + (v - z);
+    s = t;
   }
-  block_sum_store1<T>(dot, part + blockIdx.y * gridDim.x + blockIdx.x);
+  __device__ __forceinline__ T value() const { return s + c; }
+};
+
+template <typename T, int N, int FORM>
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 6 : 4) k_ls_dir(const T *__restrict__ x, const T *__restrict__ ob,
+                                                   const T *__restrict__ rt, const T *__restrict__ v1,
+                                                   const uint8_t *__restrict__ mask, Geo gf, Geo gc, int chunks,
+                                                   T *__restrict__ d, double *__restrict__ part) {
+  NodeSum<T> dot;
+  const int64_t nodes = (int64_t)gf.Wn * (gf.H + 1);
+  for (int q = 0; q < chunks; ++q) {
+    const int64_t n = ((int64_t)blockIdx.x * chunks + q) * kBlock + threadIdx.x;
+    if (n < nodes) {
+      const int y = (int)((unsigned)n / (unsigned)gf.Wn), xx = (int)((unsigned)n % (unsigned)gf.Wn);
+      const int64_t sl = fslot<T>(gf, xx, y);
+      const unsigned fr = mask[n];
+      T dn[N];
+      if (fr) {
+        T w[N], xk[N], r[N], o[N];
+        prolong_at<T, N>(v1, gc, xx, y, w);
+        T s = T(0);
+        int cnt = 0;
+#pragma unroll
+        for (int i = 0; i < N; ++i)
+          if ((fr >> i) & 1u) {
+            s += w[i];
+            ++cnt;
+          }
+        const T mean = s * rcp_small<T>(cnt);
+        ldn<T, N>(x + sl * N, xk);
+        if constexpr (FORM != kDirect) ldn<T, N>(ob + sl * N, o);
+#pragma unroll
+        for (int i = 0; i < N; ++i) w[i] = xk[i] + (((fr >> i) & 1u) ? w[i] - mean : T(0));
+        proj_box<T, N, FORM>(w, o);
+        ldn<T, N>(rt + sl * N, r);
+        T loc = T(0);
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+          dn[i] = w[i] - xk[i];
+          loc += r[i] * dn[i];
+        }
+        dot.add(loc);
+      } else {
+#pragma unroll
+        for (int i = 0; i < N; ++i) dn[i] = T(0);
+      }
+      stn<T, N>(d + sl * N, dn);
+    }
+  }
+  block_sum_store1<T>(dot.value(), part + blockIdx.x);
 }
 
 // d'Sd = sum_n S_nn |d_n|^2 - 2 tau eps sum over axis edges (n, m) of
 // w_nm d_n . d_m, each edge counted once at its west / south end: three
 // node reads per thread (own, east, north) instead of the five of S d.  A
 // node with no free phase has d_n = 0 (k_ls_dir), so its terms vanish and
-// only its mask byte is read.
+// only its mask byte is read.  part: k_ls_dir's block partials, then this
+// kernel's; *done counts the blocks that have stored theirs (0 between
+// launches).
 template <typename T, int N>
-__global__ void __launch_bounds__(kBlock) k_ls_curv(const T *__restrict__ d, const uint8_t *__restrict__ mask, Geo g,
-                                                    double *__restrict__ part) {
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
-  T dot = T(0);
-  if (x <= g.W && mask[(int64_t)y * g.Wn + x]) {
-    T dk[N], t[N];
-    ldn<T, N>(d + fslot<T>(g, x, y) * N, dk);
-    const Weights w = edge_weights(g, x, y);
-    T sq = T(0), cross = T(0);
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 6 : 5) k_ls_curv(const T *__restrict__ d, const uint8_t *__restrict__ mask, Geo g,
+                                                    int chunks, double *part, unsigned *done,
+                                                    double *__restrict__ omega) {
+  const int blocks = (int)gridDim.x;
+  NodeSum<T> dot;
+  const int64_t nodes = (int64_t)g.Wn * (g.H + 1);
+  for (int q = 0; q < chunks; ++q) {
+    const int64_t n = ((int64_t)blockIdx.x * chunks + q) * kBlock + threadIdx.x;
+    if (n < nodes && mask[n]) {
+      const int y = (int)((unsigned)n / (unsigned)g.Wn), x = (int)((unsigned)n % (unsigned)g.Wn);
+      T dk[N], t[N];
+      ldn<T, N>(d + fslot<T>(g, x, y) * N, dk);
+      const Weights w = edge_weights(g, x, y);
+      T sq = T(0), cross = T(0);
 #pragma unroll
-    for (int i = 0; i < N; ++i) sq += dk[i] * dk[i];
-    if (x < g.W) {
-      ldn<T, N>(d + fslot<T>(g, x + 1, y) * N, t);
-      T e = T(0);
+      for (int i = 0; i < N; ++i) sq += dk[i] * dk[i];
+      if (x < g.W) {
+        ldn<T, N>(d + fslot<T>(g, x + 1, y) * N, t);
+        T e = T(0);
 #pragma unroll
-      for (int i = 0; i < N; ++i) e += dk[i] * t[i];
-      cross += T(w.e) * e;
+        for (int i = 0; i < N; ++i) e += dk[i] * t[i];
+        cross += T(w.e) * e;
+      }
+      if (y < g.H) {
+        ldn<T, N>(d + fslot<T>(g, x, y + 1) * N, t);
+        T e = T(0);
+#pragma unroll
+        for (int i = 0; i < N; ++i) e += dk[i] * t[i];
+        cross += T(w.n) * e;
+      }
+      dot.add(geo_D<T>(g, node_class(g, x, y)) * sq - T(2) * geo_te<T>(g) * cross);
     }
-    if (y < g.H) {
-      ldn<T, N>(d + fslot<T>(g, x, y + 1) * N, t);
-      T e = T(0);
-#pragma unroll
-      for (int i = 0; i < N; ++i) e += dk[i] * t[i];
-      cross += T(w.n) * e;
-    }
-    dot = geo_D<T>(g, node_class(g, x, y)) * sq - T(2) * geo_te<T>(g) * cross;
   }
-  block_sum_store1<T>(dot, part + blockIdx.y * gridDim.x + blockIdx.x);
-}
-
-static __global__ void k_ls_finish(const double *__restrict__ tot, double *__restrict__ omega) {
-  if (threadIdx.x != 0 || blockIdx.x != 0) return;
-  const double rd = tot[0], dsd = tot[1];
-  double w = 0.0;
-  if (dsd > 0.0 && rd > 0.0) w = fmin(1.0, rd / dsd);
-  omega[0] = w;
-  reinterpret_cast<float *>(omega + 1)[0] = (float)w;
+  block_sum_store1<T>(dot.value(), part + blocks + blockIdx.x);
+  __shared__ bool last;
+  if (threadIdx.x == 0) {
+    __threadfence();  // this block's partial before its count
+    last = atomicAdd(done, 1u) == (unsigned)blocks - 1u;
+  }
+  __syncthreads();
+  if (!last) return;
+  __threadfence();
+  double v[2] = {0.0, 0.0}, a[3][2] = {};
+  int k = threadIdx.x;
+  for (; k + 3 * kBlock < blocks; k += 4 * kBlock) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const volatile double *p = part + (int64_t)q * blocks + k;
+      v[q] += p[0];
+      a[0][q] += p[kBlock];
+      a[1][q] += p[2 * kBlock];
+      a[2][q] += p[3 * kBlock];
+    }
+  }
+  for (; k < blocks; k += kBlock) {
+    v[0] += ((const volatile double *)part)[k];
+    v[1] += ((const volatile double *)part)[blocks + k];
+  }
+#pragma unroll
+  for (int q = 0; q < 2; ++q) v[q] = (v[q] + a[0][q]) + (a[1][q] + a[2][q]);
+  __shared__ double tot[2];
+  block_sum_store<2>(v, tot);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double w = 0.0;
+    if (tot[1] > 0.0 && tot[0] > 0.0) w = fmin(1.0, tot[0] / tot[1]);
+    omega[0] = w;
+    reinterpret_cast<float *>(omega + 1)[0] = (float)w;
+    *done = 0u;
+  }
 }
 
 // ---------------------------------------------------------------------------

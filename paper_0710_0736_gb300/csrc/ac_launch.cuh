@@ -59,19 +59,21 @@ struct SolverLaunch {
   // `sweeps` red-black sweeps in place, one launch per colour; the pending
   // coarse correction (corr != null) is applied inside the first launch.
   // With mask != null the last launch (colour 1) also stores its nodes' free
-  // mask (and rt = 0 if rt != null), so that resid(color = 0) completes them.
+  // mask (and rt = 0 if rt != null), so that resid(color = 0) completes them,
+  // and clears rho[0..1] for it.
   static int smooth(void *x, const void *rhs, const void *ob, const void *corr, const double *omega, const Geo &g,
-                    int sweeps, void *rt, uint8_t *mask, const MaskDirty &dirty, cudaStream_t s) {
+                    int sweeps, void *rt, uint8_t *mask, const MaskDirty &dirty, double *rho, cudaStream_t s) {
     const dim3 grid = row_grid((g.W + 2) / 2, g.H + 1);
     for (int k = 0; k < sweeps; ++k)
       for (int c = 0; c < 2; ++c) {
         const T *cr = k == 0 && c == 0 ? (const T *)corr : nullptr;
         if (mask && k == sweeps - 1 && c == 1)
           k_smooth_fine<T, N, FORM, true><<<grid, kBlock, 0, s>>>((T *)x, (const T *)rhs, (const T *)ob, cr, omega,
-                                                                g, c, (T *)rt, mask, dirty);
+                                                                g, c, (T *)rt, mask, dirty, rho);
         else
           k_smooth_fine<T, N, FORM, false><<<grid, kBlock, 0, s>>>((T *)x, (const T *)rhs, (const T *)ob, cr, omega,
-                                                                 g, c, nullptr, nullptr, MaskDirty{nullptr, 0, 0});
+                                                                 g, c, nullptr, nullptr, MaskDirty{nullptr, 0, 0},
+                                                                 nullptr);
       }
     return 2 * sweeps;
   }
@@ -223,17 +225,21 @@ struct SolverLaunch {
               : coarse_tail_t<false>(a, r0, v0, coarse_sweeps, coarsest_sweeps, smem, s);
   }
   static int line_search(const void *x, const void *ob, const void *rt, const void *v1, const uint8_t *mask,
-                         const Geo &gf, const Geo &gc, void *d, double *part, double *tot, double *omega,
+                         const Geo &gf, const Geo &gc, void *d, double *part, unsigned *done, double *omega,
                          cudaStream_t s) {
-    const dim3 grid = row_grid(gf.W + 1, gf.H + 1);
-    const int blocks = (int)(grid.x * grid.y);
+    // one resident set of blocks while a block then takes at most eight
+    // chunks, so that the closing sum of the last block stays near 1 us
+    // (1024^2: 821 blocks); four sets on larger grids, whose blocks differ in
+    // their share of free nodes
+    constexpr int64_t kSet = 152 * 6;
+    const int64_t all = ((int64_t)(gf.W + 1) * (gf.H + 1) + kBlock - 1) / kBlock;
+    const int64_t want = all <= 8 * kSet ? kSet : 4 * kSet;
+    const int chunks = (int)((all + want - 1) / want);
+    const unsigned grid = (unsigned)((all + chunks - 1) / chunks);
     k_ls_dir<T, N, FORM><<<grid, kBlock, 0, s>>>((const T *)x, (const T *)ob, (const T *)rt, (const T *)v1, mask, gf,
-                                               gc, (T *)d, part);
-    k_ls_curv<T, N><<<grid, kBlock, 0, s>>>((const T *)d, mask, gf, part + blocks);
-    k_colsum<<<1, 1024, 0, s>>>(part, blocks, 1, tot);
-    k_colsum<<<1, 1024, 0, s>>>(part + blocks, blocks, 1, tot + 1);
-    k_ls_finish<<<1, 32, 0, s>>>(tot, omega);
-    return 5;
+                                               gc, chunks, (T *)d, part);
+    k_ls_curv<T, N><<<grid, kBlock, 0, s>>>((const T *)d, mask, gf, chunks, part, done, omega);
+    return 2;
   }
   static SolverOps table() {
     return SolverOps{(int)sizeof(T), smooth,       resid,        restrict0,   galerkin0,   galerkin,   coarse_smooth,

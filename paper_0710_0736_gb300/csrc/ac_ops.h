@@ -54,10 +54,10 @@ struct SolverOps {
   // sweeps red-black sweeps in place; with corr != null the pending coarse
   // correction x += (*omega) corr is applied inside the first launch; with
   // mask != null the last launch stores its colour's free mask (and rt = 0
-  // for that colour if rt != null)
+  // for that colour if rt != null) and clears rho[0..1]
   // (dirty: the first coarse level's tiles to mark where the mask changes)
   int (*smooth)(void *x, const void *rhs, const void *ob, const void *corr, const double *omega, const Geo &g,
-                int sweeps, void *rt, uint8_t *mask, const MaskDirty &dirty, cudaStream_t s);
+                int sweeps, void *rt, uint8_t *mask, const MaskDirty &dirty, double *rho, cudaStream_t s);
   // color < 0: every node; 0: the first colour only (completes a masked smooth)
   int (*resid)(const void *x, const void *rhs, const void *ob, const Geo &g, void *rt, uint8_t *mask, double *rho,
                int color, const MaskDirty &dirty, cudaStream_t s);
@@ -94,9 +94,11 @@ struct SolverOps {
   // TailArgs); smem bytes of dynamic shared memory per block
   int (*coarse_tail)(const TailArgs &a, const void *r0, void *v0, int coarse_sweeps, int coarsest_sweeps,
                      size_t smem, bool gs, cudaStream_t s);
-  // line search: part needs 2 x (blocks of the fine grid) doubles, tot 2 doubles
+  // line search: part needs 2 x (blocks of the fine grid) doubles, done is
+  // a counter that is 0 between calls
   int (*line_search)(const void *x, const void *ob, const void *rt, const void *v1, const uint8_t *mask,
-                     const Geo &gf, const Geo &gc, void *d, double *part, double *tot, double *omega, cudaStream_t s);
+                     const Geo &gf, const Geo &gc, void *d, double *part, unsigned *done, double *omega,
+                     cudaStream_t s);
 };
 
 struct Ops {
