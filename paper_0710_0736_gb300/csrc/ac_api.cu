@@ -1529,6 +1529,7 @@ int ac_create(ac_ctx **out, const ac_params *p) {
     }
     AC_ALLOC(S.rt, fNs);
     AC_ALLOC(S.mask, (size_t)ctx->n);
+    AC_CUDA(cudaMemsetAsync(S.mask, 0, (size_t)ctx->n, ctx->s));  // read as a hint before the first cycle sets it
     if (S.lv.size() > 1) AC_ALLOC(S.d, fNs);
     AC_ALLOC(ctx->part, (size_t)ac::kMaxPartBlocks * 7 * N * sizeof(double));
     AC_ALLOC(ctx->tot, (size_t)7 * N * sizeof(double));

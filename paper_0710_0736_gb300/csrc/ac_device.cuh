@@ -422,6 +422,179 @@ __device__ __forceinline__ void nbr_sum(const T *u, const Geo &g, int x, int y, 
   }
 }
 
+// ---- the FP64 direct form's nodal problem ------------------------------------
+// GB300 runs binary64 arithmetic at 1/64 of its float rate, and the FP64
+// form's smoother and residual were bound by it: five operations per phase for
+// z = (b + tau eps sum_m w_nm u_m) / S_nn, then two per kept phase and
+// projection pass.  But a node keeps one to three phases once they form, and
+// the others' values are only ever compared with the threshold.  So a float
+// pass on the values' heads finds the set the projection keeps, binary64 runs
+// on those phases alone, and the set is checked afterwards: a kept z above the
+// binary64 theta, a dropped one's float value below it by more than its error
+// bound.  Where the check holds, the binary64 iteration of proj_box ends on
+// the same set and sums it in the same order (see outer_update_node): the
+// result is bit-identical to it.  Near ties, and for values a float cannot
+// hold, the plain path runs.
+// At 1024^2, N = 4, formed phases: smoother pass 77 -> 34 us, residual 130 ->
+// 89 us; on a random start, where the nodes keep most phases and many_free64
+// takes the plain path, the step is 1% slower.
+
+template <typename T, int FORM>
+constexpr bool kFilter64 = std::is_same<T, double>::value && FORM == kDirect;
+
+// Whether the warp's nodes, by their free masks of the last cycle, keep more
+// than three quarters of the phases between them: the plain path is then
+// faster (both give the same bits, so a stale mask costs time only).
+template <int N>
+__device__ __forceinline__ bool many_free64(uint8_t mask) {
+  return 4 * __popc(__reduce_or_sync(__activemask(), (unsigned)mask)) > 3 * N;
+}
+
+// The heads' sums over all phases, acc += f sum_m w_nm u_m and mag += the sum
+// of magnitudes.
+template <int N>
+__device__ __forceinline__ void nbr_heads(const double *u, const Geo &g, int x, int y, const Weights &w, float f,
+                                          float (&acc)[N], float (&mag)[N]) {
+  const double *p = u + ((int64_t)y * g.Wn + x) * N;
+  auto add = [&](const double *q, float we) {
+    if (we > 0.f) {
+      double t[N];
+      ldn_rw<double, N>(q, t);
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        const float h = (f * we) * f64_head(t[i]);
+        acc[i] += h;
+        mag[i] += fabsf(h);
+      }
+    }
+  };
+  add(p + N, w.e);
+  add(p - N, w.w);
+  add(p + (int64_t)g.Wn * N, w.n);
+  add(p - (int64_t)g.Wn * N, w.s);
+}
+
+// sum_m w_nm u_m for phase i alone in binary64 (nbr_sum's order), read again
+// from L1: keeping the neighbours' values in registers instead (N = 4: 94
+// against 62) was slower, 2.47 against 2.30 ms of smoothing at 1024^2.
+template <int N>
+__device__ __forceinline__ double nbr_sum1(const double *u, const Geo &g, int x, int y, const Weights &w, bool inside,
+                                           int i) {
+  const double *p = u + ((int64_t)y * g.Wn + x) * N + i;
+  const int64_t row = (int64_t)g.Wn * N;
+  if (inside) return ((p[N] + p[-N]) + p[row]) + p[-row];
+  double acc = 0.0;
+  if (w.e > 0.f) acc += (double)w.e * p[N];
+  if (w.w > 0.f) acc += (double)w.w * p[-N];
+  if (w.n > 0.f) acc += (double)w.n * p[row];
+  if (w.s > 0.f) acc += (double)w.s * p[-row];
+  return acc;
+}
+
+// q_i = b_i + te (sum_m w_nm u_m + omega sum_m w_nm d_m)_i and z_i = q_i / S_nn
+// at node (x, y), and the set and threshold of z's projection: out_i = z_i -
+// theta on keep, 0 elsewhere.  q and z are set for the phases of keep and
+// `also` (all phases where the plain path runs).  d null: no correction.
+template <int N>
+__device__ __forceinline__ void direct_node64(const double *u, const double *d, double omega, const double (&b)[N],
+                                              const Geo &g, int x, int y, unsigned also, double (&q)[N],
+                                              double (&z)[N], unsigned &keep, double &theta) {
+  const int cls = node_class(g, x, y);
+  const Weights w = edge_weights(g, x, y);
+  const bool inside = cls == 4;
+  float zf[N], er[N];
+  {
+    float acc[N], mag[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) acc[i] = mag[i] = 0.f;
+    nbr_heads<N>(u, g, x, y, w, 1.f, acc, mag);
+    if (d) nbr_heads<N>(d, g, x, y, w, f64_head(omega), acc, mag);
+    // heads within 2^-23 of their values, at most eight terms, the constants
+    // and three more operations rounded: |zf - z| < 2^-19 (|b| + te mag) / S_nn
+    // (2^-100: values flushed to 0)
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const float bf = f64_head(b[i]);
+      zf[i] = (bf + g.tef * acc[i]) * g.invDf[cls];
+      er[i] = (fabsf(bf) + g.tef * mag[i]) * g.invDf[cls] * 0x1.0p-19f + 0x1.0p-100f;
+    }
+  }
+  // Michelot's iteration on the float values
+  keep = (1u << N) - 1u;
+  {
+    float s = 0.f;
+#pragma unroll
+    for (int i = 0; i < N; ++i) s += zf[i];
+    float t = (s - 1.f) * rcp_small<float>(N);
+#pragma unroll 1
+    for (int pass = 1; pass < N; ++pass) {
+      unsigned drop = 0;
+#pragma unroll
+      for (int i = 0; i < N; ++i)
+        if (((keep >> i) & 1u) && zf[i] <= t) drop |= 1u << i;
+      if (!drop || drop == keep) break;
+      keep &= ~drop;
+      s = 0.f;
+#pragma unroll
+      for (int i = 0; i < N; ++i)
+        if ((keep >> i) & 1u) s += zf[i];
+      t = (s - 1.f) * rcp_small<float>(__popc(keep));
+    }
+  }
+  const double te = g.te, invD = g.invD[cls];
+  const unsigned lanes = __activemask();
+  auto value = [&](int i) {
+    double acc = nbr_sum1<N>(u, g, x, y, w, inside, i);
+    if (d && omega != 0.0) acc += omega * nbr_sum1<N>(d, g, x, y, w, inside, i);
+    q[i] = b[i] + te * acc;
+    z[i] = q[i] * invD;
+  };
+  const unsigned need = keep | also, any = __reduce_or_sync(lanes, need);
+  double s = 0.0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    if (!((any >> i) & 1u)) continue;  // no lane of the warp needs phase i
+    if ((need >> i) & 1u) value(i);
+    if ((keep >> i) & 1u) s += z[i];
+  }
+  theta = (s - 1.0) * rcp_small<double>(__popc(keep));
+  const float t32 = f64_head(theta);
+  bool ok = true;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    if ((keep >> i) & 1u) {
+      const float h = f64_head(z[i]);
+      ok = ok && h - t32 > (fabsf(h) + fabsf(t32)) * 0x1.0p-21f + 0x1.0p-120f;
+    } else {
+      ok = ok && t32 - zf[i] > er[i] + fabsf(t32) * 0x1.0p-21f;
+    }
+  }
+  if (ok) return;
+  // the plain path: every phase, the iteration in binary64 (proj_box)
+  s = 0.0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    value(i);
+    s += z[i];
+  }
+  keep = (1u << N) - 1u;
+  theta = (s - 1.0) * rcp_small<double>(N);
+#pragma unroll 1
+  for (int pass = 1; pass < N; ++pass) {
+    unsigned drop = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      if (((keep >> i) & 1u) && z[i] - theta <= 0.0) drop |= 1u << i;
+    if (!drop || drop == keep) break;
+    keep &= ~drop;
+    s = 0.0;
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      if ((keep >> i) & 1u) s += z[i];
+    theta = (s - 1.0) * rcp_small<double>(__popc(keep));
+  }
+}
+
 // P1 interpolation weight of coarse node L at fine node b (fine coordinates),
 // for nested right-diagonal meshes: 1 at 2L, 1/2 at the six neighbours of 2L
 // along the coarse edges (E, W, N, S, NE, SW), 0 elsewhere.

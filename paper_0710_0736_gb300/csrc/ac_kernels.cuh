@@ -878,23 +878,35 @@ __global__ void __launch_bounds__(kBlock) k_smooth_fine(T *__restrict__ x, const
   // the mask byte this pass replaces, loaded first so its latency overlaps
   const uint8_t old_mask = (MASK && dirty.p) ? mask[(int64_t)y * g.Wn + xx] : (uint8_t)0;
   T acc[N], bk[N], o[N];
-  nbr_sum<T, N>(x, g, xx, y, acc);
-  if (corr) {
-    const T w = omega_t<T>(omega);
-    if (w != T(0)) {
-      T dc[N];
-      nbr_sum<T, N>(corr, g, xx, y, dc);
+  // FP64 direct form: phases the projection drops need no binary64 at all
+  bool plain = true;
+  if constexpr (kFilter64<T, FORM>) plain = many_free64<N>(mask[(int64_t)y * g.Wn + xx]);
+  if (plain) {
+    nbr_sum<T, N>(x, g, xx, y, acc);
+    if (corr) {
+      const T w = omega_t<T>(omega);
+      if (w != T(0)) {
+        T dc[N];
+        nbr_sum<T, N>(corr, g, xx, y, dc);
 #pragma unroll
-      for (int i = 0; i < N; ++i) acc[i] += w * dc[i];
+        for (int i = 0; i < N; ++i) acc[i] += w * dc[i];
+      }
     }
-  }
-  ldn<T, N>(rhs + n * N, bk);
-  if constexpr (FORM != kDirect) ldn<T, N>(ob + n * N, o);
-  const int cls = node_class(g, xx, y);
-  const T te = geo_te<T>(g), invD = geo_invD<T>(g, cls);
+    ldn<T, N>(rhs + n * N, bk);
+    if constexpr (FORM != kDirect) ldn<T, N>(ob + n * N, o);
+    const int cls = node_class(g, xx, y);
+    const T te = geo_te<T>(g), invD = geo_invD<T>(g, cls);
 #pragma unroll
-  for (int i = 0; i < N; ++i) acc[i] = (bk[i] + te * acc[i]) * invD;
-  proj_box<T, N, FORM>(acc, o);
+    for (int i = 0; i < N; ++i) acc[i] = (bk[i] + te * acc[i]) * invD;
+    proj_box<T, N, FORM>(acc, o);
+  } else if constexpr (kFilter64<T, FORM>) {
+    ldn<T, N>(rhs + n * N, bk);
+    double q[N], z[N], theta;
+    unsigned keep;
+    direct_node64<N>(x, corr, corr ? omega[0] : 0.0, bk, g, xx, y, 0u, q, z, keep, theta);
+#pragma unroll
+    for (int i = 0; i < N; ++i) acc[i] = ((keep >> i) & 1u) ? z[i] - theta : 0.0;
+  }
   stn<T, N>(x + n * N, acc);
   if constexpr (MASK) {
     // last pass of a smoothing sequence: this node's nodal problem is solved
@@ -950,18 +962,37 @@ __global__ void __launch_bounds__(kBlock) k_fine_resid(const T *__restrict__ x, 
     // the mask byte this kernel replaces, loaded first so its latency overlaps
     const uint8_t old_mask = (rt && dirty.p) ? mask[n] : (uint8_t)0;
     T acc[N], xk[N], bk[N], r[N], o[N];
-    nbr_sum<T, N>(x, g, xx, y, acc);
     ldn<T, N>(x + sl * N, xk);
     ldn<T, N>(rhs + sl * N, bk);
-    if constexpr (FORM != kDirect) ldn<T, N>(ob + sl * N, o);
     const int cls = node_class(g, xx, y);
-    const T D = geo_D<T>(g, cls), invD = geo_invD<T>(g, cls), te = geo_te<T>(g);
+    const T D = geo_D<T>(g, cls);
+    bool plain = true;
+    if constexpr (kFilter64<T, FORM>) plain = !mask || many_free64<N>(mask[n]);
+    if (plain) {
+      nbr_sum<T, N>(x, g, xx, y, acc);
+      if constexpr (FORM != kDirect) ldn<T, N>(ob + sl * N, o);
+      const T invD = geo_invD<T>(g, cls), te = geo_te<T>(g);
 #pragma unroll
-    for (int i = 0; i < N; ++i) {
-      r[i] = bk[i] + te * acc[i] - D * xk[i];
-      acc[i] = (bk[i] + te * acc[i]) * invD;
+      for (int i = 0; i < N; ++i) {
+        r[i] = bk[i] + te * acc[i] - D * xk[i];
+        acc[i] = (bk[i] + te * acc[i]) * invD;
+      }
+      proj_box<T, N, FORM>(acc, o);
+    } else if constexpr (kFilter64<T, FORM>) {
+      // the residual is wanted on the phases above 0, the projection on those
+      // it keeps; elsewhere x and P(z) are both 0
+      unsigned above = 0u, keep;
+#pragma unroll
+      for (int i = 0; i < N; ++i) above |= xk[i] > 0.0 ? 1u << i : 0u;
+      double q[N], z[N], theta;
+      direct_node64<N>(x, nullptr, 0.0, bk, g, xx, y, above, q, z, keep, theta);
+      const unsigned any = __reduce_or_sync(__activemask(), above | keep);
+#pragma unroll
+      for (int i = 0; i < N; ++i) {
+        r[i] = ((any >> i) & 1u) && ((above >> i) & 1u) ? q[i] - D * xk[i] : 0.0;
+        acc[i] = ((any >> i) & 1u) && ((keep >> i) & 1u) ? z[i] - theta : 0.0;
+      }
     }
-    proj_box<T, N, FORM>(acc, o);
     int cnt = 0;
     unsigned pos = 0;
     T et = T(0);

@@ -72,7 +72,7 @@ struct SolverLaunch {
                                                                 g, c, (T *)rt, mask, dirty, rho);
         else
           k_smooth_fine<T, N, FORM, false><<<grid, kBlock, 0, s>>>((T *)x, (const T *)rhs, (const T *)ob, cr, omega,
-                                                                 g, c, nullptr, nullptr, MaskDirty{nullptr, 0, 0},
+                                                                 g, c, nullptr, mask, MaskDirty{nullptr, 0, 0},
                                                                  nullptr);
       }
     return 2 * sweeps;
