@@ -884,6 +884,7 @@ int solve_mixed(ac_ctx *ctx, int *cycles_out, double *rho_out, int64_t *sweeps_o
 // stays on the host).
 
 __global__ void k_ctl_reset(LoopCtl *c, int warm) {
+  ac::pdl_sync();
   c->total_cycles = 0;
   c->total_sweeps = 0;
   c->total_outer = 0;
@@ -896,6 +897,7 @@ __global__ void k_ctl_reset(LoopCtl *c, int warm) {
 }
 
 __global__ void k_ctl_step_begin(LoopCtl *c, double tol, int cap) {
+  ac::pdl_sync();
   c->cycles = 0;
   c->outer = 0;
   c->sweeps = 0;
@@ -910,6 +912,7 @@ __global__ void k_ctl_step_begin(LoopCtl *c, double tol, int cap) {
 // After a cycle's residual (solve_mg): stop on a non-finite rho, on rho <=
 // tol, or at the cycle limit; otherwise run another cycle.
 __global__ void k_ctl_cycle(LoopCtl *c, const double *rho, int nsw, cudaGraphConditionalHandle h) {
+  ac::pdl_sync();
   c->cyc += 1;
   c->cycles += 1;
   c->sweeps += nsw;
@@ -933,6 +936,7 @@ __global__ void k_ctl_cycle(LoopCtl *c, const double *rho, int nsw, cudaGraphCon
 // correction starts from the previous step's).
 __global__ void k_ctl_outer(LoopCtl *c, const double *rho, double accept, double tol, double tol_frac,
                             double reduction, int max_cycles, int inner_max, int nu1, cudaGraphConditionalHandle h) {
+  ac::pdl_sync();
   const double r = rho[0];
   c->rho = r;
   unsigned go = 0;
@@ -958,17 +962,20 @@ __global__ void k_ctl_outer(LoopCtl *c, const double *rho, double accept, double
 
 // The correction's start: zero unless k_ctl_outer chose the warm start.
 __global__ void k_zero_unless_warm(const LoopCtl *c, float *x, int64_t count) {
+  ac::pdl_sync();
   if (!c->zero_x) return;
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < count; k += (int64_t)gridDim.x * blockDim.x)
     x[k] = 0.0f;
 }
 
 __global__ void k_ctl_after_update(LoopCtl *c) {
+  ac::pdl_sync();
   c->outer += 1;
   c->warm = c->inner_status == 0 && c->outer == 1;
 }
 
 __global__ void k_ctl_step_end(LoopCtl *c, int fp64) {
+  ac::pdl_sync();
   if (fp64) {
     c->rho = c->rho_inner;
     c->status = c->inner_status;
@@ -1086,7 +1093,7 @@ int enqueue_step_loop(ac_ctx *ctx, cudaGraph_t top, bool energy, StepGraph &sg) 
     }
   } guard{ctx, top_s, saved};
   ctx->capturing = &cnt_fixed;
-  AC_RUN(AC_PROF_SETUP, (k_ctl_step_begin<<<1, 1, 0, ctx->s>>>(ctx->ctl, ctx->p.tol, ctx->p.max_cycles), 1));
+  AC_RUN(AC_PROF_SETUP, (ac::launch(k_ctl_step_begin, 1, 1, 0, ctx->s, ctx->ctl, ctx->p.tol, ctx->p.max_cycles), 1));
   double *en = energy ? ctx->energy : nullptr;
   if (mixed) {
     AC_RUNB(AC_PROF_SETUP, mean_bytes,
@@ -1101,7 +1108,7 @@ int enqueue_step_loop(ac_ctx *ctx, cudaGraph_t top, bool energy, StepGraph &sg) 
   auto solve = [&](int d) -> int {
     int rc = enqueue_smooth_resid(ctx, S, false);
     if (rc) return rc;
-    AC_RUN(AC_PROF_RESID, (k_ctl_cycle<<<1, 1, 0, ctx->s>>>(ctx->ctl, ctx->rho, ctx->p.nu1, h_cyc), 1));
+    AC_RUN(AC_PROF_RESID, (ac::launch(k_ctl_cycle, 1, 1, 0, ctx->s, ctx->ctl, ctx->rho, ctx->p.nu1, h_cyc), 1));
     rc = begin_while(ctx->s, h_cyc, ctx->body_s[d]);
     if (rc) return rc;
     cudaStream_t const outer_s = ctx->s;
@@ -1112,7 +1119,7 @@ int enqueue_step_loop(ac_ctx *ctx, cudaGraph_t top, bool energy, StepGraph &sg) 
     if (!rc) rc = enqueue_smooth_resid(ctx, S, true);
     if (rc) return rc;
     AC_RUN(AC_PROF_RESID,
-           (k_ctl_cycle<<<1, 1, 0, ctx->s>>>(ctx->ctl, ctx->rho, ctx->p.nu1 + ctx->p.nu2, h_cyc), 1));
+           (ac::launch(k_ctl_cycle, 1, 1, 0, ctx->s, ctx->ctl, ctx->rho, ctx->p.nu1 + ctx->p.nu2, h_cyc), 1));
     rc = end_body(ctx->s);
     if (rc) return rc;
     ctx->s = outer_s;
@@ -1130,7 +1137,7 @@ int enqueue_step_loop(ac_ctx *ctx, cudaGraph_t top, bool energy, StepGraph &sg) 
       AC_RUNB(AC_PROF_OUTER, (double)ctx->n * ctx->N * 24,
               o->outer_resid(ctx->u, (const float *)ctx->b, ctx->g0, ctx->r32, ctx->u32, ctx->rho, true, ctx->s));
       AC_RUN(AC_PROF_OUTER,
-             (k_ctl_outer<<<1, 1, 0, ctx->s>>>(ctx->ctl, ctx->rho, accept, ctx->p.tol, kInnerTolFrac, kInnerReduction,
+             (ac::launch(k_ctl_outer, 1, 1, 0, ctx->s, ctx->ctl, ctx->rho, accept, ctx->p.tol, kInnerTolFrac, kInnerReduction,
                                                ctx->p.max_cycles, kInnerMaxCycles, ctx->p.nu1, h_out),
               1));
       return AC_OK;
@@ -1142,14 +1149,14 @@ int enqueue_step_loop(ac_ctx *ctx, cudaGraph_t top, bool energy, StepGraph &sg) 
     ctx->s = ctx->body_s[0];
     ctx->capturing = &cnt_pass;
     const int64_t xs = fine_slots(ctx->n) * ctx->N;
-    AC_RUN(AC_PROF_OUTER, (k_zero_unless_warm<<<(unsigned)std::min<int64_t>((xs + 255) / 256, 8 * ctx->sms), 256, 0,
-                                                ctx->s>>>(ctx->ctl, (float *)S.x, xs),
+    AC_RUN(AC_PROF_OUTER, (ac::launch(k_zero_unless_warm, (unsigned)std::min<int64_t>((xs + 255) / 256, 8 * ctx->sms), 256, 0,
+                                                ctx->s, ctx->ctl, (float *)S.x, xs),
                            1));
     rc = solve(1);
     if (rc) return rc;
     AC_RUNB(AC_PROF_OUTER, (double)ctx->n * ctx->N * 20,
             o->outer_update(ctx->u, (const float *)S.x, ctx->g0, ctx->s));
-    AC_RUN(AC_PROF_OUTER, (k_ctl_after_update<<<1, 1, 0, ctx->s>>>(ctx->ctl), 1));
+    AC_RUN(AC_PROF_OUTER, (ac::launch(k_ctl_after_update, 1, 1, 0, ctx->s, ctx->ctl), 1));
     rc = outer_resid();
     if (rc) return rc;
     rc = end_body(ctx->s);
@@ -1157,7 +1164,7 @@ int enqueue_step_loop(ac_ctx *ctx, cudaGraph_t top, bool energy, StepGraph &sg) 
     ctx->s = top_s;
     ctx->capturing = &cnt_fixed;
   }
-  AC_RUN(AC_PROF_SETUP, (k_ctl_step_end<<<1, 1, 0, ctx->s>>>(ctx->ctl, mixed ? 0 : 1), 1));
+  AC_RUN(AC_PROF_SETUP, (ac::launch(k_ctl_step_end, 1, 1, 0, ctx->s, ctx->ctl, mixed ? 0 : 1), 1));
   sg.fixed = cnt_fixed.total;
   sg.per_pass = cnt_pass.total;
   sg.per_cycle = cnt_cycle.total;
@@ -1224,7 +1231,7 @@ int loop_stats(ac_ctx *ctx, const StepGraph &sg, int n_steps, ac_stats *out) {
 // ac_step with the device-side loop: one graph launch per time step and one
 // synchronisation per call.
 int step_device(ac_ctx *ctx, int n_steps, ac_stats *out) {
-  AC_CUDA((k_ctl_reset<<<1, 1, 0, ctx->s>>>(ctx->ctl, ctx->delta_warm ? 1 : 0), cudaGetLastError()));
+  AC_CUDA((ac::launch(k_ctl_reset, 1, 1, 0, ctx->s, ctx->ctl, ctx->delta_warm ? 1 : 0), cudaGetLastError()));
   for (int t = 0; t < n_steps; ++t)
     AC_CUDA(cudaGraphLaunch(ctx->step_graph[(out && t == n_steps - 1) ? 1 : 0].exec, ctx->s));
   AC_CUDA(cudaMemcpyAsync(ctx->h_ctl, ctx->ctl, sizeof(LoopCtl), cudaMemcpyDeviceToHost, ctx->s));
@@ -2490,7 +2497,7 @@ int batch_step_one_graph(ac_batch *b, int n_steps, std::vector<ac_stats> &st, st
   for (cudaStream_t st2 : b->streams) AC_CUDA(cudaStreamSynchronize(st2));
   const int count = (int)b->ctx.size();
   for (int k = 0; k < count; ++k)
-    AC_CUDA((k_ctl_reset<<<1, 1, 0, s0>>>(b->ctx[k]->ctl, b->ctx[k]->delta_warm ? 1 : 0), cudaGetLastError()));
+    AC_CUDA((ac::launch(k_ctl_reset, 1, 1, 0, s0, b->ctx[k]->ctl, b->ctx[k]->delta_warm ? 1 : 0), cudaGetLastError()));
   for (int t = 0; t < n_steps; ++t) AC_CUDA(cudaGraphLaunch(b->group, s0));
   for (int k = 0; k < count; ++k)
     AC_CUDA(cudaMemcpyAsync(b->ctx[k]->h_ctl, b->ctx[k]->ctl, sizeof(LoopCtl), cudaMemcpyDeviceToHost, s0));

@@ -129,6 +129,7 @@ __device__ __forceinline__ void block_sum_store1(T v, double *dst) {
 // for a fixed grid and block size).
 static __global__ void __launch_bounds__(1024) k_colsum(const double *__restrict__ part, int rows, int cols,
                                                         double *__restrict__ out) {
+  pdl_sync();
   __shared__ double sm[32];
   const int c = blockIdx.x, B = blockDim.x;
   double s0 = 0.0, s1 = 0.0, s2 = 0.0, s3 = 0.0;
@@ -157,6 +158,7 @@ static __global__ void __launch_bounds__(1024) k_colsum(const double *__restrict
 // ---------------------------------------------------------------------------
 template <typename TI>
 __global__ void k_moments(const TI *__restrict__ img, Geo g, double *__restrict__ mom) {
+  pdl_sync();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y;
   if (x > g.W || y > g.H) return;
@@ -195,6 +197,7 @@ __device__ __forceinline__ uint64_t splitmix64(uint64_t z) {
 
 template <int N>
 __global__ void k_init_random(double *__restrict__ u, int64_t n, uint64_t seed) {
+  pdl_sync();
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
   // -log U in float for a uniform U on the 2^23 midpoints (j + 1/2) 2^-23
@@ -226,6 +229,7 @@ __global__ void k_init_random(double *__restrict__ u, int64_t n, uint64_t seed) 
 template <int N, bool ENERGY>
 __global__ void __launch_bounds__(kBlock) k_means_partial(const double *__restrict__ u, const double *__restrict__ mom,
                                                           Geo g, double *__restrict__ part) {
+  pdl_sync();
   constexpr int Q = ENERGY ? 7 : 4;
   double acc[Q * N];
 #pragma unroll
@@ -273,6 +277,7 @@ __global__ void __launch_bounds__(kBlock) k_means_partial(const double *__restri
 template <int N, bool ENERGY>
 __global__ void k_means_finish(const double *__restrict__ tot, double *__restrict__ c, double *__restrict__ energy,
                                double eps, double lam) {
+  pdl_sync();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   double E = 0.0;
   for (int i = 0; i < N; ++i) {
@@ -298,6 +303,7 @@ __global__ void k_means_finish(const double *__restrict__ tot, double *__restric
 template <int N>
 __global__ void k_rhs(const double *__restrict__ u, const double *__restrict__ mom, const double *__restrict__ c, Geo g,
                       double a1, double tl, double *__restrict__ b) {
+  pdl_sync();
   // per phase, once per block: 2 tau lambda c_i (RGB) and tau lambda |c_i|^2,
   // so that b_i = a1 m0 u_i - tau lambda m2 + (2 tau lambda c_i).m1
   //             - (tau lambda |c_i|^2) m0
@@ -342,6 +348,7 @@ template <int N, bool ENERGY>
 __global__ void __launch_bounds__(kBlock, 2) k_means_partial_df(const double *__restrict__ u,
                                                              const double *__restrict__ mom, Geo g,
                                                              double *__restrict__ part) {
+  pdl_sync();
   // 4N sums per phase (k_means_partial's q = 0..3), and with ENERGY three
   // sums over all phases: u m2, m0 u (1 - u), w (u_a - u_b)^2
   constexpr int QN = ENERGY ? 4 * N + 3 : 4 * N;
@@ -420,6 +427,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_means_partial_df(const double *__
 template <int N>
 __global__ void k_means_finish_df(const double *__restrict__ tot, double *__restrict__ c, double *__restrict__ energy,
                                   double eps, double lam) {
+  pdl_sync();
   if (threadIdx.x != 0 || blockIdx.x != 0) return;
   double fit = 0.0;
   for (int i = 0; i < N; ++i) {
@@ -438,6 +446,7 @@ __global__ void k_means_finish_df(const double *__restrict__ tot, double *__rest
 template <int N>
 __global__ void k_rhs_df(const double *__restrict__ u, const double *__restrict__ mom, const double *__restrict__ c,
                          Geo g, double a1, double tl, float *__restrict__ b) {
+  pdl_sync();
   // per phase, once per block: 2 tau lambda c_i (RGB) and tau lambda |c_i|^2
   // as double-floats; a1 = 1 + 2 tau/eps and tau lambda likewise
   __shared__ float coef[N][4][2];
@@ -513,6 +522,7 @@ template <int N>
 __global__ void __launch_bounds__(kBlock) k_outer_resid(const double *__restrict__ u, const float *__restrict__ b, Geo g,
                                                         float *__restrict__ r32, float *__restrict__ u32,
                                                         double *__restrict__ rho) {
+  pdl_sync();
   const int x = blockIdx.x * blockDim.x + threadIdx.x;
   const int y = blockIdx.y;
   double e = 0.0;
@@ -769,6 +779,7 @@ __global__ void __launch_bounds__(kOrThreads, kOrMinBlocks) k_outer_resid_df(con
                                                                const float *__restrict__ b, Geo g,
                                                                float *__restrict__ r32, float *__restrict__ u32,
                                                                double *__restrict__ rho) {
+  pdl_sync();
   __shared__ float s_h[2][N][kOrThreads], s_l[2][N][kOrThreads];
   extern __shared__ __align__(16) unsigned char or_ring[];
   // slots: u of rows in flight at [0, 2), b at [2, 4)
@@ -837,6 +848,7 @@ __global__ void __launch_bounds__(kOrThreads, kOrMinBlocks) k_outer_resid_df(con
 // its warp-wide skips of binary64 operations by __reduce_or_sync.
 template <int N>
 __global__ void k_outer_update(double *__restrict__ u, const float *__restrict__ delta, Geo g) {
+  pdl_sync();
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
   if (x > g.W) return;
   const unsigned lanes = __activemask();
@@ -869,6 +881,7 @@ __global__ void __launch_bounds__(kBlock) k_smooth_fine(T *__restrict__ x, const
                                                         const double *__restrict__ omega, Geo g, int color,
                                                         T *__restrict__ rt, uint8_t *__restrict__ mask,
                                                         MaskDirty dirty, double *__restrict__ rho) {
+  pdl_sync();
   const int y = blockIdx.y;
   // the residual that follows accumulates into rho and the free-node count
   if (MASK && rho && blockIdx.x == 0 && y == 0 && threadIdx.x == 0) rho[0] = rho[1] = 0.0;
@@ -950,6 +963,7 @@ __global__ void __launch_bounds__(kBlock) k_fine_resid(const T *__restrict__ x, 
                                                        const T *__restrict__ ob, Geo g, T *__restrict__ rt,
                                                        uint8_t *__restrict__ mask, double *__restrict__ rho,
                                                        int color, MaskDirty dirty) {
+  pdl_sync();
   // color < 0: every node; color 0 or 1: the nodes of that colour only (the
   // other colour's share was stored by the last smoothing pass)
   const int y = blockIdx.y;
@@ -1054,6 +1068,7 @@ __global__ void __launch_bounds__(kTileThreads) k_restrict0(const T *__restrict_
                                                             const T *__restrict__ opc, T *__restrict__ rc,
                                                             const uint64_t *__restrict__ tiles,
                                                             const int *__restrict__ count) {
+  pdl_sync();
   if (!tiles) {
     restrict0_tile<T, N>(t, gf, gc, opc, rc, (int)blockIdx.x, (int)blockIdx.y, (1u << N) - 1u, (1u << N) - 1u);
     return;
@@ -1135,6 +1150,7 @@ template <typename T, int N>
 __global__ void __launch_bounds__(kTileThreads) k_restrict_tiled(const T *__restrict__ t, Geo gf, Geo gc,
                                                                  const T *__restrict__ opc, T *__restrict__ rc,
                                                                  TileList L) {
+  pdl_sync();
   for_each_tile(L, gc, [&](int tx, int ty, int i, bool dying) {
     const int64_t nc = (int64_t)gc.Wn * (gc.H + 1);
     const int X = tx * kJ2X + (int)(threadIdx.x % kJ2X);
@@ -1152,6 +1168,7 @@ __global__ void __launch_bounds__(kTileThreads) k_restrict_tiled(const T *__rest
 
 template <typename T, int N>
 __global__ void k_restrict(const T *__restrict__ t, Geo gf, Geo gc, const T *__restrict__ opc, T *__restrict__ rc) {
+  pdl_sync();
   const int X = blockIdx.x * blockDim.x + threadIdx.x, Y = blockIdx.y, i = blockIdx.z;
   if (X > gc.W) return;
   constexpr int dx[7] = {0, 1, -1, 0, 0, 1, -1};
@@ -1335,6 +1352,7 @@ __global__ void __launch_bounds__(kTileThreads) k_galerkin0(const uint8_t *__res
                                                             uint64_t *__restrict__ tiles, int *__restrict__ count,
                                                             uint8_t *__restrict__ dirty,
                                                             uint8_t *__restrict__ changed) {
+  pdl_sync();
   __shared__ unsigned s_now, s_prev;
   __shared__ int s_base, s_dirty;
   unsigned wmask = (1u << N) - 1u;
@@ -1499,6 +1517,7 @@ __device__ __forceinline__ void galerkin_phase(const T *__restrict__ opf, const 
 // per (coarse node, phase) (phase = blockIdx.z; phase-major arrays).
 template <typename T, int N>
 __global__ void __launch_bounds__(kBlock) k_galerkin(const T *__restrict__ opf, Geo gf, Geo gc, T *__restrict__ opc) {
+  pdl_sync();
   const int X = blockIdx.x * blockDim.x + threadIdx.x, Y = blockIdx.y, i = blockIdx.z;
   if (X > gc.W) return;
   const int64_t nf = (int64_t)gf.Wn * (gf.H + 1), nc = (int64_t)gc.Wn * (gc.H + 1);
@@ -1541,6 +1560,7 @@ __global__ void __launch_bounds__(kTileThreads) k_galerkin_tiled(const T *__rest
                                                                  int *__restrict__ count,
                                                                  const uint8_t *__restrict__ changed_f,
                                                                  uint8_t *__restrict__ changed_c) {
+  pdl_sync();
   __shared__ int s_fine, s_changed;
   __shared__ unsigned s_prev;
   const int i = blockIdx.z;
@@ -1936,6 +1956,7 @@ constexpr int pair_min_blocks(int elem, bool gs) { return gs ? (elem == 4 ? AC_G
 template <typename T, int N, bool ZERO_IN, bool GS>
 __global__ void __launch_bounds__(GS ? kGsThreads : kJ2Threads, pair_min_blocks(sizeof(T), GS)) k_coarse_pair(const T *__restrict__ op, const T *__restrict__ r,
                                                                   const T *vin, T *vout, Geo g, TileList L) {
+  pdl_sync();
   for_each_tile(L, g, [&](int tx, int ty, int i, bool dying) {
     const int64_t nc = (int64_t)g.Wn * (g.H + 1);
     if (dying)
@@ -2051,6 +2072,7 @@ template <typename T, int N, bool GS>
 __global__ void __launch_bounds__(GS ? kGsThreads : kJ2Threads, pair_min_blocks(sizeof(T), GS)) k_coarse_pair_resid(const T *__restrict__ op,
                                                                         const T *__restrict__ r, T *__restrict__ vout,
                                                                         T *__restrict__ tout, Geo g, TileList L) {
+  pdl_sync();
   for_each_tile(L, g, [&](int tx, int ty, int i, bool dying) {
     const int64_t nc = (int64_t)g.Wn * (g.H + 1);
     if (dying)
@@ -2273,6 +2295,7 @@ __device__ __forceinline__ void tail_galerkin(const TailLevel<T> &F, const TailL
 template <typename T, int N, bool GS>
 __global__ void __launch_bounds__(kTailThreads) k_coarse_tail(TailArgs a, const T *__restrict__ r0, T *__restrict__ v0,
                                                               int coarse_sweeps, int coarsest_sweeps) {
+  pdl_sync();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   T *const base = reinterpret_cast<T *>(smem_raw);
   const int i = blockIdx.x;
@@ -2372,6 +2395,7 @@ __device__ __forceinline__ void coarse_resid_row(const T *__restrict__ op, const
 template <typename T, int N>
 __global__ void k_coarse_resid(const T *__restrict__ op, const T *__restrict__ r, const T *__restrict__ v, Geo g,
                                T *__restrict__ t) {
+  pdl_sync();
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y, i = blockIdx.z;
   if (x > g.W) return;
   coarse_resid_row<T, N>(op, r, v, g, t, x, y, i);
@@ -2382,6 +2406,7 @@ template <typename T, int N>
 __global__ void __launch_bounds__(kTileThreads) k_coarse_resid_tiled(const T *__restrict__ op, const T *__restrict__ r,
                                                                      const T *__restrict__ v, Geo g, T *__restrict__ t,
                                                                      TileList L) {
+  pdl_sync();
   for_each_tile(L, g, [&](int tx, int ty, int i, bool dying) {
     const int x = tx * kJ2X + (int)(threadIdx.x % kJ2X);
 #pragma unroll
@@ -2447,6 +2472,7 @@ __device__ __forceinline__ void prolong_at(const T *vc, const Geo &gc, int x, in
 template <typename T, int N, bool PHASES_IN_Z>
 __global__ void k_prolong_add(const T *__restrict__ vc, Geo gf, Geo gc, const T *__restrict__ opf,
                               T *__restrict__ vf) {
+  pdl_sync();
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
   if (x > gf.W) return;
   const int64_t nc = (int64_t)gc.Wn * (gc.H + 1), nf = (int64_t)gf.Wn * (gf.H + 1);
@@ -2471,6 +2497,7 @@ template <typename T, int N>
 __global__ void __launch_bounds__(kTileThreads) k_prolong_add_tiled(const T *__restrict__ vc, Geo gf, Geo gc,
                                                                     const T *__restrict__ opf, T *__restrict__ vf,
                                                                     TileList L) {
+  pdl_sync();
   for_each_tile(L, gf, [&](int tx, int ty, int i, bool dying) {
     if (dying) return;
     const int64_t nc = (int64_t)gc.Wn * (gc.H + 1), nf = (int64_t)gf.Wn * (gf.H + 1);
@@ -2525,6 +2552,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 6 : 4) k_ls_dir(const
                                                    const T *__restrict__ rt, const T *__restrict__ v1,
                                                    const uint8_t *__restrict__ mask, Geo gf, Geo gc, int chunks,
                                                    T *__restrict__ d, double *__restrict__ part) {
+  pdl_sync();
   NodeSum<T> dot;
   const int64_t nodes = (int64_t)gf.Wn * (gf.H + 1);
   for (int q = 0; q < chunks; ++q) {
@@ -2580,6 +2608,7 @@ template <typename T, int N>
 __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 6 : 5) k_ls_curv(const T *__restrict__ d, const uint8_t *__restrict__ mask, Geo g,
                                                     int chunks, double *part, unsigned *done,
                                                     double *__restrict__ omega) {
+  pdl_sync();
   const int blocks = (int)gridDim.x;
   NodeSum<T> dot;
   const int64_t nodes = (int64_t)g.Wn * (g.H + 1);
@@ -2661,6 +2690,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 6 : 5) k_ls_curv(cons
 template <int N>
 __global__ void k_adj_prepare(const double *__restrict__ up, const double *__restrict__ g, int64_t n,
                               double *__restrict__ freeset, double *__restrict__ rhs) {
+  pdl_sync();
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= n) return;
   double uk[N], gk[N], f[N];
@@ -2687,6 +2717,7 @@ __global__ void __launch_bounds__(kBlock) k_adj_accum(const double *__restrict__
                                                       const double *__restrict__ up, const double *__restrict__ mom,
                                                       const double *__restrict__ c, Geo g, double tau, double eps,
                                                       double lam, double *__restrict__ gm, double *__restrict__ part) {
+  pdl_sync();
   double acc[2 + 3 * N];
 #pragma unroll
   for (int k = 0; k < 2 + 3 * N; ++k) acc[k] = 0.0;
@@ -2735,6 +2766,7 @@ __global__ void k_adj_back(const double *__restrict__ w, const double *__restric
                            const double *__restrict__ c, const double *__restrict__ tot,
                            const double *__restrict__ mass, Geo g, double a1, double *__restrict__ gout,
                            double *__restrict__ gm) {
+  pdl_sync();
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
   if (x > g.W) return;
   const int64_t n = (int64_t)y * g.Wn + x;
@@ -2768,6 +2800,7 @@ __global__ void k_adj_back(const double *__restrict__ w, const double *__restric
 // m1 (I) and m2 (|I|^2): dL/dI_p = sum_n w_np (dL/dm1_n + 2 I_p dL/dm2_n).
 static __global__ void k_adj_image(const double *__restrict__ gm, const double *__restrict__ img, Geo g,
                             double *__restrict__ gimg) {
+  pdl_sync();
   const int px = blockIdx.x * blockDim.x + threadIdx.x, py = blockIdx.y;
   if (px >= g.W) return;
   const int64_t n00 = (int64_t)py * g.Wn + px;
@@ -2789,6 +2822,7 @@ static __global__ void k_adj_image(const double *__restrict__ gm, const double *
 
 // acc[0..1] += tot[0..1] (the lambda and eps gradients of one step).
 static __global__ void k_adj_scalars(const double *__restrict__ tot, double *__restrict__ acc) {
+  pdl_sync();
   if (threadIdx.x == 0 && blockIdx.x == 0) {
     acc[0] += tot[0];
     acc[1] += tot[1];
@@ -2802,6 +2836,7 @@ static __global__ void k_adj_scalars(const double *__restrict__ tot, double *__r
 template <int N>
 __global__ void k_tangent_apply(const double *__restrict__ p, const double *__restrict__ f, Geo g,
                                 double *__restrict__ q) {
+  pdl_sync();
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
   if (x > g.W) return;
   const int64_t n = (int64_t)y * g.Wn + x;
@@ -2821,6 +2856,7 @@ __global__ void k_tangent_apply(const double *__restrict__ p, const double *__re
 static __global__ void __launch_bounds__(kBlock) k_dot2(const double *__restrict__ a0, const double *__restrict__ b0,
                                                         const double *__restrict__ a1, const double *__restrict__ b1,
                                                         int64_t count, double *__restrict__ part) {
+  pdl_sync();
   double acc[2] = {0.0, 0.0};
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < count; k += (int64_t)gridDim.x * blockDim.x) {
     acc[0] += a0[k] * b0[k];
@@ -2832,6 +2868,7 @@ static __global__ void __launch_bounds__(kBlock) k_dot2(const double *__restrict
 // x += alpha p, r -= alpha q.
 static __global__ void k_fcg_step(double *__restrict__ x, double *__restrict__ r, const double *__restrict__ p,
                                   const double *__restrict__ q, double alpha, int64_t count) {
+  pdl_sync();
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= count) return;
   x[k] += alpha * p[k];
@@ -2840,12 +2877,14 @@ static __global__ void k_fcg_step(double *__restrict__ x, double *__restrict__ r
 
 // p = z + beta p.
 static __global__ void k_fcg_dir(double *__restrict__ p, const double *__restrict__ z, double beta, int64_t count) {
+  pdl_sync();
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= count) return;
   p[k] = z[k] + beta * p[k];
 }
 
 static __global__ void k_absmax(const double *__restrict__ v, int64_t count, double *__restrict__ out) {
+  pdl_sync();
   double e = 0.0;
   for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < count; k += (int64_t)gridDim.x * blockDim.x)
     e = nanmax<double>(e, fabs(v[k]));
@@ -2895,6 +2934,7 @@ __device__ __forceinline__ int argmax_low(const double (&v)[N]) {
 template <int N>
 __global__ void k_composite(const double *__restrict__ u, const double *__restrict__ c, Geo g, int r, int rounded,
                             float *__restrict__ out) {
+  pdl_sync();
   const int W0 = g.W >> r, H0 = g.H >> r;
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
   if (x >= W0 || y >= H0) return;
@@ -2917,6 +2957,7 @@ __global__ void k_composite(const double *__restrict__ u, const double *__restri
 // Node label = argmax_i u_n,i (lowest index on ties), on the solve grid.
 template <int N>
 __global__ void k_labels(const double *__restrict__ u, Geo g, int8_t *__restrict__ node_lab) {
+  pdl_sync();
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
   if (x > g.W) return;
   const int64_t n = (int64_t)y * g.Wn + x;
@@ -2930,6 +2971,7 @@ __global__ void k_labels(const double *__restrict__ u, Geo g, int8_t *__restrict
 // cells; lowest index on ties.  Output (H >> r) x (W >> r).
 template <int N>
 __global__ void k_pixel_labels(const double *__restrict__ u, Geo g, int r, int8_t *__restrict__ pix_lab) {
+  pdl_sync();
   const int W0 = g.W >> r, H0 = g.H >> r;
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
   if (x >= W0 || y >= H0) return;
@@ -2981,6 +3023,7 @@ __global__ void k_pixel_labels(const double *__restrict__ u, Geo g, int r, int8_
 // preconditioner takes the FCG residual and returns its correction this way.
 template <int N>
 __global__ void k_to_split32(const double *__restrict__ in, Geo g, float *__restrict__ out) {
+  pdl_sync();
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
   if (x > g.W) return;
   double v[N];
@@ -2998,6 +3041,7 @@ __global__ void k_to_split32(const double *__restrict__ in, Geo g, float *__rest
 template <int N>
 __global__ void k_from_split32(const float *__restrict__ in, Geo g, const double *__restrict__ freeset,
                                double *__restrict__ out) {
+  pdl_sync();
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
   if (x > g.W) return;
   const int64_t n = (int64_t)y * g.Wn + x;
@@ -3017,6 +3061,7 @@ __global__ void k_from_split32(const float *__restrict__ in, Geo g, const double
 // Kernel-level projection of count independent N-vectors onto the simplex.
 template <int N>
 __global__ void k_project(const double *y, double *x, int64_t count) {
+  pdl_sync();
   const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= count) return;
   double v[N];

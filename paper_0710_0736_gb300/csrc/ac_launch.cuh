@@ -68,10 +68,10 @@ struct SolverLaunch {
       for (int c = 0; c < 2; ++c) {
         const T *cr = k == 0 && c == 0 ? (const T *)corr : nullptr;
         if (mask && k == sweeps - 1 && c == 1)
-          k_smooth_fine<T, N, FORM, true><<<grid, kBlock, 0, s>>>((T *)x, (const T *)rhs, (const T *)ob, cr, omega,
+          launch(k_smooth_fine<T, N, FORM, true>, grid, kBlock, 0, s, (T *)x, (const T *)rhs, (const T *)ob, cr, omega,
                                                                 g, c, (T *)rt, mask, dirty, rho);
         else
-          k_smooth_fine<T, N, FORM, false><<<grid, kBlock, 0, s>>>((T *)x, (const T *)rhs, (const T *)ob, cr, omega,
+          launch(k_smooth_fine<T, N, FORM, false>, grid, kBlock, 0, s, (T *)x, (const T *)rhs, (const T *)ob, cr, omega,
                                                                  g, c, nullptr, mask, MaskDirty{nullptr, 0, 0},
                                                                  nullptr);
       }
@@ -81,7 +81,7 @@ struct SolverLaunch {
   static int resid(const void *x, const void *rhs, const void *ob, const Geo &g, void *rt, uint8_t *mask,
                    double *rho, int color, const MaskDirty &dirty, cudaStream_t s) {
     const dim3 grid = color < 0 ? row_grid(g.W + 1, g.H + 1) : row_grid((g.W + 2) / 2, g.H + 1);
-    k_fine_resid<T, N, FORM><<<grid, kBlock, 0, s>>>((const T *)x, (const T *)rhs, (const T *)ob, g, (T *)rt, mask,
+    launch(k_fine_resid<T, N, FORM>, grid, kBlock, 0, s, (const T *)x, (const T *)rhs, (const T *)ob, g, (T *)rt, mask,
                                                    rho, color, dirty);
     return 1;
   }
@@ -89,14 +89,14 @@ struct SolverLaunch {
                        cudaStream_t s) {
     const dim3 grid = L1 ? list_grid(L1, L1->cap / N, k_restrict0<T, N>, kTileThreads)
                          : dim3((unsigned)tiles_x(gc), (unsigned)tiles_y(gc));
-    k_restrict0<T, N><<<grid, kTileThreads, 0, s>>>((const T *)rt, gf, gc, (const T *)op1, (T *)r1,
+    launch(k_restrict0<T, N>, grid, kTileThreads, 0, s, (const T *)rt, gf, gc, (const T *)op1, (T *)r1,
                                                   L1 ? L1->tiles : nullptr, L1 ? L1->count + 1 : nullptr);
     return 1;
   }
   static int galerkin0(const uint8_t *mask, const Geo &gf, const Geo &gc, const Galerkin0Table &tab, void *op,
                        const LevelLists *L1, uint8_t *dirty, cudaStream_t s) {
     const dim3 grid((unsigned)tiles_x(gc), (unsigned)tiles_y(gc));
-    k_galerkin0<T, N><<<grid, kTileThreads, 0, s>>>(mask, gf, gc, tab, (T *)op, L1 ? L1->flags : nullptr,
+    launch(k_galerkin0<T, N>, grid, kTileThreads, 0, s, mask, gf, gc, tab, (T *)op, L1 ? L1->flags : nullptr,
                                                   L1 ? L1->items : nullptr, L1 ? L1->tiles : nullptr,
                                                   L1 ? L1->count : nullptr, L1 ? L1->dirty : dirty,
                                                   L1 ? L1->changed : nullptr);
@@ -106,11 +106,11 @@ struct SolverLaunch {
                       const LevelLists *Lc, cudaStream_t s) {
     if (Lc) {
       const dim3 grid((unsigned)tiles_x(gc), (unsigned)tiles_y(gc), (unsigned)N);
-      k_galerkin_tiled<T, N><<<grid, kTileThreads, 0, s>>>((const T *)opf, gf, gc, (T *)opc, Lf->flags, Lc->flags,
+      launch(k_galerkin_tiled<T, N>, grid, kTileThreads, 0, s, (const T *)opf, gf, gc, (T *)opc, Lf->flags, Lc->flags,
                                                          Lc->items, Lc->count, Lf->changed, Lc->changed);
     } else {
       const PhaseLaunch L = phase_grid(gc.W + 1, gc.H + 1, N);
-      k_galerkin<T, N><<<L.grid, L.block, 0, s>>>((const T *)opf, gf, gc, (T *)opc);
+      launch(k_galerkin<T, N>, L.grid, L.block, 0, s, (const T *)opf, gf, gc, (T *)opc);
     }
     return 1;
   }
@@ -125,12 +125,12 @@ struct SolverLaunch {
         // v is not read: the pair can write it
         constexpr int th = GS ? kGsThreads : kJ2Threads;
         const dim3 grid = tile_grid(g, L, N, k_coarse_pair<T, N, true, GS>, th);
-        k_coarse_pair<T, N, true, GS><<<grid, th, 0, s>>>((const T *)op, (const T *)r, (const T *)v, (T *)v, g, tf);
+        launch(k_coarse_pair<T, N, true, GS>, grid, th, 0, s, (const T *)op, (const T *)r, (const T *)v, (T *)v, g, tf);
       } else {
         void *nxt = cur == v ? tmp : v;
         constexpr int th = GS ? kGsThreads : kJ2Threads;
         const dim3 grid = tile_grid(g, L, N, k_coarse_pair<T, N, false, GS>, th);
-        k_coarse_pair<T, N, false, GS><<<grid, th, 0, s>>>((const T *)op, (const T *)r, (const T *)cur, (T *)nxt, g,
+        launch(k_coarse_pair<T, N, false, GS>, grid, th, 0, s, (const T *)op, (const T *)r, (const T *)cur, (T *)nxt, g,
                                                             tf);
         cur = nxt;
       }
@@ -153,12 +153,12 @@ struct SolverLaunch {
     if constexpr (sizeof(T) == 4) {
       constexpr int th = GS ? kGsThreads : kJ2Threads;
       const dim3 grid = tile_grid(g, L, N, k_coarse_pair_resid<T, N, GS>, th);
-      k_coarse_pair_resid<T, N, GS><<<grid, th, 0, s>>>((const T *)op, (const T *)r, (T *)v, (T *)t, g, tf);
+      launch(k_coarse_pair_resid<T, N, GS>, grid, th, 0, s, (const T *)op, (const T *)r, (T *)v, (T *)t, g, tf);
       return 1;
     } else {
       constexpr int th = GS ? kGsThreads : kJ2Threads;
       const dim3 grid = tile_grid(g, L, N, k_coarse_pair<T, N, true, GS>, th);
-      k_coarse_pair<T, N, true, GS><<<grid, th, 0, s>>>((const T *)op, (const T *)r, (const T *)v, (T *)v, g, tf);
+      launch(k_coarse_pair<T, N, true, GS>, grid, th, 0, s, (const T *)op, (const T *)r, (const T *)v, (T *)v, g, tf);
       return 1 + coarse_resid(op, r, v, g, t, L, s);
     }
   }
@@ -169,38 +169,38 @@ struct SolverLaunch {
   static int coarse_resid(const void *op, const void *r, const void *v, const Geo &g, void *t, const LevelLists *Lv,
                           cudaStream_t s) {
     if (Lv) {
-      k_coarse_resid_tiled<T, N><<<list_grid(Lv, Lv->cap, k_coarse_resid_tiled<T, N>, kTileThreads), kTileThreads, 0,
-                                   s>>>((const T *)op, (const T *)r, (const T *)v, g,
+      launch(k_coarse_resid_tiled<T, N>, list_grid(Lv, Lv->cap, k_coarse_resid_tiled<T, N>, kTileThreads), kTileThreads, 0,
+                                   s, (const T *)op, (const T *)r, (const T *)v, g,
                                                                     (T *)t, item_list(Lv));
     } else {
       const PhaseLaunch L = phase_grid(g.W + 1, g.H + 1, N);
-      k_coarse_resid<T, N><<<L.grid, L.block, 0, s>>>((const T *)op, (const T *)r, (const T *)v, g, (T *)t);
+      launch(k_coarse_resid<T, N>, L.grid, L.block, 0, s, (const T *)op, (const T *)r, (const T *)v, g, (T *)t);
     }
     return 1;
   }
   static int restrict_(const void *t, const Geo &gf, const Geo &gc, const void *opc, void *rc, const LevelLists *Lc,
                        cudaStream_t s) {
     if (Lc) {
-      k_restrict_tiled<T, N><<<list_grid(Lc, Lc->cap, k_restrict_tiled<T, N>, kTileThreads), kTileThreads, 0, s>>>((const T *)t, gf, gc, (const T *)opc, (T *)rc,
+      launch(k_restrict_tiled<T, N>, list_grid(Lc, Lc->cap, k_restrict_tiled<T, N>, kTileThreads), kTileThreads, 0, s, (const T *)t, gf, gc, (const T *)opc, (T *)rc,
                                                                item_list(Lc));
     } else {
       const PhaseLaunch L = phase_grid(gc.W + 1, gc.H + 1, N);
-      k_restrict<T, N><<<L.grid, L.block, 0, s>>>((const T *)t, gf, gc, (const T *)opc, (T *)rc);
+      launch(k_restrict<T, N>, L.grid, L.block, 0, s, (const T *)t, gf, gc, (const T *)opc, (T *)rc);
     }
     return 1;
   }
   static int prolong_add(const void *vc, const Geo &gf, const Geo &gc, const void *opf, void *vf, const LevelLists *Lf,
                          cudaStream_t s) {
     if (Lf) {
-      k_prolong_add_tiled<T, N><<<list_grid(Lf, Lf->cap, k_prolong_add_tiled<T, N>, kTileThreads), kTileThreads, 0,
-                                  s>>>((const T *)vc, gf, gc, (const T *)opf, (T *)vf,
+      launch(k_prolong_add_tiled<T, N>, list_grid(Lf, Lf->cap, k_prolong_add_tiled<T, N>, kTileThreads), kTileThreads, 0,
+                                  s, (const T *)vc, gf, gc, (const T *)opf, (T *)vf,
                                                                   item_list(Lf));
     } else if ((int64_t)(gf.W + 1) * (gf.H + 1) >= kWideLevelNodes) {
-      k_prolong_add<T, N, false><<<row_grid(gf.W + 1, gf.H + 1), kBlock, 0, s>>>((const T *)vc, gf, gc,
+      launch(k_prolong_add<T, N, false>, row_grid(gf.W + 1, gf.H + 1), kBlock, 0, s, (const T *)vc, gf, gc,
                                                                                  (const T *)opf, (T *)vf);
     } else {
       const PhaseLaunch L = phase_grid(gf.W + 1, gf.H + 1, N);
-      k_prolong_add<T, N, true><<<L.grid, L.block, 0, s>>>((const T *)vc, gf, gc, (const T *)opf, (T *)vf);
+      launch(k_prolong_add<T, N, true>, L.grid, L.block, 0, s, (const T *)vc, gf, gc, (const T *)opf, (T *)vf);
     }
     return 1;
   }
@@ -216,7 +216,7 @@ struct SolverLaunch {
     // makes the barriers slower)
     const int64_t third = (int64_t)(a.W[0] / 3 + 1) * (a.H[0] + 1);
     const int threads = (int)std::min<int64_t>(kTailThreads, std::max<int64_t>(128, (third + 31) / 32 * 32));
-    k_coarse_tail<T, N, GS><<<N, threads, smem, s>>>(a, (const T *)r0, (T *)v0, coarse_sweeps, coarsest_sweeps);
+    launch(k_coarse_tail<T, N, GS>, N, threads, smem, s, a, (const T *)r0, (T *)v0, coarse_sweeps, coarsest_sweeps);
     return 1;
   }
   static int coarse_tail(const TailArgs &a, const void *r0, void *v0, int coarse_sweeps, int coarsest_sweeps,
@@ -236,9 +236,9 @@ struct SolverLaunch {
     const int64_t want = all <= 8 * kSet ? kSet : 4 * kSet;
     const int chunks = (int)((all + want - 1) / want);
     const unsigned grid = (unsigned)((all + chunks - 1) / chunks);
-    k_ls_dir<T, N, FORM><<<grid, kBlock, 0, s>>>((const T *)x, (const T *)ob, (const T *)rt, (const T *)v1, mask, gf,
+    launch(k_ls_dir<T, N, FORM>, grid, kBlock, 0, s, (const T *)x, (const T *)ob, (const T *)rt, (const T *)v1, mask, gf,
                                                gc, chunks, (T *)d, part);
-    k_ls_curv<T, N><<<grid, kBlock, 0, s>>>((const T *)d, mask, gf, chunks, part, done, omega);
+    launch(k_ls_curv<T, N>, grid, kBlock, 0, s, (const T *)d, mask, gf, chunks, part, done, omega);
     return 2;
   }
   static SolverOps table() {
@@ -251,15 +251,15 @@ struct SolverLaunch {
 template <int N>
 struct Launch {
   static int moments_f32(const float *img, const Geo &g, double *mom, cudaStream_t s) {
-    k_moments<float><<<row_grid(g.W + 1, g.H + 1), kBlock, 0, s>>>(img, g, mom);
+    launch(k_moments<float>, row_grid(g.W + 1, g.H + 1), kBlock, 0, s, img, g, mom);
     return 1;
   }
   static int moments_f64(const double *img, const Geo &g, double *mom, cudaStream_t s) {
-    k_moments<double><<<row_grid(g.W + 1, g.H + 1), kBlock, 0, s>>>(img, g, mom);
+    launch(k_moments<double>, row_grid(g.W + 1, g.H + 1), kBlock, 0, s, img, g, mom);
     return 1;
   }
   static int init_random(double *u, int64_t n, uint64_t seed, cudaStream_t s) {
-    k_init_random<N><<<blocks_for(n), kBlock, 0, s>>>(u, n, seed);
+    launch(k_init_random<N>, blocks_for(n), kBlock, 0, s, u, n, seed);
     return 1;
   }
   static int means(const double *u, const double *mom, const Geo &g, double *part, double *tot, double *c,
@@ -268,19 +268,19 @@ struct Launch {
     const int64_t b = (n + kBlock - 1) / kBlock;
     const int blocks = (int)(b < kMaxPartBlocks ? b : kMaxPartBlocks);
     if (energy) {
-      k_means_partial<N, true><<<blocks, kBlock, 0, s>>>(u, mom, g, part);
-      k_colsum<<<7 * N, 1024, 0, s>>>(part, blocks, 7 * N, tot);
-      k_means_finish<N, true><<<1, 32, 0, s>>>(tot, c, energy, eps, lam);
+      launch(k_means_partial<N, true>, blocks, kBlock, 0, s, u, mom, g, part);
+      launch(k_colsum, 7 * N, 1024, 0, s, part, blocks, 7 * N, tot);
+      launch(k_means_finish<N, true>, 1, 32, 0, s, tot, c, energy, eps, lam);
     } else {
-      k_means_partial<N, false><<<blocks, kBlock, 0, s>>>(u, mom, g, part);
-      k_colsum<<<4 * N, 1024, 0, s>>>(part, blocks, 4 * N, tot);
-      k_means_finish<N, false><<<1, 32, 0, s>>>(tot, c, nullptr, eps, lam);
+      launch(k_means_partial<N, false>, blocks, kBlock, 0, s, u, mom, g, part);
+      launch(k_colsum, 4 * N, 1024, 0, s, part, blocks, 4 * N, tot);
+      launch(k_means_finish<N, false>, 1, 32, 0, s, tot, c, nullptr, eps, lam);
     }
     return 3;
   }
   static int rhs(const double *u, const double *mom, const double *c, const Geo &g, double a1, double tl, double *b,
                  cudaStream_t s) {
-    k_rhs<N><<<row_grid(g.W + 1, g.H + 1), kBlock, 0, s>>>(u, mom, c, g, a1, tl, b);
+    launch(k_rhs<N>, row_grid(g.W + 1, g.H + 1), kBlock, 0, s, u, mom, c, g, a1, tl, b);
     return 1;
   }
   static int means_df(const double *u, const double *mom, const Geo &g, double *part, double *tot, double *c,
@@ -289,19 +289,19 @@ struct Launch {
     const int64_t b = (n + kBlock - 1) / kBlock;
     const int blocks = (int)(b < kMaxPartBlocks ? b : kMaxPartBlocks);
     if (energy) {
-      k_means_partial_df<N, true><<<blocks, kBlock, 0, s>>>(u, mom, g, part);
-      k_colsum<<<4 * N + 3, 1024, 0, s>>>(part, blocks, 4 * N + 3, tot);
-      k_means_finish_df<N><<<1, 32, 0, s>>>(tot, c, energy, eps, lam);
+      launch(k_means_partial_df<N, true>, blocks, kBlock, 0, s, u, mom, g, part);
+      launch(k_colsum, 4 * N + 3, 1024, 0, s, part, blocks, 4 * N + 3, tot);
+      launch(k_means_finish_df<N>, 1, 32, 0, s, tot, c, energy, eps, lam);
     } else {
-      k_means_partial_df<N, false><<<blocks, kBlock, 0, s>>>(u, mom, g, part);
-      k_colsum<<<4 * N, 1024, 0, s>>>(part, blocks, 4 * N, tot);
-      k_means_finish<N, false><<<1, 32, 0, s>>>(tot, c, nullptr, eps, lam);
+      launch(k_means_partial_df<N, false>, blocks, kBlock, 0, s, u, mom, g, part);
+      launch(k_colsum, 4 * N, 1024, 0, s, part, blocks, 4 * N, tot);
+      launch(k_means_finish<N, false>, 1, 32, 0, s, tot, c, nullptr, eps, lam);
     }
     return 3;
   }
   static int rhs_df(const double *u, const double *mom, const double *c, const Geo &g, double a1, double tl,
                     float *b, cudaStream_t s) {
-    k_rhs_df<N><<<row_grid(g.W + 1, g.H + 1), kBlock, 0, s>>>(u, mom, c, g, a1, tl, b);
+    launch(k_rhs_df<N>, row_grid(g.W + 1, g.H + 1), kBlock, 0, s, u, mom, c, g, a1, tl, b);
     return 1;
   }
   static int outer_resid(const double *u, const float *b, const Geo &g, float *r32, float *u32, double *rho,
@@ -310,44 +310,44 @@ struct Launch {
       static const cudaError_t attr = cudaFuncSetAttribute(
           k_outer_resid_df<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)outer_resid_smem<N>());
       (void)attr;
-      k_outer_resid_df<N><<<dim3((g.W + 1 + kOrThreads - 3) / (kOrThreads - 2), (g.H + kOrRows) / kOrRows),
-                            kOrThreads, outer_resid_smem<N>(), s>>>(u, b, g, r32, u32, rho);
+      launch(k_outer_resid_df<N>, dim3((g.W + 1 + kOrThreads - 3) / (kOrThreads - 2), (g.H + kOrRows) / kOrRows),
+                            kOrThreads, outer_resid_smem<N>(), s, u, b, g, r32, u32, rho);
     }
     else
-      k_outer_resid<N><<<row_grid(g.W + 1, g.H + 1), kBlock, 0, s>>>(u, b, g, r32, u32, rho);
+      launch(k_outer_resid<N>, row_grid(g.W + 1, g.H + 1), kBlock, 0, s, u, b, g, r32, u32, rho);
     return 1;
   }
   static int outer_update(double *u, const float *delta, const Geo &g, cudaStream_t s) {
-    k_outer_update<N><<<row_grid(g.W + 1, g.H + 1), kBlock, 0, s>>>(u, delta, g);
+    launch(k_outer_update<N>, row_grid(g.W + 1, g.H + 1), kBlock, 0, s, u, delta, g);
     return 1;
   }
   static int composite(const double *u, const double *c, const Geo &g, int r, int rounded, float *out,
                        cudaStream_t s) {
-    k_composite<N><<<row_grid(g.W >> r, g.H >> r), kBlock, 0, s>>>(u, c, g, r, rounded, out);
+    launch(k_composite<N>, row_grid(g.W >> r, g.H >> r), kBlock, 0, s, u, c, g, r, rounded, out);
     return 1;
   }
   static int labels(const double *u, const Geo &g, int r, int8_t *node_lab, int8_t *pix_lab, cudaStream_t s) {
     int k = 0;
     if (node_lab) {
-      k_labels<N><<<row_grid(g.W + 1, g.H + 1), kBlock, 0, s>>>(u, g, node_lab);
+      launch(k_labels<N>, row_grid(g.W + 1, g.H + 1), kBlock, 0, s, u, g, node_lab);
       ++k;
     }
     if (pix_lab) {
-      k_pixel_labels<N><<<row_grid(g.W >> r, g.H >> r), kBlock, 0, s>>>(u, g, r, pix_lab);
+      launch(k_pixel_labels<N>, row_grid(g.W >> r, g.H >> r), kBlock, 0, s, u, g, r, pix_lab);
       ++k;
     }
     return k;
   }
   static int to_split32(const double *in, const Geo &g, float *out, cudaStream_t s) {
-    k_to_split32<N><<<row_grid(g.W + 1, g.H + 1), kBlock, 0, s>>>(in, g, out);
+    launch(k_to_split32<N>, row_grid(g.W + 1, g.H + 1), kBlock, 0, s, in, g, out);
     return 1;
   }
   static int from_split32(const float *in, const Geo &g, const double *freeset, double *out, cudaStream_t s) {
-    k_from_split32<N><<<row_grid(g.W + 1, g.H + 1), kBlock, 0, s>>>(in, g, freeset, out);
+    launch(k_from_split32<N>, row_grid(g.W + 1, g.H + 1), kBlock, 0, s, in, g, freeset, out);
     return 1;
   }
   static int adj_prepare(const double *up, const double *g, int64_t n, double *freeset, double *rhs, cudaStream_t s) {
-    k_adj_prepare<N><<<blocks_for(n), kBlock, 0, s>>>(up, g, n, freeset, rhs);
+    launch(k_adj_prepare<N>, blocks_for(n), kBlock, 0, s, up, g, n, freeset, rhs);
     return 1;
   }
   static int adj_accum(const double *w, const double *u, const double *up, const double *mom, const double *c,
@@ -355,46 +355,46 @@ struct Launch {
                        double *scal, cudaStream_t s) {
     const dim3 grid = row_grid(g.W + 1, g.H + 1);
     const int blocks = (int)(grid.x * grid.y);
-    k_adj_accum<N><<<grid, kBlock, 0, s>>>(w, u, up, mom, c, g, tau, eps, lam, gm, part);
-    k_colsum<<<2 + 3 * N, 1024, 0, s>>>(part, blocks, 2 + 3 * N, tot);
-    k_adj_scalars<<<1, 32, 0, s>>>(tot, scal);
+    launch(k_adj_accum<N>, grid, kBlock, 0, s, w, u, up, mom, c, g, tau, eps, lam, gm, part);
+    launch(k_colsum, 2 + 3 * N, 1024, 0, s, part, blocks, 2 + 3 * N, tot);
+    launch(k_adj_scalars, 1, 32, 0, s, tot, scal);
     return 3;
   }
   static int adj_back(const double *w, const double *u, const double *mom, const double *c, const double *tot,
                       const double *mass, const Geo &g, double a1, double *gout, double *gm, cudaStream_t s) {
-    k_adj_back<N><<<row_grid(g.W + 1, g.H + 1), kBlock, 0, s>>>(w, u, mom, c, tot, mass, g, a1, gout, gm);
+    launch(k_adj_back<N>, row_grid(g.W + 1, g.H + 1), kBlock, 0, s, w, u, mom, c, tot, mass, g, a1, gout, gm);
     return 1;
   }
   static int adj_image(const double *gm, const double *img, const Geo &g, double *gimg, cudaStream_t s) {
-    k_adj_image<<<row_grid(g.W, g.H), kBlock, 0, s>>>(gm, img, g, gimg);
+    launch(k_adj_image, row_grid(g.W, g.H), kBlock, 0, s, gm, img, g, gimg);
     return 1;
   }
   static int tangent_apply(const double *p, const double *f, const Geo &g, double *q, cudaStream_t s) {
-    k_tangent_apply<N><<<row_grid(g.W + 1, g.H + 1), kBlock, 0, s>>>(p, f, g, q);
+    launch(k_tangent_apply<N>, row_grid(g.W + 1, g.H + 1), kBlock, 0, s, p, f, g, q);
     return 1;
   }
   static int dot2(const double *a0, const double *b0, const double *a1, const double *b1, int64_t count,
                   double *part, double *tot, cudaStream_t s) {
-    k_dot2<<<kMaxPartBlocks, kBlock, 0, s>>>(a0, b0, a1, b1, count, part);
-    k_colsum<<<2, 1024, 0, s>>>(part, kMaxPartBlocks, 2, tot);
+    launch(k_dot2, kMaxPartBlocks, kBlock, 0, s, a0, b0, a1, b1, count, part);
+    launch(k_colsum, 2, 1024, 0, s, part, kMaxPartBlocks, 2, tot);
     return 2;
   }
   static int fcg_step(double *x, double *r, const double *p, const double *q, double alpha, int64_t count,
                       cudaStream_t s) {
-    k_fcg_step<<<blocks_for(count), kBlock, 0, s>>>(x, r, p, q, alpha, count);
+    launch(k_fcg_step, blocks_for(count), kBlock, 0, s, x, r, p, q, alpha, count);
     return 1;
   }
   static int fcg_dir(double *p, const double *z, double beta, int64_t count, cudaStream_t s) {
-    k_fcg_dir<<<blocks_for(count), kBlock, 0, s>>>(p, z, beta, count);
+    launch(k_fcg_dir, blocks_for(count), kBlock, 0, s, p, z, beta, count);
     return 1;
   }
   static int absmax(const double *v, int64_t count, double *out, cudaStream_t s) {
-    k_absmax<<<kMaxPartBlocks, kBlock, 0, s>>>(v, count, out);
+    launch(k_absmax, kMaxPartBlocks, kBlock, 0, s, v, count, out);
     return 1;
   }
   static int project(const double *y, double *x, int64_t count, cudaStream_t s) {
     if (count <= 0) return 0;
-    k_project<N><<<blocks_for(count), kBlock, 0, s>>>(y, x, count);
+    launch(k_project<N>, blocks_for(count), kBlock, 0, s, y, x, count);
     return 1;
   }
   static const Ops *table() {
