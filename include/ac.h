@@ -129,7 +129,8 @@ enum {
 typedef struct {
   double ms[AC_PROF_COUNT];        /* summed device time per class (CUDA events on the context's stream) */
   int64_t launches[AC_PROF_COUNT]; /* kernel launches per class while profiling was on */
-  double smooth_bytes_per_launch;  /* algorithmic HBM bytes of one smoother launch (one colour): AC_FP64
+  double smooth_bytes_per_launch;  /* algorithmic HBM bytes of one smoother launch (one colour), on average where
+                                      cycles visited part of the nodes: AC_FP64
                                       1.5 n N 8 (b of the colour, u of the other colour read, u of the
                                       colour written), AC_MIXED 2 n N 4 (r and obstacle of the colour,
                                       delta of the other colour read, delta of the colour written) */
@@ -140,7 +141,8 @@ typedef struct {
                                       0.5 n N 4 (AC_MIXED) */
   double bytes[AC_PROF_COUNT];     /* algorithmic HBM bytes of the class's launches while profiling was on:
                                       every array element a launch is defined on read once and written once
-                                      (dense counts: rows the coarse kernels skip are still counted) */
+                                      (dense counts: rows the coarse kernels skip are still counted; fine
+                                      tiles that a cycle does not visit are not) */
 } ac_profile;
 
 /* Defaults: tol 1e-10, nu1 = nu2 = 2, max_cycles 200, coarse_min 4, AC_FP64,
@@ -230,13 +232,17 @@ int ac_project_simplex(const double *y, double *x, int64_t count, int n_phases, 
  * nonzero row (live) and lists them, and the level's other kernels work on
  * the listed tiles only (tiles that stay dead hold exact zeros and are not
  * visited).  Both forms compute the same numbers; the tiled one pays when
- * few tiles are live, i.e. once the phases have separated.
+ * few tiles are live, i.e. once the phases have separated.  The fine level
+ * has the same choice, in 8 x 8-node tiles: all, or those that can change in
+ * the cycle (with a free node, changed by the last pass, or beside such one).
  *   AC_TILES_AUTO (default): tiled for levels with at least 32 (tile, phase)
  *     pairs per multiprocessor, chosen per V-cycle when fewer than a quarter
- *     of the fine nodes have a free phase;
+ *     of the fine nodes have a free phase; the fine level in the host loop
+ *     below a fifth, from 1 M unknowns on (0.25 M in AC_FP64);
  *   AC_TILES_NEVER: dense always;
  *   AC_TILES_ALWAYS: tiled on every coarse level above the coarsest and the
- *     one-launch tail, whatever its size (a check of the tiled kernels). */
+ *     one-launch tail and on the fine level, whatever its size (a check of the
+ *     tiled kernels). */
 enum { AC_TILES_AUTO = 0, AC_TILES_NEVER = 1, AC_TILES_ALWAYS = 2 };
 int ac_set_coarse_tiling(ac_ctx *ctx, int mode);
 
@@ -277,8 +283,11 @@ int ac_set_coarse_smoother(ac_ctx *ctx, int mode);
  *     is off (a profiled cycle brackets its kernels with events, which a
  *     conditional body cannot hold), and no coarse level can run tiled
  *     (ac_set_coarse_tiling; with AC_TILES_AUTO that is every image whose
- *     coarse levels are too small for tiles, e.g. 1024^2 and below at N <= 8)
- *     -- and on the host otherwise;
+ *     coarse levels are too small for tiles, e.g. 1024^2 and below at N <= 8),
+ *     and on the host otherwise, as it is for an image of at least 3 M
+ *     unknowns (0.5 M in AC_FP64) whose last cycle found few free nodes: the
+ *     host loop then visits only the fine tiles that can change
+ *     (ac_set_coarse_tiling);
  *   AC_LOOP_HOST: always on the host.
  * If the graph cannot be captured or instantiated (a driver without
  * conditional nodes), the context switches itself to AC_LOOP_HOST and the

@@ -174,6 +174,12 @@ struct StepGraph {
   int64_t fixed = 0, per_pass = 0, per_cycle = 0;
 };
 
+// Smoothing and residual of a cycle: the first one of a solve (nu1 sweeps) or
+// a later one (nu1 + nu2, a correction pending), by the plain kernels or on
+// the tiles that have work, with the tiles' record kept so far or started
+// anew (the first cycle always starts it: rhs and bounds are new).
+enum SmoothVariant { kFirst, kLater, kFirstSettled, kLaterSettledAll, kLaterSettled, kSmoothVariants };
+
 // One multigrid solve: min_x sum_i 1/2 x_i'S x_i - rhs_i'x_i over the
 // constraint set of the instantiation (see ac_kernels.cuh).
 struct Solve {
@@ -184,10 +190,15 @@ struct Solve {
   std::vector<Level> lv;  // lv[0]: fine level geometry
   int depth = 0;          // levels in use (<= lv.size()); a schedule can cut the hierarchy short
   ac::Galerkin0Table tab0{};
-  // graphs [profiling][variant]: smoothing + residual of the first / a later
-  // cycle, and the coarse correction with its line search [profiling][form:
-  // dense levels / tiled levels with live flags and work lists]
-  GraphSlot smooth_resid[2][2], correction[2][2];
+  // the settled fine tiles' record (changed null: none, the adjoint's solves);
+  // whether the last cycle kept it, and the free fraction it found
+  ac::SettledTiles settled{};
+  bool record = false;
+  double free_frac = 1.0;
+  // graphs [profiling][variant]: smoothing + residual (SmoothVariant), and
+  // the coarse correction with its line search [profiling][form: dense levels
+  // / tiled levels with live flags and work lists]
+  GraphSlot smooth_resid[2][kSmoothVariants], correction[2][2];
   // the form of the next coarse correction: tiled while few fine nodes are
   // free (its kernels then skip the dead tiles), dense otherwise (when most
   // tiles are live the work lists cost more than they skip); was_tiled: the
@@ -201,6 +212,22 @@ struct Solve {
 // nodes have a free phase (about 45% of the first level's tiles are then
 // live at 4096^2, N = 8, where both forms take the same time).
 constexpr double kTiledFreeFraction = 0.25;
+
+// A cycle smooths only the tiles that can change when fewer than this
+// fraction of the fine nodes had a free phase in the last one (4096^2, N = 8
+// over its first 48 steps: 0.15, 0.2 and 0.25 take 25.6, 22.4 and 22.4 ms in
+// steps 17-20, 0.25 30.4 against 29.6 in steps 9-12), on grids of at least so
+// many unknowns -- below, a cycle is bound by its launches, and the list is
+// one more (host loop, formed phases, mixed: 384^2 N = 4 1.06 against 0.99 ms,
+// 512^2 1.15 and 1.16, 768^2 1.37 against 1.50; FP64 256^2 N = 4 1.50 against
+// 1.56).
+constexpr double kSettledFreeFraction = 0.2;
+int64_t settled_min_unknowns(int elem) { return elem == 4 ? 1 << 20 : 1 << 18; }
+// From so many unknowns on it pays to run the cycle loop on the host for it
+// (device loop without, host loop with: mixed N = 4 768^2 1.35 / 1.37 ms,
+// 1024^2 1.86 / 1.64; FP64 N = 4 256^2 1.46 / 1.50, 384^2 1.76 / 1.69, 1024^2
+// 5.51 / 3.36).
+int64_t settled_host_unknowns(int elem) { return elem == 4 ? 3 << 20 : 1 << 19; }
 
 // Pre/post l1-Jacobi sweeps on coarse levels (even); a build option
 // (-DAC_COARSE_SWEEPS=k) for tuning.
@@ -311,6 +338,8 @@ struct ac_ctx {
   int64_t prof_launches[AC_PROF_COUNT] = {};
   double prof_bytes[AC_PROF_COUNT] = {};
   int64_t prof_corr_launches = 0;  // smoother launches that applied a pending correction
+  double settled_bytes[AC_PROF_COUNT] = {};  // bytes of a later cycle's smoothing and residual over all nodes
+  bool prof_settled = false;                 // the profile holds cycles that did not visit all nodes
   // CUDA graphs (off on the legacy default stream, which cannot be captured)
   bool use_graphs = false;
   GraphSlot *capturing = nullptr;
@@ -535,7 +564,8 @@ int run_graph(ac_ctx *ctx, GraphSlot &slot, F &&enqueue) {
 // nullable).  While profiling, the finished event pairs are summed here: the
 // graphs re-record their events on every replay.
 int read_rho(ac_ctx *ctx, double *out, int64_t *nfree = nullptr) {
-  AC_CUDA(cudaMemcpyAsync(ctx->h_scalars, ctx->rho, 2 * sizeof(double), cudaMemcpyDeviceToHost, ctx->s));
+  AC_CUDA(cudaMemcpyAsync(ctx->h_scalars, ctx->rho, 2 * sizeof(double) + sizeof(ac::SettledCtl),
+                          cudaMemcpyDeviceToHost, ctx->s));
   AC_CUDA(cudaStreamSynchronize(ctx->s));
   *out = ctx->h_scalars[0];
   if (nfree) {
@@ -666,7 +696,9 @@ int coarse_vcycle(ac_ctx *ctx, Solve &S, int k, void **res) {
 // false), nu2 + nu1 and the pending coarse correction in a later one; then
 // r = rhs - S x, rho and the free-node count (zeroed first), the mask and
 // the tangent residual.
-int enqueue_smooth_resid(ac_ctx *ctx, Solve &S, bool later) {
+int enqueue_smooth_resid(ac_ctx *ctx, Solve &S, SmoothVariant variant) {
+  const bool later = variant != kFirst && variant != kFirstSettled;
+  const bool settled = variant >= kFirstSettled, all = settled && variant != kLaterSettled;
   const ac::SolverOps *o = S.o;
   const ac::Geo &g0 = S.lv[0].g;
   const ByteModel bm = byte_model(ctx, S);
@@ -687,6 +719,17 @@ int enqueue_smooth_resid(ac_ctx *ctx, Solve &S, bool later) {
   const ac::MaskDirty dirty = S.lv.size() > 1
                                   ? ac::MaskDirty{S.lv[1].lists.dirty, ac::tiles_x(S.lv[1].g), ac::tiles_y(S.lv[1].g)}
                                   : ac::MaskDirty{nullptr, 0, 0};
+  if (settled) {
+    if (variant == kLaterSettled) {
+      ctx->settled_bytes[AC_PROF_SMOOTH] = sm_bytes;
+      ctx->settled_bytes[AC_PROF_RESID] = 0.5 * bm.n * (bm.ns * (4 + bm.ob) + 1);
+    }
+    AC_RUNB(AC_PROF_SMOOTH, sm_bytes, o->smooth_settled(S.x, S.rhs, S.ob, corr, ctx->omega, g0, nsw, rt_zero, S.mask,
+                                                        dirty, ctx->rho, S.settled, all, ctx->s));
+    AC_RUNB(AC_PROF_RESID, 0.5 * bm.n * (bm.ns * (4 + bm.ob) + 1),
+            o->resid_settled(S.x, S.rhs, S.ob, g0, S.rt, S.mask, ctx->rho, dirty, S.settled, all, ctx->s));
+    return AC_OK;
+  }
   AC_RUNB(AC_PROF_SMOOTH, sm_bytes, o->smooth(S.x, S.rhs, S.ob, corr, ctx->omega, g0, nsw, rt_zero,
                                               fused ? S.mask : nullptr, dirty, ctx->rho, ctx->s));
   // rho and the free-node count (a masked smoothing sequence has cleared them)
@@ -736,6 +779,13 @@ int enqueue_correction(ac_ctx *ctx, Solve &S) {
   return AC_OK;
 }
 
+// Whether the next cycle smooths only the tiles that can change.
+bool settled_form(const ac_ctx *ctx, const Solve &S, int64_t min_unknowns) {
+  // a cycle's passes must not reach past a tile (k_smooth_settled)
+  if (!S.settled.changed || 2 * (ctx->p.nu1 + ctx->p.nu2) > ac::kSetT || S.tiling == AC_TILES_NEVER) return false;
+  return S.tiling == AC_TILES_ALWAYS || (S.lv[0].n * ctx->N >= min_unknowns && S.free_frac < kSettledFreeFraction);
+}
+
 // Multigrid solve of one step problem.  Cycle structure:
 //   smooth (nu1 red-black projected sweeps; nu2 + nu1 after a correction)
 //   -> residual r = rhs - S x, natural residual rho, free-phase mask, tangent
@@ -756,7 +806,13 @@ int solve_mg(ac_ctx *ctx, Solve &S, double tol, int max_cycles, int *cycles_out,
   for (;;) {
     const int later = cyc > 0 ? 1 : 0;  // nu1 + nu2 sweeps, and the pending coarse correction if any
     const int nsw = later ? ctx->p.nu1 + ctx->p.nu2 : ctx->p.nu1;
-    int rc = run_graph(ctx, S.smooth_resid[prof][later], [&]() { return enqueue_smooth_resid(ctx, S, later); });
+    // only the tiles that can change while few nodes are free
+    const bool settled = nsw >= 1 && settled_form(ctx, S, settled_min_unknowns(S.o->elem));
+    const SmoothVariant variant = !settled ? (later ? kLater : kFirst)
+                                  : !later ? kFirstSettled
+                                           : (S.record ? kLaterSettled : kLaterSettledAll);
+    S.record = settled;
+    int rc = run_graph(ctx, S.smooth_resid[prof][variant], [&]() { return enqueue_smooth_resid(ctx, S, variant); });
     if (rc) return rc;
     if (ctx->profiling && later && coarse && nsw > 0) ++ctx->prof_corr_launches;
     sweeps += nsw;
@@ -764,28 +820,43 @@ int solve_mg(ac_ctx *ctx, Solve &S, double tol, int max_cycles, int *cycles_out,
     int64_t nfree = 0;
     rc = read_rho(ctx, &rho, &nfree);
     if (rc) return rc;
+    // the part of the tiles that the cycle visited
+    double listed = 1.0;
+    if (variant == kLaterSettled) {
+      ac::SettledCtl sc;
+      std::memcpy(&sc, ctx->h_scalars + 2, sizeof sc);
+      listed = (double)sc.count / ((double)S.settled.tx * S.settled.ty);
+      if (ctx->profiling) {
+        // the graph books every node: take the nodes not visited off again
+        for (int cls : {(int)AC_PROF_SMOOTH, (int)AC_PROF_RESID})
+          ctx->prof_bytes[cls] -= (1.0 - listed) * ctx->settled_bytes[cls];
+        ctx->prof_settled = true;
+      }
+    }
 #ifdef AC_TRACE_CYCLES
     {  // build option: one line per cycle (rho, the omega the cycle applied, free nodes, form)
       double om[2] = {0, 0};
       cudaMemcpy(om, ctx->omega, sizeof om, cudaMemcpyDeviceToHost);
-      std::fprintf(stderr, "cycle %d rho %.3e omega %.4f free %lld tiled %d elem %d\n", cyc, rho, later ? om[0] : 0.0,
-                   (long long)nfree, S.tiled ? 1 : 0, S.o->elem);
+      std::fprintf(stderr, "cycle %d rho %.3e omega %.4f free %lld tiled %d elem %d settled %d list %.4f\n",
+                   cyc, rho, later ? om[0] : 0.0, (long long)nfree, S.tiled ? 1 : 0, S.o->elem, (int)variant,
+                   listed);
     }
 #endif
     if (std::isnan(rho) || std::isinf(rho)) {
       status = fail(AC_ERR_NUMERIC, "non-finite residual");
       break;
     }
+    // free nodes: only one colour is counted after a smoothing sequence, about
+    // half of them
+    S.free_frac = (double)nfree * (nsw >= 1 ? 2.0 : 1.0) / (double)S.lv[0].n;
     if (rho <= tol) {
       status = AC_OK;
       break;
     }
     if (cyc >= max_cycles) break;
     if (!coarse) continue;
-    // the coarse correction's form from the free nodes (only one colour is
-    // counted after a smoothing sequence: about half of them)
-    const double free_frac = (double)nfree * (nsw >= 1 ? 2.0 : 1.0) / (double)S.lv[0].n;
-    S.tiled = tiled_end(S) > 1 && (S.tiling == AC_TILES_ALWAYS || free_frac < kTiledFreeFraction);
+    // the coarse correction's form from the free nodes
+    S.tiled = tiled_end(S) > 1 && (S.tiling == AC_TILES_ALWAYS || S.free_frac < kTiledFreeFraction);
     if (S.tiled && !S.was_tiled) {
       // the flags are stale: let this correction compute and write every
       // tile (kLiveNow), whatever the mask changes since the last one
@@ -1056,7 +1127,8 @@ void release_step_graphs(ac_ctx *ctx) {
 
 // Whether ac_step runs the device-side loop (see above).
 bool loop_on_device(const ac_ctx *ctx) {
-  return ctx->loop_mode == AC_LOOP_AUTO && ctx->use_graphs && !ctx->profiling && tiled_end(ctx->sv) <= 1;
+  return ctx->loop_mode == AC_LOOP_AUTO && ctx->use_graphs && !ctx->profiling && tiled_end(ctx->sv) <= 1 &&
+         !settled_form(ctx, ctx->sv, settled_host_unknowns(ctx->sv.o->elem));
 }
 
 // Enqueue one time step with the device-side loop on ctx->s, which is
@@ -1106,7 +1178,7 @@ int enqueue_step_loop(ac_ctx *ctx, cudaGraph_t top, bool energy, StepGraph &sg) 
   }
   // one multigrid solve; its cycles' body is captured on body_s[d]
   auto solve = [&](int d) -> int {
-    int rc = enqueue_smooth_resid(ctx, S, false);
+    int rc = enqueue_smooth_resid(ctx, S, kFirst);
     if (rc) return rc;
     AC_RUN(AC_PROF_RESID, (ac::launch(k_ctl_cycle, 1, 1, 0, ctx->s, ctx->ctl, ctx->rho, ctx->p.nu1, h_cyc), 1));
     rc = begin_while(ctx->s, h_cyc, ctx->body_s[d]);
@@ -1116,7 +1188,7 @@ int enqueue_step_loop(ac_ctx *ctx, cudaGraph_t top, bool energy, StepGraph &sg) 
     ctx->s = ctx->body_s[d];
     ctx->capturing = &cnt_cycle;
     if (coarse) rc = enqueue_correction(ctx, S);
-    if (!rc) rc = enqueue_smooth_resid(ctx, S, true);
+    if (!rc) rc = enqueue_smooth_resid(ctx, S, kLater);
     if (rc) return rc;
     AC_RUN(AC_PROF_RESID,
            (ac::launch(k_ctl_cycle, 1, 1, 0, ctx->s, ctx->ctl, ctx->rho, ctx->p.nu1 + ctx->p.nu2, h_cyc), 1));
@@ -1236,7 +1308,14 @@ int step_device(ac_ctx *ctx, int n_steps, ac_stats *out) {
     AC_CUDA(cudaGraphLaunch(ctx->step_graph[(out && t == n_steps - 1) ? 1 : 0].exec, ctx->s));
   AC_CUDA(cudaMemcpyAsync(ctx->h_ctl, ctx->ctl, sizeof(LoopCtl), cudaMemcpyDeviceToHost, ctx->s));
   if (out) AC_CUDA(cudaMemcpyAsync(ctx->h_scalars + 1, ctx->energy, sizeof(double), cudaMemcpyDeviceToHost, ctx->s));
+  AC_CUDA(cudaMemcpyAsync(ctx->h_scalars + 2, ctx->rho + 1, sizeof(double), cudaMemcpyDeviceToHost, ctx->s));
   AC_CUDA(cudaStreamSynchronize(ctx->s));
+  {
+    // the free nodes of the last cycle (one colour) choose the next call's loop
+    unsigned long long c = 0;
+    std::memcpy(&c, ctx->h_scalars + 2, sizeof c);
+    if (ctx->p.nu1 + ctx->p.nu2 > 0) ctx->sv.free_frac = 2.0 * (double)c / (double)ctx->sv.lv[0].n;
+  }
   ac_stats st{};
   int rc = loop_stats(ctx, ctx->step_graph[0], n_steps, &st);
   if (out) {
@@ -1538,12 +1617,32 @@ int ac_create(ac_ctx **out, const ac_params *p) {
     AC_ALLOC(S.mask, (size_t)ctx->n);
     AC_CUDA(cudaMemsetAsync(S.mask, 0, (size_t)ctx->n, ctx->s));  // read as a hint before the first cycle sets it
     if (S.lv.size() > 1) AC_ALLOC(S.d, fNs);
+    {
+      // the settled tiles' record, one allocation: rho (8 bytes a tile for
+      // either scalar), list, then the byte arrays
+      ac::SettledTiles &st = S.settled;
+      st.tx = ctx->g0.W / ac::kSetT + 1;
+      st.ty = ctx->g0.H / ac::kSetT + 1;
+      st.sms = ctx->sms;
+      const size_t nt = (size_t)st.tx * st.ty;
+      uint8_t *mem = nullptr;
+      AC_ALLOC(mem, 17 * nt + 4);
+      st.rho = mem;
+      st.list = reinterpret_cast<unsigned *>(mem + 8 * nt);
+      st.listed = mem + 12 * nt;
+      st.changed = st.listed + (nt + 3) / 4 * 4;
+      st.free = st.changed + nt;
+      st.nfree = st.free + 2 * nt;
+    }
     AC_ALLOC(ctx->part, (size_t)ac::kMaxPartBlocks * 7 * N * sizeof(double));
     AC_ALLOC(ctx->tot, (size_t)7 * N * sizeof(double));
     AC_ALLOC(ctx->c, (size_t)3 * N * sizeof(double));
     AC_ALLOC(ctx->c_tmp, (size_t)3 * N * sizeof(double));
     AC_ALLOC(ctx->energy, sizeof(double));
-    AC_ALLOC(ctx->rho, 2 * sizeof(double));  // rho and the free-node count of the fine residual
+    // rho, the free-node count of the fine residual, and the settled tiles'
+    // list counters (read back together)
+    AC_ALLOC(ctx->rho, 2 * sizeof(double) + sizeof(ac::SettledCtl));
+    S.settled.ctl = reinterpret_cast<ac::SettledCtl *>(ctx->rho + 2);
     AC_ALLOC(ctx->omega, 2 * sizeof(double));  // omega and its float rounding
     AC_ALLOC(ctx->ls_part, (size_t)2 * ls_blocks * sizeof(double));
     AC_ALLOC(ctx->ls_done, sizeof(unsigned));
@@ -1592,7 +1691,7 @@ void ac_destroy(ac_ctx *ctx) {
     cudaDeviceSynchronize();
   for (Solve *S : {&ctx->sv, &ctx->adj.sv, &ctx->adj.sv32})
     for (int a = 0; a < 2; ++a) {
-      for (int b = 0; b < 2; ++b) slot_release(S->smooth_resid[a][b]);
+      for (int b = 0; b < kSmoothVariants; ++b) slot_release(S->smooth_resid[a][b]);
       for (int f = 0; f < 2; ++f) slot_release(S->correction[a][f]);
     }
   release_step_graphs(ctx);
@@ -1943,6 +2042,7 @@ int ac_set_profiling_mask(ac_ctx *ctx, unsigned class_mask) {
     ctx->prof_bytes[k] = 0;
   }
   ctx->prof_corr_launches = 0;
+  ctx->prof_settled = false;
   class_mask &= (1u << AC_PROF_COUNT) - 1u;
   ctx->profiling = class_mask != 0;
   ctx->prof_mask = class_mask ? class_mask : (1u << AC_PROF_COUNT) - 1u;
@@ -1950,7 +2050,7 @@ int ac_set_profiling_mask(ac_ctx *ctx, unsigned class_mask) {
     // the profiled graphs carry the events of the old mask: capture them again
     if (ctx->s) cudaStreamSynchronize(ctx->s);
     for (Solve *S : {&ctx->sv, &ctx->adj.sv, &ctx->adj.sv32}) {
-      for (int b = 0; b < 2; ++b) slot_release(S->smooth_resid[1][b]);
+      for (int b = 0; b < kSmoothVariants; ++b) slot_release(S->smooth_resid[1][b]);
       for (int f = 0; f < 2; ++f) slot_release(S->correction[1][f]);
     }
     ctx->prof_graph_mask = ctx->prof_mask;
@@ -2025,10 +2125,13 @@ int ac_get_profile(ac_ctx *ctx, ac_profile *out) {
   }
   out->smooth_bytes_per_launch = ctx->p.precision == AC_MIXED ? 2.0 * (double)ctx->n * ctx->N * sizeof(float)
                                                                : 1.5 * (double)ctx->n * ctx->N * sizeof(double);
+  const double corr_extra = 0.5 * (double)ctx->n * ctx->N * (ctx->p.precision == AC_MIXED ? sizeof(float) : sizeof(double));
+  if (ctx->prof_settled && ctx->prof_launches[AC_PROF_SMOOTH] > 0)
+    out->smooth_bytes_per_launch = (ctx->prof_bytes[AC_PROF_SMOOTH] - corr_extra * (double)ctx->prof_corr_launches) /
+                                   (double)ctx->prof_launches[AC_PROF_SMOOTH];
   out->total_launches = ctx->total_launches;
   out->smooth_corr_launches = ctx->prof_corr_launches;
-  out->smooth_corr_extra_bytes = 0.5 * (double)ctx->n * ctx->N * (ctx->p.precision == AC_MIXED ? sizeof(float)
-                                                                                                 : sizeof(double));
+  out->smooth_corr_extra_bytes = corr_extra;
   return AC_OK;
 }
 
@@ -2065,7 +2168,7 @@ void adj_release(ac_ctx *ctx) {
   AdjState &A = ctx->adj;
   for (Solve *S : {&A.sv, &A.sv32})
     for (int a = 0; a < 2; ++a) {
-      for (int b = 0; b < 2; ++b) slot_release(S->smooth_resid[a][b]);
+      for (int b = 0; b < kSmoothVariants; ++b) slot_release(S->smooth_resid[a][b]);
       for (int f = 0; f < 2; ++f) slot_release(S->correction[a][f]);
     }
   for (void *p : A.allocs) cudaFree(p);
@@ -2418,7 +2521,7 @@ namespace {
 void set_schedule(ac_ctx *ctx, int nu1, int nu2, int depth, bool gs) {
   release_step_graphs(ctx);
   for (int a = 0; a < 2; ++a) {
-    for (int b = 0; b < 2; ++b) slot_release(ctx->sv.smooth_resid[a][b]);
+    for (int b = 0; b < kSmoothVariants; ++b) slot_release(ctx->sv.smooth_resid[a][b]);
     for (int f = 0; f < 2; ++f) slot_release(ctx->sv.correction[a][f]);
   }
   ctx->p.nu1 = nu1;

@@ -79,6 +79,23 @@ __device__ __forceinline__ void mark_dirty(const MaskDirty &d, int x, int y) {
     for (int tx = x0; tx <= x1; ++tx) d.p[(int64_t)ty * d.tx + tx] = 1;
 }
 
+// The record of the settled tiles (see k_smooth_settled), per kSetT x
+// kSetT-node tile of the fine grid: whether the last pass of the last cycle
+// changed it, whether a node of a colour is free (free[colour][tile]), its
+// share of rho (in the solve's scalar type) and of the free nodes of the first
+// colour; and the tiles of the cycle in progress.
+constexpr int kSetT = 8;
+struct SettledCtl {
+  unsigned count, joined;  // tiles in the list, and at its far end
+};
+struct SettledTiles {
+  uint8_t *changed, *free, *nfree, *listed;  // listed: 4-byte aligned
+  void *rho;
+  unsigned *list;
+  SettledCtl *ctl;
+  int tx, ty, sms;  // tiles across and down, multiprocessors of the device
+};
+
 // te, S_nn, 1/S_nn in a kernel's scalar type.
 template <typename T>
 __host__ __device__ __forceinline__ T geo_te(const Geo &g) {

@@ -869,28 +869,17 @@ __global__ void k_outer_update(double *__restrict__ u, const float *__restrict__
 // color are independent given the other colour:
 //   z_n = (rhs_n + tau eps sum_m w_nm x_m) / S_nn,   x_n <- P(z_n).
 // ---------------------------------------------------------------------------
-// MASK: the last pass of a smoothing sequence (its own instantiation, so the
-// other passes keep their register budget).
-// With corr != null (first colour of the first sweep after a coarse
-// correction) the neighbours are read as x + omega d: that is exactly the
-// pending update x += omega d, because this pass overwrites its own colour
-// and the next pass overwrites the other one without reading old values.
-template <typename T, int N, int FORM, bool MASK>
-__global__ void __launch_bounds__(kBlock) k_smooth_fine(T *__restrict__ x, const T *__restrict__ rhs,
-                                                        const T *__restrict__ ob, const T *__restrict__ corr,
-                                                        const double *__restrict__ omega, Geo g, int color,
-                                                        T *__restrict__ rt, uint8_t *__restrict__ mask,
-                                                        MaskDirty dirty, double *__restrict__ rho) {
-  pdl_sync();
-  const int y = blockIdx.y;
-  // the residual that follows accumulates into rho and the free-node count
-  if (MASK && rho && blockIdx.x == 0 && y == 0 && threadIdx.x == 0) rho[0] = rho[1] = 0.0;
-  const int xx = 2 * (blockIdx.x * blockDim.x + threadIdx.x) + ((y + color) & 1);
-  if (xx > g.W) return;
-  const int64_t n = fslot<T>(g, xx, y);
-  // the mask byte this pass replaces, loaded first so its latency overlaps
-  const uint8_t old_mask = (MASK && dirty.p) ? mask[(int64_t)y * g.Wn + xx] : (uint8_t)0;
-  T acc[N], bk[N], o[N];
+// The new value acc of node (xx, y) (slot n), and its bounds o.  With corr !=
+// null (first colour of the first sweep after a coarse correction) the
+// neighbours are read as x + omega d: that is exactly the pending update
+// x += omega d, because this pass overwrites its own colour and the next pass
+// overwrites the other one without reading old values.
+template <typename T, int N, int FORM>
+__device__ __forceinline__ void smooth_node(const T *x, const T *__restrict__ rhs, const T *__restrict__ ob,
+                                            const T *__restrict__ corr, const double *__restrict__ omega,
+                                            const Geo &g, int xx, int y, int64_t n, const uint8_t *mask, T (&acc)[N],
+                                            T (&o)[N]) {
+  T bk[N];
   // FP64 direct form: phases the projection drops need no binary64 at all
   bool plain = true;
   if constexpr (kFilter64<T, FORM>) plain = many_free64<N>(mask[(int64_t)y * g.Wn + xx]);
@@ -920,25 +909,52 @@ __global__ void __launch_bounds__(kBlock) k_smooth_fine(T *__restrict__ x, const
 #pragma unroll
     for (int i = 0; i < N; ++i) acc[i] = ((keep >> i) & 1u) ? z[i] - theta : 0.0;
   }
+}
+
+// The free mask of a node value: the phases above their bound (direct,
+// shifted) or in the frozen set (tangent), 0 when fewer than two.
+template <typename T, int N, int FORM>
+__device__ __forceinline__ unsigned free_mask(const T (&x)[N], const T (&o)[N]) {
+  unsigned pos = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i)
+    if (FORM == kTangent ? o[i] != T(0) : x[i] > (FORM == kShifted ? -o[i] : T(0))) pos |= 1u << i;
+  return __popc(pos) >= 2 ? pos : 0u;
+}
+
+// Store a node's mask byte (and mark the first coarse level's tiles over a
+// change); old: the byte it replaces.
+__device__ __forceinline__ void store_mask(uint8_t *mask, const MaskDirty &dirty, const Geo &g, int xx, int y,
+                                           uint8_t old, unsigned fr) {
+  if (dirty.p && old != (uint8_t)fr) mark_dirty(dirty, xx, y);
+  mask[(int64_t)y * g.Wn + xx] = (uint8_t)fr;
+}
+
+// MASK: the last pass of a smoothing sequence (its own instantiation, so the
+// other passes keep their register budget): a node's nodal problem is then
+// solved exactly, so its natural residual is 0 and its residual is constant
+// on the free phases (tangent part 0); it stores the free mask (and rt = 0
+// when rt != null) here, and k_fine_resid visits the other colour only.
+template <typename T, int N, int FORM, bool MASK>
+__global__ void __launch_bounds__(kBlock) k_smooth_fine(T *__restrict__ x, const T *__restrict__ rhs,
+                                                        const T *__restrict__ ob, const T *__restrict__ corr,
+                                                        const double *__restrict__ omega, Geo g, int color,
+                                                        T *__restrict__ rt, uint8_t *__restrict__ mask,
+                                                        MaskDirty dirty, double *__restrict__ rho) {
+  pdl_sync();
+  const int y = blockIdx.y;
+  // the residual that follows accumulates into rho and the free-node count
+  if (MASK && rho && blockIdx.x == 0 && y == 0 && threadIdx.x == 0) rho[0] = rho[1] = 0.0;
+  const int xx = 2 * (blockIdx.x * blockDim.x + threadIdx.x) + ((y + color) & 1);
+  if (xx > g.W) return;
+  const int64_t n = fslot<T>(g, xx, y);
+  // the mask byte this pass replaces, loaded first so its latency overlaps
+  const uint8_t old_mask = (MASK && dirty.p) ? mask[(int64_t)y * g.Wn + xx] : (uint8_t)0;
+  T acc[N], o[N];
+  smooth_node<T, N, FORM>(x, rhs, ob, corr, omega, g, xx, y, n, mask, acc, o);
   stn<T, N>(x + n * N, acc);
   if constexpr (MASK) {
-    // last pass of a smoothing sequence: this node's nodal problem is solved
-    // exactly, so its natural residual is 0 and its residual is constant on
-    // the free phases (tangent part 0); store the free mask (and rt = 0 when
-    // rt != null) here, and k_fine_resid visits the other colour only
-    int cnt = 0;
-    unsigned pos = 0;
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-      const bool fr = FORM == kTangent ? o[i] != T(0) : acc[i] > (FORM == kShifted ? -o[i] : T(0));
-      if (fr) {
-        pos |= 1u << i;
-        ++cnt;
-      }
-    }
-    const uint8_t nm = (uint8_t)(cnt >= 2 ? pos : 0u);
-    if (dirty.p && old_mask != nm) mark_dirty(dirty, xx, y);
-    mask[(int64_t)y * g.Wn + xx] = nm;
+    store_mask(mask, dirty, g, xx, y, old_mask, free_mask<T, N, FORM>(acc, o));
     if (rt) {
       T z[N];
 #pragma unroll
@@ -958,6 +974,67 @@ __global__ void __launch_bounds__(kBlock) k_smooth_fine(T *__restrict__ x, const
 // visited nodes with a free phase is added to the integer that follows *rho
 // (the host picks the coarse correction's form from it).
 // ---------------------------------------------------------------------------
+// One node: its term of rho (NaN where x is) and, with rt, its rt and mask
+// stored and whether it has a free phase (nfree).
+template <typename T, int N, int FORM>
+__device__ __forceinline__ T resid_node(const T *__restrict__ x, const T *__restrict__ rhs, const T *__restrict__ ob,
+                                        const Geo &g, int xx, int y, T *__restrict__ rt, uint8_t *__restrict__ mask,
+                                        const MaskDirty &dirty, int &nfree) {
+  const int64_t n = (int64_t)y * g.Wn + xx, sl = fslot<T>(g, xx, y);
+  // the mask byte this kernel replaces, loaded first so its latency overlaps
+  const uint8_t old_mask = (rt && dirty.p) ? mask[n] : (uint8_t)0;
+  T acc[N], xk[N], bk[N], r[N], o[N];
+  ldn<T, N>(x + sl * N, xk);
+  ldn<T, N>(rhs + sl * N, bk);
+  const int cls = node_class(g, xx, y);
+  const T D = geo_D<T>(g, cls);
+  bool plain = true;
+  if constexpr (kFilter64<T, FORM>) plain = !mask || many_free64<N>(mask[n]);
+  if (plain) {
+    nbr_sum<T, N>(x, g, xx, y, acc);
+    if constexpr (FORM != kDirect) ldn<T, N>(ob + sl * N, o);
+    const T invD = geo_invD<T>(g, cls), te = geo_te<T>(g);
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      r[i] = bk[i] + te * acc[i] - D * xk[i];
+      acc[i] = (bk[i] + te * acc[i]) * invD;
+    }
+    proj_box<T, N, FORM>(acc, o);
+  } else if constexpr (kFilter64<T, FORM>) {
+    // the residual is wanted on the phases above 0, the projection on those
+    // it keeps; elsewhere x and P(z) are both 0
+    unsigned above = 0u, keep;
+#pragma unroll
+    for (int i = 0; i < N; ++i) above |= xk[i] > 0.0 ? 1u << i : 0u;
+    double q[N], z[N], theta;
+    direct_node64<N>(x, nullptr, 0.0, bk, g, xx, y, above, q, z, keep, theta);
+    const unsigned any = __reduce_or_sync(__activemask(), above | keep);
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      r[i] = ((any >> i) & 1u) && ((above >> i) & 1u) ? q[i] - D * xk[i] : 0.0;
+      acc[i] = ((any >> i) & 1u) && ((keep >> i) & 1u) ? z[i] - theta : 0.0;
+    }
+  }
+  T e = T(0);
+#pragma unroll
+  for (int i = 0; i < N; ++i) e = nanmax<T>(e, fabs(xk[i] - acc[i]));
+  if (!(xk[0] == xk[0])) e = xk[0];
+  if (rt) {
+    const unsigned fr = free_mask<T, N, FORM>(xk, o);
+    nfree = fr != 0u;
+    T s = T(0);
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      if ((fr >> i) & 1u) s += r[i];
+    const T mean = fr ? s * rcp_small<T>(__popc(fr)) : T(0);
+#pragma unroll
+    for (int i = 0; i < N; ++i) r[i] = ((fr >> i) & 1u) ? r[i] - mean : T(0);
+    stn<T, N>(rt + sl * N, r);
+    store_mask(mask, dirty, g, xx, y, old_mask, fr);
+  }
+  return e;
+}
+
 template <typename T, int N, int FORM>
 __global__ void __launch_bounds__(kBlock) k_fine_resid(const T *__restrict__ x, const T *__restrict__ rhs,
                                                        const T *__restrict__ ob, Geo g, T *__restrict__ rt,
@@ -971,76 +1048,186 @@ __global__ void __launch_bounds__(kBlock) k_fine_resid(const T *__restrict__ x, 
   const int xx = color < 0 ? t : 2 * t + ((y + color) & 1);
   T e = T(0);
   int nfree = 0;
-  if (xx <= g.W) {
-    const int64_t n = (int64_t)y * g.Wn + xx, sl = fslot<T>(g, xx, y);
-    // the mask byte this kernel replaces, loaded first so its latency overlaps
-    const uint8_t old_mask = (rt && dirty.p) ? mask[n] : (uint8_t)0;
-    T acc[N], xk[N], bk[N], r[N], o[N];
-    ldn<T, N>(x + sl * N, xk);
-    ldn<T, N>(rhs + sl * N, bk);
-    const int cls = node_class(g, xx, y);
-    const T D = geo_D<T>(g, cls);
-    bool plain = true;
-    if constexpr (kFilter64<T, FORM>) plain = !mask || many_free64<N>(mask[n]);
-    if (plain) {
-      nbr_sum<T, N>(x, g, xx, y, acc);
-      if constexpr (FORM != kDirect) ldn<T, N>(ob + sl * N, o);
-      const T invD = geo_invD<T>(g, cls), te = geo_te<T>(g);
-#pragma unroll
-      for (int i = 0; i < N; ++i) {
-        r[i] = bk[i] + te * acc[i] - D * xk[i];
-        acc[i] = (bk[i] + te * acc[i]) * invD;
-      }
-      proj_box<T, N, FORM>(acc, o);
-    } else if constexpr (kFilter64<T, FORM>) {
-      // the residual is wanted on the phases above 0, the projection on those
-      // it keeps; elsewhere x and P(z) are both 0
-      unsigned above = 0u, keep;
-#pragma unroll
-      for (int i = 0; i < N; ++i) above |= xk[i] > 0.0 ? 1u << i : 0u;
-      double q[N], z[N], theta;
-      direct_node64<N>(x, nullptr, 0.0, bk, g, xx, y, above, q, z, keep, theta);
-      const unsigned any = __reduce_or_sync(__activemask(), above | keep);
-#pragma unroll
-      for (int i = 0; i < N; ++i) {
-        r[i] = ((any >> i) & 1u) && ((above >> i) & 1u) ? q[i] - D * xk[i] : 0.0;
-        acc[i] = ((any >> i) & 1u) && ((keep >> i) & 1u) ? z[i] - theta : 0.0;
-      }
-    }
-    int cnt = 0;
-    unsigned pos = 0;
-    T et = T(0);
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-      et = nanmax<T>(et, fabs(xk[i] - acc[i]));
-      // free: above the bound (direct, shifted), or in the frozen set (tangent)
-      const bool fr = FORM == kTangent ? o[i] != T(0) : xk[i] > (FORM == kShifted ? -o[i] : T(0));
-      if (fr) {
-        pos |= 1u << i;
-        ++cnt;
-      }
-    }
-    e = et;
-    if (!(xk[0] == xk[0])) e = xk[0];
-    if (rt) {
-      const unsigned fr = cnt >= 2 ? pos : 0u;
-      nfree = fr != 0u;
-      T s = T(0);
-#pragma unroll
-      for (int i = 0; i < N; ++i)
-        if ((fr >> i) & 1u) s += r[i];
-      const T mean = cnt >= 2 ? s * rcp_small<T>(cnt) : T(0);
-#pragma unroll
-      for (int i = 0; i < N; ++i) r[i] = ((fr >> i) & 1u) ? r[i] - mean : T(0);
-      stn<T, N>(rt + sl * N, r);
-      if (dirty.p && old_mask != (uint8_t)fr) mark_dirty(dirty, xx, y);
-      mask[n] = (uint8_t)fr;
-    }
-  }
+  if (xx <= g.W) e = resid_node<T, N, FORM>(x, rhs, ob, g, xx, y, rt, mask, dirty, nfree);
   if (rt) {
     const int c = __syncthreads_count(nfree);
     if (threadIdx.x == 0 && c) atomicAdd(reinterpret_cast<unsigned long long *>(rho + 1), (unsigned long long)c);
   }
+  block_max_atomic<T>(e, rho);
+}
+
+// ---------------------------------------------------------------------------
+// Settled tiles.  Once the phases have formed, most of the picture is pure:
+// a pass there finds every neighbour as its last pass left it, and would store
+// the value that it finds.  So a cycle visits a list of kSetT x kSetT-node
+// tiles only.  The seeds are the tiles with a free node (a pending coarse
+// correction moves no other node) and those whose second colour changed in
+// the last pass (the first colour has not seen that yet); every other node is
+// what its nodal problem gives for its neighbours.  A change travels one node
+// per pass, so the 2 (nu1 + nu2) <= kSetT passes of a cycle change no node
+// outside the seeds and the tiles around them: those are the list.  Outside
+// it the masks and rt stand as well, and the residual except beside a tile
+// that the last pass changed: such a tile joins the list for the residual.
+// Each tile's share of rho and of the free nodes is kept for the cycles that
+// do not visit it.  The numbers are those of the plain kernels.
+// A visit costs more than the plain kernels' share (a list entry, short
+// rows), so those run while many nodes are free (kSettledFreeFraction).
+// 4096^2, N = 8, formed phases (3.4% of the tiles listed): smoothing 15.3 ->
+// 2.4 ms a step, residual 2.9 -> 0.8; 1024^2, N = 4 FP64 2.30 -> 0.77 and 0.80
+// -> 0.23.
+// ---------------------------------------------------------------------------
+
+// One warp per tile: lane l has row l / 4 and the (l % 4)th node of a colour.
+static_assert(kSetT == 8, "32 nodes of a colour per tile");
+
+// The list of a cycle (st.ctl cleared before the launch) and who is in it.
+static __global__ void __launch_bounds__(kBlock) k_settled_list(SettledTiles st) {
+  pdl_sync();
+  const int nt = st.tx * st.ty, t = (int)(blockIdx.x * kBlock + threadIdx.x);
+  bool visit = false;
+  if (t < nt) {
+    const int x = t % st.tx, y = t / st.tx;
+#pragma unroll
+    for (int dy = -1; dy <= 1; ++dy)
+#pragma unroll
+      for (int dx = -1; dx <= 1; ++dx)
+        if (x + dx >= 0 && x + dx < st.tx && y + dy >= 0 && y + dy < st.ty) {
+          const int q = t + dy * st.tx + dx;
+          visit = visit || st.changed[q] || st.free[q] || st.free[nt + q];
+        }
+    st.listed[t] = visit;
+  }
+  __shared__ unsigned s_base, s_warp[kBlock / 32];
+  const unsigned b = __ballot_sync(0xffffffffu, visit);
+  const int lane = (int)(threadIdx.x & 31u), warp = (int)(threadIdx.x >> 5);
+  if (lane == 0) s_warp[warp] = __popc(b);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned sum = 0;
+    for (int w = 0; w < kBlock / 32; ++w) {
+      const unsigned c = s_warp[w];
+      s_warp[w] = sum;
+      sum += c;
+    }
+    s_base = sum ? atomicAdd(&st.ctl->count, sum) : 0u;
+  }
+  __syncthreads();
+  if (visit) st.list[s_base + s_warp[warp] + __popc(b & ((1u << lane) - 1u))] = (unsigned)t;
+}
+
+// Tile t joins the list for the residual (at its far end), once.
+__device__ __forceinline__ void settled_join(const SettledTiles &st, int t) {
+  if (st.listed[t]) return;
+  const unsigned bit = 1u << (8 * (t & 3));
+  if (atomicOr(reinterpret_cast<unsigned *>(st.listed) + (t >> 2), bit) & bit) return;
+  st.list[st.tx * st.ty - 1 - (int)atomicAdd(&st.ctl->joined, 1u)] = (unsigned)t;
+}
+
+// The tiles of the cycle, one per warp and step: every tile (all: the first
+// cycle of a solve, whose right-hand side and bounds are new) or the list's
+// (JOINED: and those that joined it).
+template <bool JOINED, class F>
+__device__ __forceinline__ void for_listed(const SettledTiles &st, bool all, F &&body) {
+  const int nt = st.tx * st.ty, cnt = all ? nt : (int)st.ctl->count;
+  const int end = JOINED && !all ? cnt + (int)st.ctl->joined : cnt;
+  const int step = (int)gridDim.x * (kBlock / 32);
+  for (int w = (int)(threadIdx.x >> 5) * (int)gridDim.x + (int)blockIdx.x; w < end; w += step) {
+    const int t = all ? w : (int)st.list[w < cnt ? w : nt - 1 - (w - cnt)];
+    body(t, t % st.tx * kSetT, t / st.tx * kSetT);
+  }
+}
+
+// k_smooth_fine on the cycle's tiles; the last pass (MASK) records which
+// tiles it changed and where nodes are free.
+template <typename T, int N, int FORM, bool MASK>
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 4 : 1)
+    k_smooth_settled(T *__restrict__ x, const T *__restrict__ rhs, const T *__restrict__ ob,
+                     const T *__restrict__ corr, const double *__restrict__ omega, Geo g, int color,
+                     T *__restrict__ rt, uint8_t *__restrict__ mask, MaskDirty dirty, double *__restrict__ rho,
+                     SettledTiles st, bool all) {
+  pdl_sync();
+  // the residual that follows accumulates into rho and the free-node count
+  if (MASK && blockIdx.x == 0 && threadIdx.x == 0) rho[0] = rho[1] = 0.0;
+  const int lane = (int)(threadIdx.x & 31u), nt = st.tx * st.ty;
+  for_listed<false>(st, all, [&](int t, int x0, int y0) {
+    const int y = y0 + lane / 4, xx = x0 + 2 * (lane % 4) + ((y + color) & 1);
+    bool changed = false, fr = false;
+    if (y <= g.H && xx <= g.W) {
+      const int64_t n = fslot<T>(g, xx, y);
+      const uint8_t old_mask = (MASK && dirty.p) ? mask[(int64_t)y * g.Wn + xx] : (uint8_t)0;
+      T acc[N], o[N], old[N];
+      if constexpr (MASK) ldn_rw<T, N>(x + n * N, old);
+      smooth_node<T, N, FORM>(x, rhs, ob, corr, omega, g, xx, y, n, mask, acc, o);
+      stn<T, N>(x + n * N, acc);
+      if constexpr (MASK) {
+        // a NaN counts as a change; the sign of a zero does not (no result depends on it)
+#pragma unroll
+        for (int i = 0; i < N; ++i) changed = changed || !(old[i] == acc[i]);
+        const unsigned nm = free_mask<T, N, FORM>(acc, o);
+        fr = nm != 0u;
+        store_mask(mask, dirty, g, xx, y, old_mask, nm);
+        if (rt) {
+          T z[N];
+#pragma unroll
+          for (int i = 0; i < N; ++i) z[i] = T(0);
+          stn<T, N>(rt + n * N, z);
+        }
+      }
+    }
+    if constexpr (MASK) {
+      changed = __any_sync(0xffffffffu, changed);
+      fr = __any_sync(0xffffffffu, fr);
+      if (lane == 0) {
+        st.changed[t] = changed;
+        st.free[color * nt + t] = fr;
+        if (changed && !all) {
+          if (x0 > 0) settled_join(st, t - 1);
+          if (x0 + kSetT <= g.W) settled_join(st, t + 1);
+          if (y0 > 0) settled_join(st, t - st.tx);
+          if (y0 + kSetT <= g.H) settled_join(st, t + st.tx);
+        }
+      }
+    }
+  });
+}
+
+// k_fine_resid (color 0) on the cycle's tiles and those beside a change; the
+// others add the shares that they kept.
+template <typename T, int N, int FORM>
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 4 : 1)
+    k_resid_settled(const T *__restrict__ x, const T *__restrict__ rhs, const T *__restrict__ ob, Geo g,
+                    T *__restrict__ rt, uint8_t *__restrict__ mask, double *__restrict__ rho, MaskDirty dirty,
+                    SettledTiles st, bool all) {
+  pdl_sync();
+  const int lane = (int)(threadIdx.x & 31u);
+  T e = T(0);     // this thread's share of rho
+  int count = 0;  // and of the free nodes
+  if (!all) {
+    const int nt = st.tx * st.ty;
+    for (int t = (int)(blockIdx.x * kBlock + threadIdx.x); t < nt; t += (int)(gridDim.x * kBlock))
+      if (!st.listed[t]) {
+        e = nanmax<T>(e, static_cast<const T *>(st.rho)[t]);
+        count += st.nfree[t];
+      }
+  }
+  for_listed<true>(st, all, [&](int t, int x0, int y0) {
+    const int y = y0 + lane / 4, xx = x0 + 2 * (lane % 4) + (y & 1);
+    T et = T(0);
+    int fr = 0;
+    if (y <= g.H && xx <= g.W) et = resid_node<T, N, FORM>(x, rhs, ob, g, xx, y, rt, mask, dirty, fr);
+    et = warp_nanmax<T>(et);
+    const int c = __popc(__ballot_sync(0xffffffffu, fr != 0));
+    e = nanmax<T>(e, et);
+    if (lane == 0) {
+      count += c;
+      static_cast<T *>(st.rho)[t] = et;
+      st.nfree[t] = (uint8_t)c;
+      st.free[t] = c != 0;
+    }
+  });
+  count = warp_sum<int>(count);
+  if (lane == 0 && count)
+    atomicAdd(reinterpret_cast<unsigned long long *>(rho + 1), (unsigned long long)count);
   block_max_atomic<T>(e, rho);
 }
 

@@ -85,6 +85,42 @@ struct SolverLaunch {
                                                    rho, color, dirty);
     return 1;
   }
+  // the same two on the tiles that have work (see k_smooth_settled): every
+  // block resident at once, its warps striding over the cycle's tiles
+  template <class K>
+  static dim3 settled_grid(const SettledTiles &st, K k) {
+    static const int per_sm = resident_blocks(k, kBlock);
+    constexpr int W = kBlock / 32;
+    return dim3((unsigned)std::min((st.tx * st.ty + W - 1) / W, st.sms * per_sm));
+  }
+  static int smooth_settled(void *x, const void *rhs, const void *ob, const void *corr, const double *omega,
+                            const Geo &g, int sweeps, void *rt, uint8_t *mask, const MaskDirty &dirty, double *rho,
+                            const SettledTiles &st, bool all, cudaStream_t s) {
+    if (!all) {
+      cudaMemsetAsync(st.ctl, 0, sizeof(SettledCtl), s);
+      launch(k_settled_list, dim3(blocks_for((int64_t)st.tx * st.ty)), kBlock, 0, s, st);
+    }
+    for (int p = 0; p < 2 * sweeps; ++p) {
+      const T *cr = p == 0 ? (const T *)corr : nullptr;
+      if (p == 2 * sweeps - 1)
+        launch(k_smooth_settled<T, N, FORM, true>, settled_grid(st, k_smooth_settled<T, N, FORM, true>), kBlock, 0, s,
+               (T *)x, (const T *)rhs, (const T *)ob, cr, omega, g, p & 1, (T *)rt, mask, dirty, rho, st, all);
+      else if (all)
+        launch(k_smooth_fine<T, N, FORM, false>, row_grid((g.W + 2) / 2, g.H + 1), kBlock, 0, s, (T *)x,
+               (const T *)rhs, (const T *)ob, cr, omega, g, p & 1, nullptr, mask, MaskDirty{nullptr, 0, 0}, nullptr);
+      else
+        launch(k_smooth_settled<T, N, FORM, false>, settled_grid(st, k_smooth_settled<T, N, FORM, false>), kBlock, 0,
+               s, (T *)x, (const T *)rhs, (const T *)ob, cr, omega, g, p & 1, nullptr, mask,
+               MaskDirty{nullptr, 0, 0}, nullptr, st, all);
+    }
+    return 2 * sweeps + (all ? 0 : 1);
+  }
+  static int resid_settled(const void *x, const void *rhs, const void *ob, const Geo &g, void *rt, uint8_t *mask,
+                           double *rho, const MaskDirty &dirty, const SettledTiles &st, bool all, cudaStream_t s) {
+    launch(k_resid_settled<T, N, FORM>, settled_grid(st, k_resid_settled<T, N, FORM>), kBlock, 0, s, (const T *)x,
+           (const T *)rhs, (const T *)ob, g, (T *)rt, mask, rho, dirty, st, all);
+    return 1;
+  }
   static int restrict0(const void *rt, const Geo &gf, const Geo &gc, const void *op1, void *r1, const LevelLists *L1,
                        cudaStream_t s) {
     const dim3 grid = L1 ? list_grid(L1, L1->cap / N, k_restrict0<T, N>, kTileThreads)
@@ -242,7 +278,13 @@ struct SolverLaunch {
     return 2;
   }
   static SolverOps table() {
-    return SolverOps{(int)sizeof(T), smooth,       resid,        restrict0,   galerkin0,   galerkin,   coarse_smooth,
+    decltype(SolverOps::smooth_settled) ss = nullptr;  // the adjoint's solves keep no record of their tiles
+    decltype(SolverOps::resid_settled) rs = nullptr;
+    if constexpr (FORM != kTangent) {
+      ss = smooth_settled;
+      rs = resid_settled;
+    }
+    return SolverOps{(int)sizeof(T), smooth,       resid,        ss, rs, restrict0,   galerkin0,   galerkin,   coarse_smooth,
                      coarse_resid, coarse_pre_resid, restrict_, prolong_add, coarse_tail,
                      line_search};
   }

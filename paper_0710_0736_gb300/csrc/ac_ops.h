@@ -10,6 +10,7 @@ namespace ac {
 struct Geo;
 struct Galerkin0Table;
 struct MaskDirty;
+struct SettledTiles;
 
 // Scratch of the block-partial reductions: at most kMaxPartBlocks rows.
 constexpr int kMaxPartBlocks = 1024;
@@ -61,6 +62,13 @@ struct SolverOps {
   // color < 0: every node; 0: the first colour only (completes a masked smooth)
   int (*resid)(const void *x, const void *rhs, const void *ob, const Geo &g, void *rt, uint8_t *mask, double *rho,
                int color, const MaskDirty &dirty, cudaStream_t s);
+  // the same two (smooth with a mask, resid of the first colour) on the tiles
+  // that can change in the cycle, or on all of them to start their record
+  int (*smooth_settled)(void *x, const void *rhs, const void *ob, const void *corr, const double *omega, const Geo &g,
+                        int sweeps, void *rt, uint8_t *mask, const MaskDirty &dirty, double *rho,
+                        const SettledTiles &st, bool all, cudaStream_t s);
+  int (*resid_settled)(const void *x, const void *rhs, const void *ob, const Geo &g, void *rt, uint8_t *mask,
+                       double *rho, const MaskDirty &dirty, const SettledTiles &st, bool all, cudaStream_t s);
   // transfers skip the rows whose diagonal in the (coarse or fine) level's
   // operator is 0: those rows and their residuals are exactly 0.  LevelLists
   // arguments: the live-tile state of a tiled level, or null for a level
