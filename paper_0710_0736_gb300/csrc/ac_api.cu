@@ -175,10 +175,11 @@ struct StepGraph {
 };
 
 // Smoothing and residual of a cycle: the first one of a solve (nu1 sweeps) or
-// a later one (nu1 + nu2, a correction pending), by the plain kernels or on
-// the tiles that have work, with the tiles' record kept so far or started
-// anew (the first cycle always starts it: rhs and bounds are new).
-enum SmoothVariant { kFirst, kLater, kFirstSettled, kLaterSettledAll, kLaterSettled, kSmoothVariants };
+// a later one (nu1 + nu2, a correction pending); by the plain kernels, on all
+// tiles with their record started anew, or on the tiles that can change (in
+// the first cycle of a mixed solve, whose right-hand side and bounds are new,
+// those that the outer residual marked too).
+enum SmoothVariant { kFirst, kLater, kFirstSettledAll, kFirstSettled, kLaterSettledAll, kLaterSettled, kSmoothVariants };
 
 // One multigrid solve: min_x sum_i 1/2 x_i'S x_i - rhs_i'x_i over the
 // constraint set of the instantiation (see ac_kernels.cuh).
@@ -187,6 +188,7 @@ struct Solve {
   int *list_counts = nullptr;  // the tiled levels' list counts, two per level (cleared by one memset per cycle)
   void *x = nullptr, *rhs = nullptr, *ob = nullptr, *rt = nullptr, *d = nullptr;
   uint8_t *mask = nullptr;
+  uint8_t *d_live = nullptr;  // per 32 nodes in row order: d may differ from 0 (k_ls_dir)
   std::vector<Level> lv;  // lv[0]: fine level geometry
   int depth = 0;          // levels in use (<= lv.size()); a schedule can cut the hierarchy short
   ac::Galerkin0Table tab0{};
@@ -338,7 +340,7 @@ struct ac_ctx {
   int64_t prof_launches[AC_PROF_COUNT] = {};
   double prof_bytes[AC_PROF_COUNT] = {};
   int64_t prof_corr_launches = 0;  // smoother launches that applied a pending correction
-  double settled_bytes[AC_PROF_COUNT] = {};  // bytes of a later cycle's smoothing and residual over all nodes
+  double settled_bytes[2][AC_PROF_COUNT] = {};  // a first / later cycle's smoothing and residual over all nodes
   bool prof_settled = false;                 // the profile holds cycles that did not visit all nodes
   // CUDA graphs (off on the legacy default stream, which cannot be captured)
   bool use_graphs = false;
@@ -697,8 +699,11 @@ int coarse_vcycle(ac_ctx *ctx, Solve &S, int k, void **res) {
 // r = rhs - S x, rho and the free-node count (zeroed first), the mask and
 // the tangent residual.
 int enqueue_smooth_resid(ac_ctx *ctx, Solve &S, SmoothVariant variant) {
-  const bool later = variant != kFirst && variant != kFirstSettled;
-  const bool settled = variant >= kFirstSettled, all = settled && variant != kLaterSettled;
+  const bool later = variant == kLater || variant == kLaterSettledAll || variant == kLaterSettled;
+  const bool settled = variant >= kFirstSettledAll;
+  const ac::SettledCycle which = variant == kFirstSettled   ? ac::kSettledStart
+                                 : variant == kLaterSettled ? ac::kSettledCycle
+                                                            : ac::kSettledAll;
   const ac::SolverOps *o = S.o;
   const ac::Geo &g0 = S.lv[0].g;
   const ByteModel bm = byte_model(ctx, S);
@@ -720,14 +725,14 @@ int enqueue_smooth_resid(ac_ctx *ctx, Solve &S, SmoothVariant variant) {
                                   ? ac::MaskDirty{S.lv[1].lists.dirty, ac::tiles_x(S.lv[1].g), ac::tiles_y(S.lv[1].g)}
                                   : ac::MaskDirty{nullptr, 0, 0};
   if (settled) {
-    if (variant == kLaterSettled) {
-      ctx->settled_bytes[AC_PROF_SMOOTH] = sm_bytes;
-      ctx->settled_bytes[AC_PROF_RESID] = 0.5 * bm.n * (bm.ns * (4 + bm.ob) + 1);
+    if (which != ac::kSettledAll) {
+      ctx->settled_bytes[later ? 1 : 0][AC_PROF_SMOOTH] = sm_bytes;
+      ctx->settled_bytes[later ? 1 : 0][AC_PROF_RESID] = 0.5 * bm.n * (bm.ns * (4 + bm.ob) + 1);
     }
     AC_RUNB(AC_PROF_SMOOTH, sm_bytes, o->smooth_settled(S.x, S.rhs, S.ob, corr, ctx->omega, g0, nsw, rt_zero, S.mask,
-                                                        dirty, ctx->rho, S.settled, all, ctx->s));
+                                                        dirty, ctx->rho, S.settled, which, ctx->s));
     AC_RUNB(AC_PROF_RESID, 0.5 * bm.n * (bm.ns * (4 + bm.ob) + 1),
-            o->resid_settled(S.x, S.rhs, S.ob, g0, S.rt, S.mask, ctx->rho, dirty, S.settled, all, ctx->s));
+            o->resid_settled(S.x, S.rhs, S.ob, g0, S.rt, S.mask, ctx->rho, dirty, S.settled, which, ctx->s));
     return AC_OK;
   }
   AC_RUNB(AC_PROF_SMOOTH, sm_bytes, o->smooth(S.x, S.rhs, S.ob, corr, ctx->omega, g0, nsw, rt_zero,
@@ -775,7 +780,7 @@ int enqueue_correction(ac_ctx *ctx, Solve &S) {
   // written; curvature: d and the mask read
   const double ls_bytes = bm.n * (bm.ns * (3 + bm.ob) + 1) + l1 + bm.n * (bm.ns + 1);
   AC_RUNB(AC_PROF_LINESEARCH, ls_bytes,
-          o->line_search(S.x, S.ob, S.rt, v1, S.mask, g0, L1.g, S.d, ctx->ls_part, ctx->ls_done, ctx->omega, ctx->s));
+          o->line_search(S.x, S.ob, S.rt, v1, S.mask, g0, L1.g, S.d, S.d_live, ctx->ls_part, ctx->ls_done, ctx->omega, ctx->s));
   return AC_OK;
 }
 
@@ -796,8 +801,10 @@ bool settled_form(const ac_ctx *ctx, const Solve &S, int64_t min_unknowns) {
 // Every stage keeps x feasible and does not raise the step energy, so the
 // limit is the unique minimiser that plain projected Gauss-Seidel (the
 // smoother alone) reaches.
+// start_list: the tiles' record and the outer residual's marks say where the
+// first cycle can change anything (solve_mixed).
 int solve_mg(ac_ctx *ctx, Solve &S, double tol, int max_cycles, int *cycles_out, double *rho_out,
-             int64_t *sweeps_out) {
+             int64_t *sweeps_out, bool start_list = false) {
   const bool coarse = S.depth > 1;
   double rho = 0;
   int cyc = 0, status = AC_ERR_NOT_CONVERGED;
@@ -809,7 +816,7 @@ int solve_mg(ac_ctx *ctx, Solve &S, double tol, int max_cycles, int *cycles_out,
     // only the tiles that can change while few nodes are free
     const bool settled = nsw >= 1 && settled_form(ctx, S, settled_min_unknowns(S.o->elem));
     const SmoothVariant variant = !settled ? (later ? kLater : kFirst)
-                                  : !later ? kFirstSettled
+                                  : !later ? (start_list ? kFirstSettled : kFirstSettledAll)
                                            : (S.record ? kLaterSettled : kLaterSettledAll);
     S.record = settled;
     int rc = run_graph(ctx, S.smooth_resid[prof][variant], [&]() { return enqueue_smooth_resid(ctx, S, variant); });
@@ -822,14 +829,14 @@ int solve_mg(ac_ctx *ctx, Solve &S, double tol, int max_cycles, int *cycles_out,
     if (rc) return rc;
     // the part of the tiles that the cycle visited
     double listed = 1.0;
-    if (variant == kLaterSettled) {
+    if (variant == kFirstSettled || variant == kLaterSettled) {
       ac::SettledCtl sc;
       std::memcpy(&sc, ctx->h_scalars + 2, sizeof sc);
       listed = (double)sc.count / ((double)S.settled.tx * S.settled.ty);
       if (ctx->profiling) {
         // the graph books every node: take the nodes not visited off again
         for (int cls : {(int)AC_PROF_SMOOTH, (int)AC_PROF_RESID})
-          ctx->prof_bytes[cls] -= (1.0 - listed) * ctx->settled_bytes[cls];
+          ctx->prof_bytes[cls] -= (1.0 - listed) * ctx->settled_bytes[later][cls];
         ctx->prof_settled = true;
       }
     }
@@ -892,12 +899,34 @@ int solve_mixed(ac_ctx *ctx, int *cycles_out, double *rho_out, int64_t *sweeps_o
   int64_t sweeps = 0;
   const bool rho32 = true;
   const double accept = ctx->p.tol * (1.0 - kRho32Rel);
+  Solve &S = ctx->sv;
+  // While the settled tiles' record stands (the last cycle of the last solve
+  // kept it), the tiles of the outer passes are known too.  The step's first
+  // residual visits every node (b is new) and marks the tiles where the
+  // correction is not 0 by itself or u not pure; x differs from 0 on the
+  // record's tiles only.  So a solve starts on the tiles with a mark, a free
+  // node or a nonzero x and those around them; the update changes u only
+  // where x is not 0 or a mark stands; and the next residual of the step
+  // differs only there and around.  4096^2, N = 8, formed phases, a step of
+  // two passes: residuals and updates 4.2 -> 1.6 ms, the solves' first cycles
+  // another 1.3 ms less.
+  bool listed = false;  // the marks describe u and b
+  int rc = AC_OK;
   for (;;) {
     AC_CUDA(cudaMemsetAsync(ctx->rho, 0, sizeof(double), ctx->s));
-    // u (binary64) and b (double-float pairs) read, r32 and u32 written
-    AC_RUNB(AC_PROF_OUTER, (double)ctx->n * ctx->N * 24,
-            o->outer_resid(ctx->u, (const float *)ctx->b, ctx->g0, ctx->r32, ctx->u32, ctx->rho, rho32, ctx->s));
-    int rc = read_rho(ctx, &rho);
+    if (outer > 0 && listed && S.record) {
+      AC_RUN(AC_PROF_OUTER, S.o->settled_list(S.settled, ac::kSetSeed | ac::kSetX, true, false, ctx->s));
+      AC_RUN(AC_PROF_OUTER, o->outer_resid_tiles(ctx->u, (const float *)ctx->b, ctx->g0, ctx->r32, ctx->u32, ctx->rho,
+                                                 S.settled, ctx->s));
+    } else {
+      listed = S.record && settled_form(ctx, S, settled_min_unknowns(S.o->elem));
+      if (listed) AC_CUDA(cudaMemsetAsync(S.settled.seed, 0, (size_t)S.settled.tx * S.settled.ty, ctx->s));
+      // u (binary64) and b (double-float pairs) read, r32 and u32 written
+      AC_RUNB(AC_PROF_OUTER, (double)ctx->n * ctx->N * 24,
+              o->outer_resid(ctx->u, (const float *)ctx->b, ctx->g0, ctx->r32, ctx->u32, ctx->rho, rho32,
+                             listed ? S.settled.seed : nullptr, S.settled.tx, ctx->s));
+    }
+    rc = read_rho(ctx, &rho);
     if (rc) return rc;
 #ifdef AC_TRACE_CYCLES
     std::fprintf(stderr, "outer %d rho %.3e\n", outer, rho);
@@ -919,20 +948,31 @@ int solve_mixed(ac_ctx *ctx, int *cycles_out, double *rho_out, int64_t *sweeps_o
     // same step starts from zero.
     const bool warm = outer == 0 && ctx->delta_warm && ctx->p.nu1 >= 1;
     ctx->delta_warm = false;
-    if (!warm) AC_CUDA(cudaMemsetAsync(ctx->sv.x, 0, (size_t)fine_slots(ctx->n) * ctx->N * sizeof(float), ctx->s));
+    if (!warm && listed) {
+      AC_RUN(AC_PROF_OUTER, S.o->settled_list(S.settled, ac::kSetX, false, false, ctx->s));
+      AC_RUN(AC_PROF_OUTER, S.o->settled_zero(S.x, ctx->g0, S.settled, ctx->s));
+    } else if (!warm) {
+      AC_CUDA(cudaMemsetAsync(S.x, 0, (size_t)fine_slots(ctx->n) * ctx->N * sizeof(float), ctx->s));
+    }
     int c = 0;
     int64_t sw = 0;
     double rin = 0;
     const int cap = ctx->p.max_cycles - cycles < kInnerMaxCycles ? ctx->p.max_cycles - cycles : kInnerMaxCycles;
-    rc = solve_mg(ctx, ctx->sv, std::fmax(kInnerTolFrac * ctx->p.tol, kInnerReduction * rho), cap, &c, &rin, &sw);
+    rc = solve_mg(ctx, S, std::fmax(kInnerTolFrac * ctx->p.tol, kInnerReduction * rho), cap, &c, &rin, &sw, listed);
     cycles += c;
     sweeps += sw;
     if (rc && rc != AC_ERR_NOT_CONVERGED) return rc;
-    // u read and written, delta read
-    AC_RUNB(AC_PROF_OUTER, (double)ctx->n * ctx->N * 20,
-            o->outer_update(ctx->u, (const float *)ctx->sv.x, ctx->g0, ctx->s));
+    const int solved = rc;
+    if (listed && S.record) {
+      AC_RUN(AC_PROF_OUTER, S.o->settled_list(S.settled, ac::kSetSeed | ac::kSetX, false, false, ctx->s));
+      AC_RUN(AC_PROF_OUTER, o->outer_update_tiles(ctx->u, (const float *)S.x, ctx->g0, S.settled, ctx->s));
+    } else {
+      // u read and written, delta read
+      AC_RUNB(AC_PROF_OUTER, (double)ctx->n * ctx->N * 20,
+              o->outer_update(ctx->u, (const float *)S.x, ctx->g0, ctx->s));
+    }
     ++outer;
-    ctx->delta_warm = rc == AC_OK && outer == 1;
+    ctx->delta_warm = solved == AC_OK && outer == 1;
   }
   *cycles_out = cycles;
   *rho_out = rho;
@@ -1207,7 +1247,8 @@ int enqueue_step_loop(ac_ctx *ctx, cudaGraph_t top, bool energy, StepGraph &sg) 
     auto outer_resid = [&]() -> int {
       AC_CUDA(cudaMemsetAsync(ctx->rho, 0, sizeof(double), ctx->s));
       AC_RUNB(AC_PROF_OUTER, (double)ctx->n * ctx->N * 24,
-              o->outer_resid(ctx->u, (const float *)ctx->b, ctx->g0, ctx->r32, ctx->u32, ctx->rho, true, ctx->s));
+              o->outer_resid(ctx->u, (const float *)ctx->b, ctx->g0, ctx->r32, ctx->u32, ctx->rho, true, nullptr, 0,
+                             ctx->s));
       AC_RUN(AC_PROF_OUTER,
              (ac::launch(k_ctl_outer, 1, 1, 0, ctx->s, ctx->ctl, ctx->rho, accept, ctx->p.tol, kInnerTolFrac, kInnerReduction,
                                                ctx->p.max_cycles, kInnerMaxCycles, ctx->p.nu1, h_out),
@@ -1284,6 +1325,7 @@ int loop_stats(ac_ctx *ctx, const StepGraph &sg, int n_steps, ac_stats *out) {
                          (c.total_cycles - solves) * sg.per_cycle;
   ctx->delta_warm = c.warm != 0;
   ctx->have_rhs = true;
+  ctx->sv.record = false;  // the device-side loop keeps no record of its tiles
   if (out) {
     out->residual = c.last_rho;
     out->cycles = c.last_cycles;
@@ -1617,6 +1659,8 @@ int ac_create(ac_ctx **out, const ac_params *p) {
     AC_ALLOC(S.mask, (size_t)ctx->n);
     AC_CUDA(cudaMemsetAsync(S.mask, 0, (size_t)ctx->n, ctx->s));  // read as a hint before the first cycle sets it
     if (S.lv.size() > 1) AC_ALLOC(S.d, fNs);
+    AC_ALLOC(S.d_live, (size_t)(ctx->n + 31) / 32);
+    AC_CUDA(cudaMemsetAsync(S.d_live, 1, (size_t)(ctx->n + 31) / 32, ctx->s));
     {
       // the settled tiles' record, one allocation: rho (8 bytes a tile for
       // either scalar), list, then the byte arrays
@@ -1626,13 +1670,15 @@ int ac_create(ac_ctx **out, const ac_params *p) {
       st.sms = ctx->sms;
       const size_t nt = (size_t)st.tx * st.ty;
       uint8_t *mem = nullptr;
-      AC_ALLOC(mem, 17 * nt + 4);
+      AC_ALLOC(mem, 20 * nt + 4);
       st.rho = mem;
       st.list = reinterpret_cast<unsigned *>(mem + 8 * nt);
       st.listed = mem + 12 * nt;
       st.changed = st.listed + (nt + 3) / 4 * 4;
       st.free = st.changed + nt;
       st.nfree = st.free + 2 * nt;
+      st.seed = st.nfree + nt;
+      st.nonzero = st.seed + nt;
     }
     AC_ALLOC(ctx->part, (size_t)ac::kMaxPartBlocks * 7 * N * sizeof(double));
     AC_ALLOC(ctx->tot, (size_t)7 * N * sizeof(double));
@@ -2014,7 +2060,8 @@ int ac_residual(ac_ctx *ctx, double *rho) {
   AC_CUDA(cudaMemsetAsync(ctx->rho, 0, sizeof(double), ctx->s));
   if (ctx->p.precision == AC_MIXED)
     AC_RUN(AC_PROF_OUTER,
-           ctx->ops->outer_resid(ctx->u, (const float *)ctx->b, ctx->g0, ctx->r32, ctx->u32, ctx->rho, false, ctx->s));
+           ctx->ops->outer_resid(ctx->u, (const float *)ctx->b, ctx->g0, ctx->r32, ctx->u32, ctx->rho, false, nullptr, 0,
+                                 ctx->s));
   else
     AC_RUN(AC_PROF_RESID,
            ctx->ops->fp64.resid(ctx->u, ctx->b, nullptr, ctx->g0, nullptr, nullptr, ctx->rho, -1,
@@ -2245,6 +2292,8 @@ int adj_setup(ac_ctx *ctx, int T, int every) {
     ADJ_ALLOC(S.rt, fS);
     ADJ_ALLOC(S.d, fS);
     ADJ_ALLOC(S.mask, (size_t)ctx->n);
+    ADJ_ALLOC(S.d_live, (size_t)(ctx->n + 31) / 32);
+    AC_CUDA(cudaMemsetAsync(S.d_live, 1, (size_t)(ctx->n + 31) / 32, ctx->s));
     AC_CUDA(cudaMemsetAsync(S.rt, 0, fS, ctx->s));  // second-colour slots stay 0 (see solve_mg)
     return AC_OK;
   };
@@ -2531,6 +2580,7 @@ void set_schedule(ac_ctx *ctx, int nu1, int nu2, int depth, bool gs) {
   ctx->sv.depth = depth < 1 ? 1 : (depth > L ? L : depth);
   ctx->delta_warm = false;  // the next step starts its correction from zero
   ctx->sv.was_tiled = false;
+  ctx->sv.record = false;
   // the tiled levels may change with the depth: let the next cycle write
   // every tile of every level again (see kLiveNow)
   for (int k = 1; k < L; ++k) {

@@ -88,8 +88,12 @@ constexpr int kSetT = 8;
 struct SettledCtl {
   unsigned count, joined;  // tiles in the list, and at its far end
 };
+// Marks of a list (k_settled_list): a cycle's seeds; where the correction is
+// not 0 by itself at the start of a solve, or u not pure (k_outer_resid_df);
+// where x is not 0 (nonzero[colour][tile]).
+enum { kSetCycle = 1, kSetSeed = 2, kSetX = 4 };
 struct SettledTiles {
-  uint8_t *changed, *free, *nfree, *listed;  // listed: 4-byte aligned
+  uint8_t *changed, *free, *nfree, *listed, *seed, *nonzero;  // listed: 4-byte aligned
   void *rho;
   unsigned *list;
   SettledCtl *ctl;

@@ -93,13 +93,21 @@ struct SolverLaunch {
     constexpr int W = kBlock / 32;
     return dim3((unsigned)std::min((st.tx * st.ty + W - 1) / W, st.sms * per_sm));
   }
+  static int settled_list(const SettledTiles &st, unsigned what, bool around, bool restart, cudaStream_t s) {
+    cudaMemsetAsync(st.ctl, 0, sizeof(SettledCtl), s);
+    launch(k_settled_list<T>, dim3(blocks_for((int64_t)st.tx * st.ty)), kBlock, 0, s, st, what, around, restart);
+    return 1;
+  }
+  static int settled_zero(void *x, const Geo &g, const SettledTiles &st, cudaStream_t s) {
+    launch(k_settled_zero<T, N>, settled_grid(st, k_settled_zero<T, N>), kBlock, 0, s, (T *)x, g, st);
+    return 1;
+  }
   static int smooth_settled(void *x, const void *rhs, const void *ob, const void *corr, const double *omega,
                             const Geo &g, int sweeps, void *rt, uint8_t *mask, const MaskDirty &dirty, double *rho,
-                            const SettledTiles &st, bool all, cudaStream_t s) {
-    if (!all) {
-      cudaMemsetAsync(st.ctl, 0, sizeof(SettledCtl), s);
-      launch(k_settled_list, dim3(blocks_for((int64_t)st.tx * st.ty)), kBlock, 0, s, st);
-    }
+                            const SettledTiles &st, SettledCycle which, cudaStream_t s) {
+    const bool all = which == kSettledAll;
+    if (which == kSettledCycle) settled_list(st, kSetCycle, true, false, s);
+    if (which == kSettledStart) settled_list(st, kSetCycle | kSetSeed | kSetX, true, true, s);
     for (int p = 0; p < 2 * sweeps; ++p) {
       const T *cr = p == 0 ? (const T *)corr : nullptr;
       if (p == 2 * sweeps - 1)
@@ -116,7 +124,9 @@ struct SolverLaunch {
     return 2 * sweeps + (all ? 0 : 1);
   }
   static int resid_settled(const void *x, const void *rhs, const void *ob, const Geo &g, void *rt, uint8_t *mask,
-                           double *rho, const MaskDirty &dirty, const SettledTiles &st, bool all, cudaStream_t s) {
+                           double *rho, const MaskDirty &dirty, const SettledTiles &st, SettledCycle which,
+                           cudaStream_t s) {
+    const bool all = which == kSettledAll;
     launch(k_resid_settled<T, N, FORM>, settled_grid(st, k_resid_settled<T, N, FORM>), kBlock, 0, s, (const T *)x,
            (const T *)rhs, (const T *)ob, g, (T *)rt, mask, rho, dirty, st, all);
     return 1;
@@ -261,7 +271,7 @@ struct SolverLaunch {
               : coarse_tail_t<false>(a, r0, v0, coarse_sweeps, coarsest_sweeps, smem, s);
   }
   static int line_search(const void *x, const void *ob, const void *rt, const void *v1, const uint8_t *mask,
-                         const Geo &gf, const Geo &gc, void *d, double *part, unsigned *done, double *omega,
+                         const Geo &gf, const Geo &gc, void *d, uint8_t *live, double *part, unsigned *done, double *omega,
                          cudaStream_t s) {
     // one resident set of blocks while a block then takes at most eight
     // chunks, so that the closing sum of the last block stays near 1 us
@@ -273,18 +283,24 @@ struct SolverLaunch {
     const int chunks = (int)((all + want - 1) / want);
     const unsigned grid = (unsigned)((all + chunks - 1) / chunks);
     launch(k_ls_dir<T, N, FORM>, grid, kBlock, 0, s, (const T *)x, (const T *)ob, (const T *)rt, (const T *)v1, mask, gf,
-                                               gc, chunks, (T *)d, part);
+                                               gc, chunks, (T *)d, live, part);
     launch(k_ls_curv<T, N>, grid, kBlock, 0, s, (const T *)d, mask, gf, chunks, part, done, omega);
     return 2;
   }
   static SolverOps table() {
     decltype(SolverOps::smooth_settled) ss = nullptr;  // the adjoint's solves keep no record of their tiles
     decltype(SolverOps::resid_settled) rs = nullptr;
+    decltype(SolverOps::settled_list) sl = nullptr;
+    decltype(SolverOps::settled_zero) sz = nullptr;
     if constexpr (FORM != kTangent) {
       ss = smooth_settled;
       rs = resid_settled;
     }
-    return SolverOps{(int)sizeof(T), smooth,       resid,        ss, rs, restrict0,   galerkin0,   galerkin,   coarse_smooth,
+    if constexpr (FORM == kShifted) {
+      sl = settled_list;
+      sz = settled_zero;
+    }
+    return SolverOps{(int)sizeof(T), smooth,       resid,        ss, rs, sl, sz, restrict0,   galerkin0,   galerkin,   coarse_smooth,
                      coarse_resid, coarse_pre_resid, restrict_, prolong_add, coarse_tail,
                      line_search};
   }
@@ -347,13 +363,14 @@ struct Launch {
     return 1;
   }
   static int outer_resid(const double *u, const float *b, const Geo &g, float *r32, float *u32, double *rho,
-                         bool rho32, cudaStream_t s) {
+                         bool rho32, uint8_t *seeds, int seeds_x, cudaStream_t s) {
     if (rho32) {
       static const cudaError_t attr = cudaFuncSetAttribute(
           k_outer_resid_df<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)outer_resid_smem<N>());
       (void)attr;
       launch(k_outer_resid_df<N>, dim3((g.W + 1 + kOrThreads - 3) / (kOrThreads - 2), (g.H + kOrRows) / kOrRows),
-                            kOrThreads, outer_resid_smem<N>(), s, u, b, g, r32, u32, rho);
+                            kOrThreads, outer_resid_smem<N>(), s, u, b, g, r32, u32, rho, seeds,
+             seeds_x);
     }
     else
       launch(k_outer_resid<N>, row_grid(g.W + 1, g.H + 1), kBlock, 0, s, u, b, g, r32, u32, rho);
@@ -361,6 +378,17 @@ struct Launch {
   }
   static int outer_update(double *u, const float *delta, const Geo &g, cudaStream_t s) {
     launch(k_outer_update<N>, row_grid(g.W + 1, g.H + 1), kBlock, 0, s, u, delta, g);
+    return 1;
+  }
+  static int outer_resid_tiles(const double *u, const float *b, const Geo &g, float *r32, float *u32, double *rho,
+                               const SettledTiles &st, cudaStream_t s) {
+    launch(k_outer_resid_tiles<N>, SolverLaunch<float, N, kShifted>::settled_grid(st, k_outer_resid_tiles<N>), kBlock, 0,
+           s, u, b, g, r32, u32, rho, st);
+    return 1;
+  }
+  static int outer_update_tiles(double *u, const float *delta, const Geo &g, const SettledTiles &st, cudaStream_t s) {
+    launch(k_outer_update_tiles<N>, SolverLaunch<float, N, kShifted>::settled_grid(st, k_outer_update_tiles<N>), kBlock,
+           0, s, u, delta, g, st);
     return 1;
   }
   static int composite(const double *u, const double *c, const Geo &g, int r, int rounded, float *out,
@@ -450,6 +478,8 @@ struct Launch {
                           rhs_df,
                           outer_resid,
                           outer_update,
+                          outer_resid_tiles,
+                          outer_update_tiles,
                           labels,
                           composite,
                           project,

@@ -48,6 +48,11 @@ struct LevelLists {
   int sms;
 };
 
+// The tiles a cycle visits: all, which starts their record; those that the
+// record of the last cycle leaves; or, at the start of a solve, those and the
+// ones that the outer residual marked.
+enum SettledCycle { kSettledAll, kSettledCycle, kSettledStart };
+
 // One multigrid solve instantiation (scalar type and constraint form); array
 // arguments are typed by that instantiation (double or float).
 struct SolverOps {
@@ -66,9 +71,14 @@ struct SolverOps {
   // that can change in the cycle, or on all of them to start their record
   int (*smooth_settled)(void *x, const void *rhs, const void *ob, const void *corr, const double *omega, const Geo &g,
                         int sweeps, void *rt, uint8_t *mask, const MaskDirty &dirty, double *rho,
-                        const SettledTiles &st, bool all, cudaStream_t s);
+                        const SettledTiles &st, SettledCycle which, cudaStream_t s);
   int (*resid_settled)(const void *x, const void *rhs, const void *ob, const Geo &g, void *rt, uint8_t *mask,
-                       double *rho, const MaskDirty &dirty, const SettledTiles &st, bool all, cudaStream_t s);
+                       double *rho, const MaskDirty &dirty, const SettledTiles &st, SettledCycle which,
+                       cudaStream_t s);
+  // mixed form: the list of the tiles with a mark in `what` (and those around
+  // them), and x = 0 on a list
+  int (*settled_list)(const SettledTiles &st, unsigned what, bool around, bool restart, cudaStream_t s);
+  int (*settled_zero)(void *x, const Geo &g, const SettledTiles &st, cudaStream_t s);
   // transfers skip the rows whose diagonal in the (coarse or fine) level's
   // operator is 0: those rows and their residuals are exactly 0.  LevelLists
   // arguments: the live-tile state of a tiled level, or null for a level
@@ -103,9 +113,9 @@ struct SolverOps {
   int (*coarse_tail)(const TailArgs &a, const void *r0, void *v0, int coarse_sweeps, int coarsest_sweeps,
                      size_t smem, bool gs, cudaStream_t s);
   // line search: part needs 2 x (blocks of the fine grid) doubles, done is
-  // a counter that is 0 between calls
+  // a counter that is 0 between calls, live one byte per 32 nodes (1 at first)
   int (*line_search)(const void *x, const void *ob, const void *rt, const void *v1, const uint8_t *mask,
-                     const Geo &gf, const Geo &gc, void *d, double *part, unsigned *done, double *omega,
+                     const Geo &gf, const Geo &gc, void *d, uint8_t *live, double *part, unsigned *done, double *omega,
                      cudaStream_t s);
 };
 
@@ -129,9 +139,14 @@ struct Ops {
   // arithmetic, with the natural residual through the float projection
   // (accurate to a few float ulps of rho near the solution); otherwise FP64
   // throughout
+  // (seeds: nullable, zeroed; the settled tiles' marks, seeds_x tiles a row)
   int (*outer_resid)(const double *u, const float *b, const Geo &g, float *r32, float *u32, double *rho, bool rho32,
-                     cudaStream_t s);
+                     uint8_t *seeds, int seeds_x, cudaStream_t s);
   int (*outer_update)(double *u, const float *delta, const Geo &g, cudaStream_t s);
+  // the solve's residual and the update on the listed tiles
+  int (*outer_resid_tiles)(const double *u, const float *b, const Geo &g, float *r32, float *u32, double *rho,
+                           const SettledTiles &st, cudaStream_t s);
+  int (*outer_update_tiles)(double *u, const float *delta, const Geo &g, const SettledTiles &st, cudaStream_t s);
   // pixel outputs are on the image's pixels: the solve grid g coarsened r times
   int (*labels)(const double *u, const Geo &g, int r, int8_t *node_lab, int8_t *pix_lab, cudaStream_t s);
   int (*composite)(const double *u, const double *c, const Geo &g, int r, int rounded, float *out, cudaStream_t s);
