@@ -375,8 +375,16 @@ __global__ void __launch_bounds__(kBlock, 2) k_means_partial_df(const double *__
 #pragma unroll
       for (int i = 0; i < N; ++i) split_f64(t[i], uh[i], ul[i]);
     }
+    // the phases that some node of the warp has: a zero adds nothing (formed
+    // phases leave one or two of N in a warp)
+    const unsigned lanes = __activemask();
+    unsigned own = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) own |= uh[i] != 0.f ? 1u << i : 0u;
+    const unsigned any = __reduce_or_sync(lanes, own);
 #pragma unroll
     for (int i = 0; i < N; ++i) {
+      if (!((any >> i) & 1u)) continue;
 #pragma unroll
       for (int q = 0; q < 4; ++q) {
         const f2 p = mul_f2(uh[i], ul[i], mh[q], ml[q]);
@@ -386,6 +394,7 @@ __global__ void __launch_bounds__(kBlock, 2) k_means_partial_df(const double *__
     if constexpr (ENERGY) {
 #pragma unroll
       for (int i = 0; i < N; ++i) {
+        if (!((any >> i) & 1u)) continue;
         f2 p = mul_f2(uh[i], ul[i], mh[4], ml[4]);  // u m2
         acc[4 * N] = add_f2(acc[4 * N], p.h, p.l);
         f2 v = two_sum(1.f, -uh[i]);  // 1 - u
@@ -399,13 +408,20 @@ __global__ void __launch_bounds__(kBlock, 2) k_means_partial_df(const double *__
       const Weights w = edge_weights(g, x, y);
       auto edge = [&](int64_t nb, float we) {
         double t[N];
+        float th[N], tl[N];
         ldn<double, N>(u + nb * N, t);
+        unsigned diff = 0;
 #pragma unroll
         for (int i = 0; i < N; ++i) {
-          float h, l;
-          split_f64(t[i], h, l);
-          f2 d = two_sum(uh[i], -h);
-          d = fast_two_sum(d.h, d.l + (ul[i] - l));
+          split_f64(t[i], th[i], tl[i]);
+          diff |= (th[i] != uh[i] || tl[i] != ul[i]) ? 1u << i : 0u;
+        }
+        diff = __reduce_or_sync(__activemask(), diff);
+#pragma unroll
+        for (int i = 0; i < N; ++i) {
+          if (!((diff >> i) & 1u)) continue;
+          f2 d = two_sum(uh[i], -th[i]);
+          d = fast_two_sum(d.h, d.l + (ul[i] - tl[i]));
           const f2 p = mul_f2(d.h, d.l, d.h, d.l);
           acc[4 * N + 2] = add_f2(acc[4 * N + 2], we * p.h, we * p.l);
         }
@@ -667,9 +683,13 @@ __device__ __forceinline__ float or_node(B &&bval, const Geo &g, int x, int y, c
     for (int i = 0; i < N; ++i) sh[i] = sl[i] = 0.f;
     if (x > 0 && x < g.W && y > 0 && y < g.H) {
       // (u_E + u_W + u_N + u_S) - 4 u: the heads summed by two-sums, 4 u_h
-      // exactly, the tails and the two-sum errors in float
+      // exactly, the tails and the two-sum errors in float; phases that are 0
+      // at and around all nodes of the warp stay 0
+      const unsigned lanes = __activemask();
 #pragma unroll
       for (int i = 0; i < N; ++i) {
+        const unsigned any = f32_bits(eh[i]) | f32_bits(wh[i]) | f32_bits(nh[i]) | f32_bits(ph[i]) | f32_bits(uh[i]);
+        if (!__any_sync(lanes, (any << 1) != 0u)) continue;
         const f2 a = two_sum(eh[i], wh[i]);
         const f2 b = two_sum(nh[i], ph[i]);
         const f2 c = two_sum(a.h, b.h);
