@@ -204,6 +204,13 @@ __device__ __forceinline__ void cp_async_wait() {
   asm volatile("cp.async.wait_group %0;\n" ::"n"(K) : "memory");
 }
 
+// Rounded operations that the compiler neither splits nor fuses: the nodal
+// problems give the same bits in every kernel that solves them.
+__device__ __forceinline__ float fma_rn(float a, float b, float c) { return __fmaf_rn(a, b, c); }
+__device__ __forceinline__ double fma_rn(double a, double b, double c) { return __fma_rn(a, b, c); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+
 // ---- vector loads / stores of one node's N values ------------------------
 
 template <typename T, int N>
@@ -315,7 +322,7 @@ __device__ __forceinline__ void proj_box(T (&z)[N], const T (&ob)[N]) {
         s += z[i];
         ++k;
       }
-    const T mean = k >= 2 ? s * rcp_small<T>(k) : T(0);
+    const T mean = k >= 2 ? mul_rn(s, rcp_small<T>(k)) : T(0);
 #pragma unroll
     for (int i = 0; i < N; ++i) z[i] = (k >= 2 && ob[i] != T(0)) ? z[i] - mean : T(0);
     return;
@@ -326,7 +333,7 @@ __device__ __forceinline__ void proj_box(T (&z)[N], const T (&ob)[N]) {
     T s = T(0);
 #pragma unroll
     for (int i = 0; i < N; ++i) s += z[i];
-    T theta = (s - total) * rcp_small<T>(N);
+    T theta = mul_rn(s - total, rcp_small<T>(N));
 #pragma unroll 1
     for (int pass = 1; pass < N; ++pass) {
       unsigned drop = 0;
@@ -351,7 +358,7 @@ __device__ __forceinline__ void proj_box(T (&z)[N], const T (&ob)[N]) {
           L -= ob[i];
         }
       }
-      theta = (s + L - total) * rcp_small<T>(k);
+      theta = mul_rn(s + L - total, rcp_small<T>(k));
     }
 #pragma unroll
     for (int i = 0; i < N; ++i) z[i] = ((keep >> i) & 1u) ? z[i] - theta : (SH ? -ob[i] : T(0));
@@ -476,49 +483,35 @@ __device__ __forceinline__ void nbr_sum(const T *u, const Geo &g, int x, int y, 
 }
 
 // ---- the FP64 direct form's nodal problem ------------------------------------
-// GB300 runs binary64 arithmetic at 1/64 of its float rate, and the FP64
-// form's smoother and residual were bound by it: five operations per phase for
-// z = (b + tau eps sum_m w_nm u_m) / S_nn, then two per kept phase and
-// projection pass.  But a node keeps one to three phases once they form, and
-// the others' values are only ever compared with the threshold.  So a float
-// pass on the values' heads finds the set the projection keeps, binary64 runs
-// on those phases alone, and the set is checked afterwards: a kept z above the
-// binary64 theta, a dropped one's float value below it by more than its error
-// bound.  Where the check holds, the binary64 iteration of proj_box ends on
-// the same set and sums it in the same order (see outer_update_node): the
-// result is bit-identical to it.  Near ties, and for values a float cannot
-// hold, the plain path runs.
-// At 1024^2, N = 4, formed phases: smoother pass 77 -> 34 us, residual 130 ->
-// 89 us; on a random start, where the nodes keep most phases and many_free64
-// takes the plain path, the step is 1% slower.
-
+// GB300 runs binary64 arithmetic at about 1/64 of its float rate, one warp
+// instruction in 26 cycles of an SM (counted: 181,530 in 23 us of a pass at
+// 512^2, N = 4), and the FP64 form's smoother and residual were bound by it:
+// per phase three additions for the neighbours' sum, two operations for z =
+// (b + tau eps sum_m w_nm u_m) / S_nn, then the projection's sums and
+// comparisons.  The phase field lies in [0, 1], so all but z's two operations
+// run in 64-bit fixed point (ac_df64.cuh): the neighbours' sum to 2^-60, the
+// projection of z to 2^-58, closer than the binary64 chain (2^-53 a step).
+// Values outside the ranges, and NaN, take the plain binary64 path.
+// Smoothing formed phases at 1024^2, N = 4: 0.77 -> 0.67 ms a step; a step from
+// random phases at 512^2, N = 8: 6.45 -> 5.25 ms; gradients at 512^2: 60 -> 47 ms.
+constexpr int kFixU = 60, kFixZ = 57;  // fractional bits of phase values and of z
 template <typename T, int FORM>
-constexpr bool kFilter64 = std::is_same<T, double>::value && FORM == kDirect;
+constexpr bool kFixed64 = std::is_same<T, double>::value && FORM == kDirect;
 
-// Whether the warp's nodes, by their free masks of the last cycle, keep more
-// than three quarters of the phases between them: the plain path is then
-// faster (both give the same bits, so a stale mask costs time only).
+// s_i += sum_m w_nm u_m in 2^-kFixU (weights 0, 1/2 and 1).
 template <int N>
-__device__ __forceinline__ bool many_free64(uint8_t mask) {
-  return 4 * __popc(__reduce_or_sync(__activemask(), (unsigned)mask)) > 3 * N;
-}
-
-// The heads' sums over all phases, acc += f sum_m w_nm u_m and mag += the sum
-// of magnitudes.
-template <int N>
-__device__ __forceinline__ void nbr_heads(const double *u, const Geo &g, int x, int y, const Weights &w, float f,
-                                          float (&acc)[N], float (&mag)[N]) {
+__device__ __forceinline__ void nbr_sum_fixed(const double *u, const Geo &g, int x, int y, int64_t (&s)[N],
+                                              bool &bad) {
+  const Weights w = edge_weights(g, x, y);
   const double *p = u + ((int64_t)y * g.Wn + x) * N;
   auto add = [&](const double *q, float we) {
-    if (we > 0.f) {
-      double t[N];
-      ldn_rw<double, N>(q, t);
+    if (we == 0.f) return;
+    double t[N];
+    ldn_rw<double, N>(q, t);
 #pragma unroll
-      for (int i = 0; i < N; ++i) {
-        const float h = (f * we) * f64_head(t[i]);
-        acc[i] += h;
-        mag[i] += fabsf(h);
-      }
+    for (int i = 0; i < N; ++i) {
+      const int64_t f = f64_to_fix<kFixU, 1>(t[i], bad);
+      s[i] += we == 1.f ? f : f >> 1;
     }
   };
   add(p + N, w.e);
@@ -527,125 +520,44 @@ __device__ __forceinline__ void nbr_heads(const double *u, const Geo &g, int x, 
   add(p - (int64_t)g.Wn * N, w.s);
 }
 
-// sum_m w_nm u_m for phase i alone in binary64 (nbr_sum's order), read again
-// from L1: keeping the neighbours' values in registers instead (N = 4: 94
-// against 62) was slower, 2.47 against 2.30 ms of smoothing at 1024^2.
-template <int N>
-__device__ __forceinline__ double nbr_sum1(const double *u, const Geo &g, int x, int y, const Weights &w, bool inside,
-                                           int i) {
-  const double *p = u + ((int64_t)y * g.Wn + x) * N + i;
-  const int64_t row = (int64_t)g.Wn * N;
-  if (inside) return ((p[N] + p[-N]) + p[row]) + p[-row];
-  double acc = 0.0;
-  if (w.e > 0.f) acc += (double)w.e * p[N];
-  if (w.w > 0.f) acc += (double)w.w * p[-N];
-  if (w.n > 0.f) acc += (double)w.n * p[row];
-  if (w.s > 0.f) acc += (double)w.s * p[-row];
-  return acc;
+// |v| 2^-F with v's sign.
+template <int F>
+__device__ __forceinline__ double fix_to_f64_signed(int64_t v) {
+  const double a = fix_to_f64<F>(v < 0 ? -v : v);
+  return v < 0 ? -a : a;
 }
 
-// q_i = b_i + te (sum_m w_nm u_m + omega sum_m w_nm d_m)_i and z_i = q_i / S_nn
-// at node (x, y), and the set and threshold of z's projection: out_i = z_i -
-// theta on keep, 0 elsewhere.  q and z are set for the phases of keep and
-// `also` (all phases where the plain path runs).  d null: no correction.
+// At node (x, y): q_i = b_i + te (sum_m w_nm u_m + omega sum_m w_nm d_m)_i (d
+// null: no correction) and the projection of z_i = q_i / S_nn onto the
+// simplex, out_i = (z_i - theta) 2^-kFixZ on keep, 0 elsewhere.  False where a
+// value leaves its range (nothing is then meaningful).
 template <int N>
-__device__ __forceinline__ void direct_node64(const double *u, const double *d, double omega, const double (&b)[N],
-                                              const Geo &g, int x, int y, unsigned also, double (&q)[N],
-                                              double (&z)[N], unsigned &keep, double &theta) {
+__device__ __forceinline__ bool direct_node_fixed(const double *u, const double *d, double omega, const double (&b)[N],
+                                                  const Geo &g, int x, int y, double (&q)[N], int64_t (&z)[N],
+                                                  unsigned &keep, int64_t &theta) {
   const int cls = node_class(g, x, y);
-  const Weights w = edge_weights(g, x, y);
-  const bool inside = cls == 4;
-  float zf[N], er[N];
-  {
-    float acc[N], mag[N];
-#pragma unroll
-    for (int i = 0; i < N; ++i) acc[i] = mag[i] = 0.f;
-    nbr_heads<N>(u, g, x, y, w, 1.f, acc, mag);
-    if (d) nbr_heads<N>(d, g, x, y, w, f64_head(omega), acc, mag);
-    // heads within 2^-23 of their values, at most eight terms, the constants
-    // and three more operations rounded: |zf - z| < 2^-19 (|b| + te mag) / S_nn
-    // (2^-100: values flushed to 0)
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-      const float bf = f64_head(b[i]);
-      zf[i] = (bf + g.tef * acc[i]) * g.invDf[cls];
-      er[i] = (fabsf(bf) + g.tef * mag[i]) * g.invDf[cls] * 0x1.0p-19f + 0x1.0p-100f;
-    }
-  }
-  // Michelot's iteration on the float values
-  keep = (1u << N) - 1u;
-  {
-    float s = 0.f;
-#pragma unroll
-    for (int i = 0; i < N; ++i) s += zf[i];
-    float t = (s - 1.f) * rcp_small<float>(N);
-#pragma unroll 1
-    for (int pass = 1; pass < N; ++pass) {
-      unsigned drop = 0;
-#pragma unroll
-      for (int i = 0; i < N; ++i)
-        if (((keep >> i) & 1u) && zf[i] <= t) drop |= 1u << i;
-      if (!drop || drop == keep) break;
-      keep &= ~drop;
-      s = 0.f;
-#pragma unroll
-      for (int i = 0; i < N; ++i)
-        if ((keep >> i) & 1u) s += zf[i];
-      t = (s - 1.f) * rcp_small<float>(__popc(keep));
-    }
-  }
   const double te = g.te, invD = g.invD[cls];
-  const unsigned lanes = __activemask();
-  auto value = [&](int i) {
-    double acc = nbr_sum1<N>(u, g, x, y, w, inside, i);
-    if (d && omega != 0.0) acc += omega * nbr_sum1<N>(d, g, x, y, w, inside, i);
-    q[i] = b[i] + te * acc;
-    z[i] = q[i] * invD;
-  };
-  const unsigned need = keep | also, any = __reduce_or_sync(lanes, need);
-  double s = 0.0;
+  int64_t s[N];
+  bool bad = false;
+#pragma unroll
+  for (int i = 0; i < N; ++i) s[i] = 0;
+  nbr_sum_fixed<N>(u, g, x, y, s, bad);
+#pragma unroll
+  for (int i = 0; i < N; ++i) q[i] = fix_to_f64_signed<kFixU>(s[i]);
+  if (d && omega != 0.0) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) s[i] = 0;
+    nbr_sum_fixed<N>(d, g, x, y, s, bad);
+#pragma unroll
+    for (int i = 0; i < N; ++i) q[i] = fma_rn(omega, fix_to_f64_signed<kFixU>(s[i]), q[i]);
+  }
 #pragma unroll
   for (int i = 0; i < N; ++i) {
-    if (!((any >> i) & 1u)) continue;  // no lane of the warp needs phase i
-    if ((need >> i) & 1u) value(i);
-    if ((keep >> i) & 1u) s += z[i];
+    q[i] = fma_rn(te, q[i], b[i]);
+    z[i] = f64_to_fix<kFixZ, 2>(mul_rn(q[i], invD), bad);
   }
-  theta = (s - 1.0) * rcp_small<double>(__popc(keep));
-  const float t32 = f64_head(theta);
-  bool ok = true;
-#pragma unroll
-  for (int i = 0; i < N; ++i) {
-    if ((keep >> i) & 1u) {
-      const float h = f64_head(z[i]);
-      ok = ok && h - t32 > (fabsf(h) + fabsf(t32)) * 0x1.0p-21f + 0x1.0p-120f;
-    } else {
-      ok = ok && t32 - zf[i] > er[i] + fabsf(t32) * 0x1.0p-21f;
-    }
-  }
-  if (ok) return;
-  // the plain path: every phase, the iteration in binary64 (proj_box)
-  s = 0.0;
-#pragma unroll
-  for (int i = 0; i < N; ++i) {
-    value(i);
-    s += z[i];
-  }
-  keep = (1u << N) - 1u;
-  theta = (s - 1.0) * rcp_small<double>(N);
-#pragma unroll 1
-  for (int pass = 1; pass < N; ++pass) {
-    unsigned drop = 0;
-#pragma unroll
-    for (int i = 0; i < N; ++i)
-      if (((keep >> i) & 1u) && z[i] - theta <= 0.0) drop |= 1u << i;
-    if (!drop || drop == keep) break;
-    keep &= ~drop;
-    s = 0.0;
-#pragma unroll
-    for (int i = 0; i < N; ++i)
-      if ((keep >> i) & 1u) s += z[i];
-    theta = (s - 1.0) * rcp_small<double>(__popc(keep));
-  }
+  fixed_simplex<N, kFixZ>(z, keep, theta);
+  return !bad;
 }
 
 // P1 interpolation weight of coarse node L at fine node b (fine coordinates),

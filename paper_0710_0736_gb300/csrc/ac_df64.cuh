@@ -77,6 +77,15 @@ AC_HD float fma_f32(float a, float b, float c) {
 #endif
 }
 
+// a b rounded, never fused with what follows.
+AC_HD double mul_f64(double a, double b) {
+#ifdef __CUDA_ARCH__
+  return __dmul_rn(a, b);
+#else
+  return a * b;
+#endif
+}
+
 AC_HD bool f64_isnan(double d) {
   uint32_t hi, lo;
   f64_words(d, hi, lo);
@@ -185,7 +194,7 @@ AC_HD f2 fast_two_sum(float a, float b) {
 AC_HD f2 mul_f2(float ah, float al, float bh, float bl) {
   const float p = ah * bh;
   const float e = fma_f32(ah, bh, -p);
-  return {p, e + (ah * bl + al * bh)};
+  return {p, e + fma_f32(ah, bl, al * bh)};
 }
 
 // (a.h + a.l) + (bh + bl): one two-sum on the heads, the tails added in
@@ -290,7 +299,7 @@ AC_HD int outer_update_node(double (&uk)[N], const float (&dk)[N], AnyOr any_or)
 #pragma unroll
     for (int i = 0; i < N; ++i)
       if (((anyk >> i) & 1u) && ((keep >> i) & 1u)) s += uk[i];
-    theta = (s - 1.0) * rcp_count<double>(popcount_hd(keep));
+    theta = mul_f64(s - 1.0, rcp_count<double>(popcount_hd(keep)));
     const float t32 = f64_head(theta);
 #pragma unroll
     for (int i = 0; i < N; ++i)
@@ -305,7 +314,7 @@ AC_HD int outer_update_node(double (&uk)[N], const float (&dk)[N], AnyOr any_or)
 #pragma unroll
     for (int i = 0; i < N; ++i)
       if (((any0 >> i) & 1u) && ((keep >> i) & 1u)) s += uk[i];
-    theta = (s - 1.0) * rcp_count<double>(cnt);
+    theta = mul_f64(s - 1.0, rcp_count<double>(cnt));
 #pragma unroll 1
     for (int pass = 1; pass < N; ++pass) {
       unsigned drop = 0;
@@ -318,7 +327,7 @@ AC_HD int outer_update_node(double (&uk)[N], const float (&dk)[N], AnyOr any_or)
 #pragma unroll
       for (int i = 0; i < N; ++i)
         if (((any0 >> i) & 1u) && ((keep >> i) & 1u)) s += uk[i];
-      theta = (s - 1.0) * rcp_count<double>(popcount_hd(keep));
+      theta = mul_f64(s - 1.0, rcp_count<double>(popcount_hd(keep)));
     }
   }
   const unsigned anyf = any_or(keep);
@@ -326,6 +335,92 @@ AC_HD int outer_update_node(double (&uk)[N], const float (&dk)[N], AnyOr any_or)
   for (int i = 0; i < N; ++i)
     uk[i] = (((anyf >> i) & 1u) && ((keep >> i) & 1u)) ? uk[i] - theta : 0.0;
   return ok ? 0 : 1;
+}
+
+// ---- 64-bit fixed point -------------------------------------------------------
+// Values of the Gibbs simplex are at most 1, so sums, comparisons and the
+// projection's threshold can run on the integer pipe: v 2^F as a 64-bit
+// integer, F = 60 for phase values (exact from 2^-7 up, within 2^-61 below;
+// binary64 rounds a sum near 1 to 2^-53) and F = 57 for the nodal problem's z
+// (rounded to 2^-58; |z| < 4 leaves room for a sum of 8).
+
+AC_HD uint64_t f64_bits(double d) {
+  uint32_t hi, lo;
+  f64_words(d, hi, lo);
+  return ((uint64_t)hi << 32) | lo;
+}
+
+// |d| 2^F rounded to nearest (halves up), with d's sign; bad is set for |d| >=
+// 2^LIM, infinities and NaN (the value is then meaningless).
+template <int F, int LIM>
+AC_HD int64_t f64_to_fix(double d, bool &bad) {
+  static_assert(F + LIM <= 62, "room for the sign and the rounding");
+  const uint64_t b = f64_bits(d);
+  const int e = (int)(b >> 52) & 0x7FF;
+  bad = bad || e >= 1023 + LIM;
+  // the significand in 63 bits: |d| = m 2^(e - 1023 - 62)
+  const uint64_t m = ((b & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull) << 10;
+  int sh = 1084 - F - e;  // one bit short of the shift, for the rounding
+  sh = sh < 0 ? 0 : (sh > 63 ? 63 : sh);
+  const int64_t v = (int64_t)(((m >> sh) + 1u) >> 1);
+  return (int64_t)b < 0 ? -v : v;
+}
+
+AC_HD int clz64(uint64_t v) {
+#ifdef __CUDA_ARCH__
+  return __clzll((long long)v);
+#else
+  return __builtin_clzll(v);
+#endif
+}
+
+// v 2^-F for v >= 0, rounded to nearest (halves up).
+template <int F>
+AC_HD double fix_to_f64(int64_t v) {
+  if (v == 0) return 0.0;
+  const int lz = clz64((uint64_t)v);
+  const uint64_t m = (uint64_t)v << lz;  // leading bit at 63
+  const uint64_t b = ((uint64_t)(1022 + 63 - F - lz) << 52) + (m >> 11) + ((m >> 10) & 1u);
+  return words_f64((uint32_t)(b >> 32), (uint32_t)b);
+}
+
+// s / k rounded to nearest (within 2^-1 + |s| 2^-64 of it), for k = 1 .. 8.
+AC_HD int64_t div_small(int64_t s, int k) {
+  s += k >> 1;
+  if ((k & (k - 1)) == 0) return s >> (k == 1 ? 0 : k == 2 ? 1 : k == 4 ? 2 : 3);
+  const uint64_t r = k == 3 ? 0x5555555555555556ull : k == 5 ? 0x3333333333333334ull
+                   : k == 6 ? 0x2AAAAAAAAAAAAAABull : 0x2492492492492493ull;  // 2^64 / k, rounded up
+#ifdef __CUDA_ARCH__
+  return __mul64hi(s, (long long)r);
+#else
+  return (int64_t)(((__int128)s * (__int128)(int64_t)r) >> 64);
+#endif
+}
+
+// Michelot's iteration (proj_box) for target sum 1: the kept set and the
+// threshold theta of z's projection onto the simplex, all in units of 2^-F:
+// x_i = z_i - theta on the kept set, 0 elsewhere.  Exact but for theta's
+// division.
+template <int N, int F>
+AC_HD void fixed_simplex(const int64_t (&z)[N], unsigned &keep, int64_t &theta) {
+  keep = (1u << N) - 1u;
+  int64_t s = -((int64_t)1 << F);
+#pragma unroll
+  for (int i = 0; i < N; ++i) s += z[i];
+  theta = div_small(s, N);
+#pragma unroll 1
+  for (int pass = 1; pass < N; ++pass) {
+    unsigned drop = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i)
+      if (((keep >> i) & 1u) && z[i] <= theta) {
+        drop |= 1u << i;
+        s -= z[i];
+      }
+    if (!drop) break;
+    keep &= ~drop;
+    theta = div_small(s, popcount_hd(keep));
+  }
 }
 
 }  // namespace ac

@@ -978,38 +978,36 @@ __global__ void k_outer_update(double *__restrict__ u, const float *__restrict__
 template <typename T, int N, int FORM>
 __device__ __forceinline__ void smooth_node(const T *x, const T *__restrict__ rhs, const T *__restrict__ ob,
                                             const T *__restrict__ corr, const double *__restrict__ omega,
-                                            const Geo &g, int xx, int y, int64_t n, const uint8_t *mask, T (&acc)[N],
-                                            T (&o)[N]) {
+                                            const Geo &g, int xx, int y, int64_t n, T (&acc)[N], T (&o)[N]) {
   T bk[N];
-  // FP64 direct form: phases the projection drops need no binary64 at all
-  bool plain = true;
-  if constexpr (kFilter64<T, FORM>) plain = many_free64<N>(mask[(int64_t)y * g.Wn + xx]);
-  if (plain) {
-    nbr_sum<T, N>(x, g, xx, y, acc);
-    if (corr) {
-      const T w = omega_t<T>(omega);
-      if (w != T(0)) {
-        T dc[N];
-        nbr_sum<T, N>(corr, g, xx, y, dc);
-#pragma unroll
-        for (int i = 0; i < N; ++i) acc[i] += w * dc[i];
-      }
-    }
+  if constexpr (kFixed64<T, FORM>) {
     ldn<T, N>(rhs + n * N, bk);
-    if constexpr (FORM != kDirect) ldn<T, N>(ob + n * N, o);
-    const int cls = node_class(g, xx, y);
-    const T te = geo_te<T>(g), invD = geo_invD<T>(g, cls);
-#pragma unroll
-    for (int i = 0; i < N; ++i) acc[i] = (bk[i] + te * acc[i]) * invD;
-    proj_box<T, N, FORM>(acc, o);
-  } else if constexpr (kFilter64<T, FORM>) {
-    ldn<T, N>(rhs + n * N, bk);
-    double q[N], z[N], theta;
+    double q[N];
+    int64_t z[N], theta;
     unsigned keep;
-    direct_node64<N>(x, corr, corr ? omega[0] : 0.0, bk, g, xx, y, 0u, q, z, keep, theta);
+    if (direct_node_fixed<N>(x, corr, corr ? omega[0] : 0.0, bk, g, xx, y, q, z, keep, theta)) {
 #pragma unroll
-    for (int i = 0; i < N; ++i) acc[i] = ((keep >> i) & 1u) ? z[i] - theta : 0.0;
+      for (int i = 0; i < N; ++i) acc[i] = ((keep >> i) & 1u) ? fix_to_f64<kFixZ>(z[i] - theta) : 0.0;
+      return;
+    }
   }
+  nbr_sum<T, N>(x, g, xx, y, acc);
+  if (corr) {
+    const T w = omega_t<T>(omega);
+    if (w != T(0)) {
+      T dc[N];
+      nbr_sum<T, N>(corr, g, xx, y, dc);
+#pragma unroll
+      for (int i = 0; i < N; ++i) acc[i] = fma_rn(w, dc[i], acc[i]);
+    }
+  }
+  ldn<T, N>(rhs + n * N, bk);
+  if constexpr (FORM != kDirect) ldn<T, N>(ob + n * N, o);
+  const int cls = node_class(g, xx, y);
+  const T te = geo_te<T>(g), invD = geo_invD<T>(g, cls);
+#pragma unroll
+  for (int i = 0; i < N; ++i) acc[i] = mul_rn(fma_rn(te, acc[i], bk[i]), invD);
+  proj_box<T, N, FORM>(acc, o);
 }
 
 // The free mask of a node value: the phases above their bound (direct,
@@ -1052,7 +1050,7 @@ __global__ void __launch_bounds__(kBlock) k_smooth_fine(T *__restrict__ x, const
   // the mask byte this pass replaces, loaded first so its latency overlaps
   const uint8_t old_mask = (MASK && dirty.p) ? mask[(int64_t)y * g.Wn + xx] : (uint8_t)0;
   T acc[N], o[N];
-  smooth_node<T, N, FORM>(x, rhs, ob, corr, omega, g, xx, y, n, mask, acc, o);
+  smooth_node<T, N, FORM>(x, rhs, ob, corr, omega, g, xx, y, n, acc, o);
   stn<T, N>(x + n * N, acc);
   if constexpr (MASK) {
     store_mask(mask, dirty, g, xx, y, old_mask, free_mask<T, N, FORM>(acc, o));
@@ -1085,41 +1083,44 @@ __device__ __forceinline__ T resid_node(const T *__restrict__ x, const T *__rest
   // the mask byte this kernel replaces, loaded first so its latency overlaps
   const uint8_t old_mask = (rt && dirty.p) ? mask[n] : (uint8_t)0;
   T acc[N], xk[N], bk[N], r[N], o[N];
-  if constexpr (!kFilter64<T, FORM>) nbr_sum<T, N>(x, g, xx, y, acc);
+  if constexpr (!kFixed64<T, FORM>) nbr_sum<T, N>(x, g, xx, y, acc);
   ldn<T, N>(x + sl * N, xk);
   ldn<T, N>(rhs + sl * N, bk);
   const int cls = node_class(g, xx, y);
   const T D = geo_D<T>(g, cls);
+  T e = T(0);
   bool plain = true;
-  if constexpr (kFilter64<T, FORM>) plain = !mask || many_free64<N>(mask[n]);
+  if constexpr (kFixed64<T, FORM>) {
+    int64_t z[N], theta;
+    unsigned keep;
+    bool bad = false;
+    plain = !direct_node_fixed<N>(x, nullptr, 0.0, bk, g, xx, y, r, z, keep, theta);
+    // |x - P(z)| in fixed point; r (q so far) is wanted where x > 0 only
+    int64_t far = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) {
+      const int64_t p = ((keep >> i) & 1u) ? z[i] - theta : 0, f = f64_to_fix<kFixZ, 2>(xk[i], bad) - p;
+      far = max(far, f < 0 ? -f : f);
+      r[i] = xk[i] > 0.0 ? fma_rn(-D, xk[i], r[i]) : 0.0;
+    }
+    e = fix_to_f64<kFixZ>(far);
+    plain = plain || bad;
+  }
   if (plain) {
-    if constexpr (kFilter64<T, FORM>) nbr_sum<T, N>(x, g, xx, y, acc);
+    if constexpr (kFixed64<T, FORM>) nbr_sum<T, N>(x, g, xx, y, acc);
     if constexpr (FORM != kDirect) ldn<T, N>(ob + sl * N, o);
     const T invD = geo_invD<T>(g, cls), te = geo_te<T>(g);
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-      r[i] = bk[i] + te * acc[i] - D * xk[i];
-      acc[i] = (bk[i] + te * acc[i]) * invD;
+      const T q = fma_rn(te, acc[i], bk[i]);
+      r[i] = fma_rn(-D, xk[i], q);
+      acc[i] = mul_rn(q, invD);
     }
     proj_box<T, N, FORM>(acc, o);
-  } else if constexpr (kFilter64<T, FORM>) {
-    // the residual is wanted on the phases above 0, the projection on those
-    // it keeps; elsewhere x and P(z) are both 0
-    unsigned above = 0u, keep;
+    e = T(0);
 #pragma unroll
-    for (int i = 0; i < N; ++i) above |= xk[i] > 0.0 ? 1u << i : 0u;
-    double q[N], z[N], theta;
-    direct_node64<N>(x, nullptr, 0.0, bk, g, xx, y, above, q, z, keep, theta);
-    const unsigned any = __reduce_or_sync(__activemask(), above | keep);
-#pragma unroll
-    for (int i = 0; i < N; ++i) {
-      r[i] = ((any >> i) & 1u) && ((above >> i) & 1u) ? q[i] - D * xk[i] : 0.0;
-      acc[i] = ((any >> i) & 1u) && ((keep >> i) & 1u) ? z[i] - theta : 0.0;
-    }
+    for (int i = 0; i < N; ++i) e = nanmax<T>(e, fabs(xk[i] - acc[i]));
   }
-  T e = T(0);
-#pragma unroll
-  for (int i = 0; i < N; ++i) e = nanmax<T>(e, fabs(xk[i] - acc[i]));
   if (!(xk[0] == xk[0])) e = xk[0];
   if (rt) {
     const unsigned fr = free_mask<T, N, FORM>(xk, o);
@@ -1128,7 +1129,7 @@ __device__ __forceinline__ T resid_node(const T *__restrict__ x, const T *__rest
 #pragma unroll
     for (int i = 0; i < N; ++i)
       if ((fr >> i) & 1u) s += r[i];
-    const T mean = fr ? s * rcp_small<T>(__popc(fr)) : T(0);
+    const T mean = fr ? mul_rn(s, rcp_small<T>(__popc(fr))) : T(0);
 #pragma unroll
     for (int i = 0; i < N; ++i) r[i] = ((fr >> i) & 1u) ? r[i] - mean : T(0);
     stn<T, N>(rt + sl * N, r);
@@ -1282,7 +1283,7 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 4 : 1)
       const uint8_t old_mask = (MASK && dirty.p) ? mask[(int64_t)y * g.Wn + xx] : (uint8_t)0;
       T acc[N], o[N], old[N];
       if constexpr (MASK) ldn_rw<T, N>(x + n * N, old);
-      smooth_node<T, N, FORM>(x, rhs, ob, corr, omega, g, xx, y, n, mask, acc, o);
+      smooth_node<T, N, FORM>(x, rhs, ob, corr, omega, g, xx, y, n, acc, o);
       stn<T, N>(x + n * N, acc);
       if constexpr (MASK) {
         // a NaN counts as a change; the sign of a zero does not (no result depends on it)
