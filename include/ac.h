@@ -119,7 +119,7 @@ enum {
   AC_PROF_SMOOTH = 0,  /* fine red-black projected Gauss-Seidel, one launch per colour */
   AC_PROF_RESID,       /* fine residual, natural residual, mask, tangent projection */
   AC_PROF_COARSE,      /* coarse-level smoothing, residuals and coarsest solve */
-  AC_PROF_TRANSFER,    /* truncated Galerkin operators, restriction, prolongation */
+  AC_PROF_TRANSFER,    /* truncated Galerkin operators, restriction */
   AC_PROF_LINESEARCH,  /* coarse-correction direction, line search, update */
   AC_PROF_SETUP,       /* colour means, energy and right-hand side of a step */
   AC_PROF_OUTER,       /* AC_MIXED: residual and update of the defect correction */

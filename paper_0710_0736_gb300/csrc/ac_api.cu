@@ -658,7 +658,7 @@ int coarse_vcycle(ac_ctx *ctx, Solve &S, int k, void **res) {
     // the coarsest level (a Gauss-Seidel sweep is worth two of l1-Jacobi)
     const int sweeps = !ends_dominated(S) ? kCoarsestSweeps : S.coarse_gs ? kDominatedSweeps : 2 * kDominatedSweeps;
     AC_RUNB(AC_PROF_COARSE, pair0 + (sweeps / 2 - 1) * pair,
-            o->coarse_smooth(L.op, L.r, L.v, L.t, L.g, sweeps, true, res, nullptr, S.coarse_gs, ctx->s));
+            o->coarse_smooth(L.op, L.r, L.v, L.t, L.g, sweeps, true, nullptr, L.g, res, nullptr, S.coarse_gs, ctx->s));
     return AC_OK;
   }
   Level &C = S.lv[k + 1];
@@ -674,7 +674,8 @@ int coarse_vcycle(ac_ctx *ctx, Solve &S, int k, void **res) {
     other = L.t;
   } else {
     AC_RUNB(AC_PROF_COARSE, pair0 + (kCoarseSweeps / 2 - 1) * pair,
-            o->coarse_smooth(L.op, L.r, L.v, L.t, L.g, kCoarseSweeps, true, &v, tf, S.coarse_gs, ctx->s));
+            o->coarse_smooth(L.op, L.r, L.v, L.t, L.g, kCoarseSweeps, true, nullptr, L.g, &v, tf, S.coarse_gs,
+                             ctx->s));
     other = v == L.v ? L.t : L.v;
     AC_RUNB(AC_PROF_COARSE, 7 * lk, o->coarse_resid(L.op, L.r, v, L.g, other, tf, ctx->s));
   }
@@ -683,10 +684,9 @@ int coarse_vcycle(ac_ctx *ctx, Solve &S, int k, void **res) {
   void *cv = nullptr;
   int rc = coarse_vcycle(ctx, S, k + 1, &cv);
   if (rc) return rc;
-  // prolongation: coarse v and this level's diagonal read, v read and written
-  AC_RUNB(AC_PROF_TRANSFER, lc + 3 * lk, o->prolong_add(cv, L.g, C.g, L.op, v, tf, ctx->s));
-  AC_RUNB(AC_PROF_COARSE, (kCoarseSweeps / 2) * pair,
-          o->coarse_smooth(L.op, L.r, v, other, L.g, kCoarseSweeps, false, res, tf, S.coarse_gs, ctx->s));
+  // the first pair also reads the coarse v and adds its prolongation
+  AC_RUNB(AC_PROF_COARSE, lc + (kCoarseSweeps / 2) * pair,
+          o->coarse_smooth(L.op, L.r, v, other, L.g, kCoarseSweeps, false, cv, C.g, res, tf, S.coarse_gs, ctx->s));
   return AC_OK;
 }
 

@@ -2034,9 +2034,30 @@ __device__ __forceinline__ void tile_zero(const Geo &g, int tx, int ty, T *__res
   }
 }
 
+// The coarser level's correction vc of one phase, prolonged to node (x, y) of
+// the finer level (P1 on the nested right-diagonal meshes, as prolong_at).
+// The post-smoothing pair adds it to the iterate while it loads its tile: as
+// a kernel of its own it read and wrote that iterate once more and was one
+// of four launches of a level (1024^2, N = 4: 2.11 -> 2.05 ms a pass; 4096^2,
+// N = 8 from a random start: 46.5 -> 45.5).  Added on rows with a
+// zero diagonal too: their update gives 0 and their coefficients are 0.
+// In binary64 warps whose coarse values are all 0 (settled phases) leave the
+// two slow operations out.
+template <typename T>
+__device__ __forceinline__ T add_prolonged(T v, const T *vc, int Wnc, int x, int y) {
+  const int64_t K0 = (int64_t)(y >> 1) * Wnc + (x >> 1);
+  const bool mid = ((x | y) & 1) != 0;
+  const T a = vc[K0], b = vc[K0 + (x & 1) + (int64_t)(y & 1) * Wnc];
+  if constexpr (sizeof(T) == 8) {
+    if (((__double_as_longlong(a) | __double_as_longlong(b)) & 0x7fffffffffffffffll) == 0) return v;
+  }
+  return v + (mid ? T(0.5) * (a + b) : a);
+}
+
 template <typename T, int N, bool ZERO_IN>
 __device__ __forceinline__ void jacobi2_tile(const T *__restrict__ op, const T *__restrict__ r, const T *vin,
-                                             T *vout, const Geo &g, int bxt, int byt, int i) {
+                                             T *vout, const T *vc, const Geo &g, const Geo &gc, int bxt, int byt,
+                                             int i) {
   constexpr int AX = kJ2X + 4, AY = kJ2Y + 4;  // tile + halo 2
   constexpr int BX = kJ2X + 2, BY = kJ2Y + 2;  // tile + halo 1
   __shared__ T sC[AY][AX], sE[AY][AX], sN[AY][AX], sNE[AY][AX], sV[AY][AX];
@@ -2044,6 +2065,7 @@ __device__ __forceinline__ void jacobi2_tile(const T *__restrict__ op, const T *
   const int64_t nc = (int64_t)g.Wn * (g.H + 1);
   const T *C = op + (0 * N + i) * nc, *E = op + (1 * N + i) * nc, *Nn = op + (2 * N + i) * nc,
           *NE = op + (3 * N + i) * nc, *ri = r + i * nc, *vi = vin + i * nc;
+  const T *vci = !ZERO_IN && vc ? vc + i * (int64_t)gc.Wn * (gc.H + 1) : nullptr;
   T *vo = vout + i * nc;
   const int x0 = bxt * kJ2X - 2, y0 = byt * kJ2Y - 2;  // grid position of [0][0] of the A arrays
   // A tile whose rows all have a zero diagonal (no free fine node of this
@@ -2071,7 +2093,9 @@ __device__ __forceinline__ void jacobi2_tile(const T *__restrict__ op, const T *
     sE[ay][ax] = in ? E[K] : T(0);
     sN[ay][ax] = in ? Nn[K] : T(0);
     sNE[ay][ax] = in ? NE[K] : T(0);
-    sV[ay][ax] = (!ZERO_IN && in) ? vi[K] : T(0);
+    T v = (!ZERO_IN && in) ? vi[K] : T(0);
+    if (!ZERO_IN && in && vci) v = add_prolonged(v, vci, gc.Wn, x, y);
+    sV[ay][ax] = v;
   }
   for (int t = threadIdx.x; t < BX * BY; t += kJ2Threads) {
     const int bx = t % BX, by = t / BX, x = x0 + 1 + bx, y = y0 + 1 + by;
@@ -2160,7 +2184,8 @@ struct GsShape {
 
 template <typename T, int N, int MODE, bool INTERIOR>
 __device__ __forceinline__ void gs_tile_body(const T *__restrict__ op, const T *__restrict__ r, const T *vin, T *vout,
-                                             T *__restrict__ tout, const Geo &g, int i, int xs, int ys,
+                                             T *__restrict__ tout, const T *vc, int Wnc, const Geo &g, int i, int xs,
+                                             int ys,
                                              T (&sV)[GsShape<MODE>::AY][GsShape<MODE>::AX]) {
   using S = GsShape<MODE>;
   constexpr int H1 = S::H1, W1 = S::W1, R1 = S::R1, X1 = S::X1, AX = S::AX, AY = S::AY;
@@ -2210,8 +2235,10 @@ __device__ __forceinline__ void gs_tile_body(const T *__restrict__ op, const T *
   for (int t = threadIdx.x; t < AX * AY; t += kGsThreads) {
     const int bx = t % AX, by = t / AX, gx = xs + bx, gy = ys + by;
     T v = T(0);
-    if (MODE == kGsPost && (INTERIOR || (gx >= 0 && gx <= g.W && gy >= 0 && gy <= g.H)))
+    if (MODE == kGsPost && (INTERIOR || (gx >= 0 && gx <= g.W && gy >= 0 && gy <= g.H))) {
       v = vi[(int64_t)gy * g.Wn + gx];
+      if (sizeof(T) == 4 && vc) v = add_prolonged(v, vc, Wnc, gx, gy);
+    }
     sV[by][bx] = v;
   }
   int live = 0;
@@ -2229,6 +2256,18 @@ __device__ __forceinline__ void gs_tile_body(const T *__restrict__ op, const T *
         if (MODE == kGsPreResid) tout[i * nc + K0 + q] = T(0);
       }
     return;
+  }
+  if constexpr (sizeof(T) == 8 && MODE == kGsPost) {
+    // in live tiles only: adding while loading, as in float, cost the tiles
+    // without one more than it gave (1024^2, N = 4 formed: 3.22 -> 3.29 ms)
+    if (vc) {
+      for (int t = threadIdx.x; t < AX * AY; t += kGsThreads) {
+        const int bx = t % AX, by = t / AX, gx = xs + bx, gy = ys + by;
+        if (INTERIOR || (gx >= 0 && gx <= g.W && gy >= 0 && gy <= g.H))
+          sV[by][bx] = add_prolonged(sV[by][bx], vc, Wnc, gx, gy);
+      }
+      __syncthreads();
+    }
   }
   T *const sv = &sV[owner ? cy : 1][cx0];  // node 0 of the thread's triplet (read only by owners)
 #define AC_GS_UPDATE(q)                                          \
@@ -2274,16 +2313,18 @@ __device__ __forceinline__ void gs_tile_body(const T *__restrict__ op, const T *
 
 template <typename T, int N, int MODE>
 __device__ __forceinline__ void gs_tile_rt(const T *__restrict__ op, const T *__restrict__ r, const T *vin, T *vout,
-                                           T *__restrict__ tout, const Geo &g, int bxt, int byt, int i) {
+                                           T *__restrict__ tout, const T *vc, const Geo &g, const Geo &gc, int bxt,
+                                           int byt, int i) {
   using S = GsShape<MODE>;
   __shared__ T sV[S::AY][S::AX];
   const int xs = bxt * kJ2X - S::H1 - S::X1, ys = byt * kJ2Y - S::H1 - 1;
+  const T *vci = MODE == kGsPost && vc ? vc + i * (int64_t)gc.Wn * (gc.H + 1) : nullptr;
   // every node the block can read: columns xs - 1 .. xs + AX - 1 (a west
   // neighbour of the first triplet), rows ys - 1 .. ys + AY - 1
   if (xs >= 1 && xs + S::AX <= g.W && ys >= 1 && ys + S::AY <= g.H)
-    gs_tile_body<T, N, MODE, true>(op, r, vin, vout, tout, g, i, xs, ys, sV);
+    gs_tile_body<T, N, MODE, true>(op, r, vin, vout, tout, vci, gc.Wn, g, i, xs, ys, sV);
   else
-    gs_tile_body<T, N, MODE, false>(op, r, vin, vout, tout, g, i, xs, ys, sV);
+    gs_tile_body<T, N, MODE, false>(op, r, vin, vout, tout, vci, gc.Wn, g, i, xs, ys, sV);
 }
 
 // (the register bound keeps as many blocks per SM as the shared memory
@@ -2296,19 +2337,21 @@ constexpr int j2_min_blocks(int elem) { return elem == 4 ? 8 : 5; }
 #endif
 constexpr int pair_min_blocks(int elem, bool gs) { return gs ? (elem == 4 ? AC_GS_BLOCKS : 2) : j2_min_blocks(elem); }
 // Two smoothing sweeps per tile of a coarse level: 3-colour Gauss-Seidel
-// (GS) or l1-Jacobi.
+// (GS) or l1-Jacobi.  vc (nullable, grid gc): the coarser level's correction,
+// added to vin first.
 template <typename T, int N, bool ZERO_IN, bool GS>
 __global__ void __launch_bounds__(GS ? kGsThreads : kJ2Threads, pair_min_blocks(sizeof(T), GS)) k_coarse_pair(const T *__restrict__ op, const T *__restrict__ r,
-                                                                  const T *vin, T *vout, Geo g, TileList L) {
+                                                                  const T *vin, T *vout, const T *vc, Geo g, Geo gc,
+                                                                  TileList L) {
   pdl_sync();
   for_each_tile(L, g, [&](int tx, int ty, int i, bool dying) {
     const int64_t nc = (int64_t)g.Wn * (g.H + 1);
     if (dying)
       tile_zero<T>(g, tx, ty, vout + i * nc, (T *)nullptr);
     else if constexpr (GS)
-      gs_tile_rt<T, N, ZERO_IN ? kGsZero : kGsPost>(op, r, vin, vout, (T *)nullptr, g, tx, ty, i);
+      gs_tile_rt<T, N, ZERO_IN ? kGsZero : kGsPost>(op, r, vin, vout, (T *)nullptr, vc, g, gc, tx, ty, i);
     else
-      jacobi2_tile<T, N, ZERO_IN>(op, r, vin, vout, g, tx, ty, i);
+      jacobi2_tile<T, N, ZERO_IN>(op, r, vin, vout, vc, g, gc, tx, ty, i);
   });
 }
 
@@ -2422,7 +2465,7 @@ __global__ void __launch_bounds__(GS ? kGsThreads : kJ2Threads, pair_min_blocks(
     if (dying)
       tile_zero<T>(g, tx, ty, vout + i * nc, tout + i * nc);
     else if constexpr (GS)
-      gs_tile_rt<T, N, kGsPreResid>(op, r, (const T *)nullptr, vout, tout, g, tx, ty, i);
+      gs_tile_rt<T, N, kGsPreResid>(op, r, (const T *)nullptr, vout, tout, (const T *)nullptr, g, g, tx, ty, i);
     else
       jacobi2_resid_tile<T, N>(op, r, vout, tout, g, tx, ty, i);
   });
@@ -2804,61 +2847,6 @@ __device__ __forceinline__ void prolong_at(const T *vc, const Geo &gc, int x, in
   const int64_t K1 = K0 + (x & 1) + (int64_t)(y & 1) * gc.Wn;
 #pragma unroll
   for (int i = 0; i < N; ++i) o[i] = T(0.5) * (o[i] + vc[i * nc + K1]);
-}
-
-// v_f += P v_c (coarse levels, phase-major), the arithmetic of prolong_at.
-// PHASES_IN_Z: one thread per (node, phase), phase = blockIdx.z (narrow
-// levels, where latency dominates); otherwise one thread per node doing all
-// phases (wide levels, fewer blocks for the same bytes).  Rows of the fine
-// level's operator opf with a zero diagonal are skipped: the smoothing that
-// follows sets them to 0 whatever they hold (and their coefficients are 0),
-// and the pre-smoothing left them 0.
-template <typename T, int N, bool PHASES_IN_Z>
-__global__ void k_prolong_add(const T *__restrict__ vc, Geo gf, Geo gc, const T *__restrict__ opf,
-                              T *__restrict__ vf) {
-  pdl_sync();
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
-  if (x > gf.W) return;
-  const int64_t nc = (int64_t)gc.Wn * (gc.H + 1), nf = (int64_t)gf.Wn * (gf.H + 1);
-  const int64_t K0 = (int64_t)(y >> 1) * gc.Wn + (x >> 1), a = (int64_t)y * gf.Wn + x;
-  const bool mid = (x & 1) || (y & 1);
-  const int64_t K1 = K0 + (x & 1) + (int64_t)(y & 1) * gc.Wn;
-  constexpr int I = PHASES_IN_Z ? 1 : N;
-#pragma unroll
-  for (int j = 0; j < I; ++j) {
-    const int i = PHASES_IN_Z ? (int)blockIdx.z : j;
-    if (!(opf[i * nf + a] > T(0))) continue;
-    const T *vi = vc + i * nc;
-    T p = vi[K0];
-    if (mid) p = T(0.5) * (p + vi[K1]);
-    vf[i * nf + a] += p;
-  }
-}
-
-// The same onto a tiled level, driven by that level's list: the live tiles
-// only (a dying tile's v is 0 and stays 0, see kLiveNow).
-template <typename T, int N>
-__global__ void __launch_bounds__(kTileThreads) k_prolong_add_tiled(const T *__restrict__ vc, Geo gf, Geo gc,
-                                                                    const T *__restrict__ opf, T *__restrict__ vf,
-                                                                    TileList L) {
-  pdl_sync();
-  for_each_tile(L, gf, [&](int tx, int ty, int i, bool dying) {
-    if (dying) return;
-    const int64_t nc = (int64_t)gc.Wn * (gc.H + 1), nf = (int64_t)gf.Wn * (gf.H + 1);
-    const int x = tx * kJ2X + (int)(threadIdx.x % kJ2X);
-    const T *vi = vc + i * nc;
-#pragma unroll
-    for (int q = 0; q < kTileRows; ++q) {
-      const int y = ty * kJ2Y + (int)(threadIdx.x / kJ2X) + q * (kTileThreads / kJ2X);
-      if (x > gf.W || y > gf.H) continue;
-      const int64_t a = (int64_t)y * gf.Wn + x;
-      if (!(opf[i * nf + a] > T(0))) continue;
-      const int64_t K0 = (int64_t)(y >> 1) * gc.Wn + (x >> 1);
-      T p = vi[K0];
-      if ((x & 1) || (y & 1)) p = T(0.5) * (p + vi[K0 + (x & 1) + (int64_t)(y & 1) * gc.Wn]);
-      vf[i * nf + a] += p;
-    }
-  });
 }
 
 // ---------------------------------------------------------------------------

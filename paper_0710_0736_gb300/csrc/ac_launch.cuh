@@ -17,9 +17,6 @@ struct PhaseLaunch {
   dim3 grid;
   unsigned block;
 };
-// Levels at least this large take the node-wide variant of the light
-// transfer kernels (one thread per node, all phases).
-constexpr int64_t kWideLevelNodes = 1 << 20;
 
 inline PhaseLaunch phase_grid(int count_per_row, int rows, int phases) {
   const unsigned b = count_per_row >= kBlock ? (unsigned)kBlock : (unsigned)(((count_per_row + 31) / 32) * 32);
@@ -162,8 +159,10 @@ struct SolverLaunch {
   }
   template <bool GS>
   static int coarse_smooth_t(const void *op, const void *r, void *v, void *tmp, const Geo &g, int sweeps,
-                             bool zero_start, void **out, const LevelLists *L, cudaStream_t s) {
+                             bool zero_start, const void *vc, const Geo &gc, void **out, const LevelLists *L,
+                             cudaStream_t s) {
     const TileList tf = item_list(L);
+    const T *corr = (const T *)vc;
     void *cur = v;
     int k = 0;
     for (int p = 0; p < sweeps / 2; ++p) {
@@ -171,13 +170,15 @@ struct SolverLaunch {
         // v is not read: the pair can write it
         constexpr int th = GS ? kGsThreads : kJ2Threads;
         const dim3 grid = tile_grid(g, L, N, k_coarse_pair<T, N, true, GS>, th);
-        launch(k_coarse_pair<T, N, true, GS>, grid, th, 0, s, (const T *)op, (const T *)r, (const T *)v, (T *)v, g, tf);
+        launch(k_coarse_pair<T, N, true, GS>, grid, th, 0, s, (const T *)op, (const T *)r, (const T *)v, (T *)v,
+               (const T *)nullptr, g, g, tf);
       } else {
         void *nxt = cur == v ? tmp : v;
         constexpr int th = GS ? kGsThreads : kJ2Threads;
         const dim3 grid = tile_grid(g, L, N, k_coarse_pair<T, N, false, GS>, th);
-        launch(k_coarse_pair<T, N, false, GS>, grid, th, 0, s, (const T *)op, (const T *)r, (const T *)cur, (T *)nxt, g,
-                                                            tf);
+        launch(k_coarse_pair<T, N, false, GS>, grid, th, 0, s, (const T *)op, (const T *)r, (const T *)cur, (T *)nxt,
+               corr, g, gc, tf);
+        corr = nullptr;
         cur = nxt;
       }
       ++k;
@@ -186,9 +187,10 @@ struct SolverLaunch {
     return k;
   }
   static int coarse_smooth(const void *op, const void *r, void *v, void *tmp, const Geo &g, int sweeps,
-                           bool zero_start, void **out, const LevelLists *L, bool gs, cudaStream_t s) {
-    return gs ? coarse_smooth_t<true>(op, r, v, tmp, g, sweeps, zero_start, out, L, s)
-              : coarse_smooth_t<false>(op, r, v, tmp, g, sweeps, zero_start, out, L, s);
+                           bool zero_start, const void *vc, const Geo &gc, void **out, const LevelLists *L, bool gs,
+                           cudaStream_t s) {
+    return gs ? coarse_smooth_t<true>(op, r, v, tmp, g, sweeps, zero_start, vc, gc, out, L, s)
+              : coarse_smooth_t<false>(op, r, v, tmp, g, sweeps, zero_start, vc, gc, out, L, s);
   }
   // two sweeps from v = 0, then t = r - S v; float: one fused launch (its
   // shared memory is over the static limit in double)
@@ -204,7 +206,8 @@ struct SolverLaunch {
     } else {
       constexpr int th = GS ? kGsThreads : kJ2Threads;
       const dim3 grid = tile_grid(g, L, N, k_coarse_pair<T, N, true, GS>, th);
-      launch(k_coarse_pair<T, N, true, GS>, grid, th, 0, s, (const T *)op, (const T *)r, (const T *)v, (T *)v, g, tf);
+      launch(k_coarse_pair<T, N, true, GS>, grid, th, 0, s, (const T *)op, (const T *)r, (const T *)v, (T *)v,
+             (const T *)nullptr, g, g, tf);
       return 1 + coarse_resid(op, r, v, g, t, L, s);
     }
   }
@@ -232,21 +235,6 @@ struct SolverLaunch {
     } else {
       const PhaseLaunch L = phase_grid(gc.W + 1, gc.H + 1, N);
       launch(k_restrict<T, N>, L.grid, L.block, 0, s, (const T *)t, gf, gc, (const T *)opc, (T *)rc);
-    }
-    return 1;
-  }
-  static int prolong_add(const void *vc, const Geo &gf, const Geo &gc, const void *opf, void *vf, const LevelLists *Lf,
-                         cudaStream_t s) {
-    if (Lf) {
-      launch(k_prolong_add_tiled<T, N>, list_grid(Lf, Lf->cap, k_prolong_add_tiled<T, N>, kTileThreads), kTileThreads, 0,
-                                  s, (const T *)vc, gf, gc, (const T *)opf, (T *)vf,
-                                                                  item_list(Lf));
-    } else if ((int64_t)(gf.W + 1) * (gf.H + 1) >= kWideLevelNodes) {
-      launch(k_prolong_add<T, N, false>, row_grid(gf.W + 1, gf.H + 1), kBlock, 0, s, (const T *)vc, gf, gc,
-                                                                                 (const T *)opf, (T *)vf);
-    } else {
-      const PhaseLaunch L = phase_grid(gf.W + 1, gf.H + 1, N);
-      launch(k_prolong_add<T, N, true>, L.grid, L.block, 0, s, (const T *)vc, gf, gc, (const T *)opf, (T *)vf);
     }
     return 1;
   }
@@ -301,7 +289,7 @@ struct SolverLaunch {
       sz = settled_zero;
     }
     return SolverOps{(int)sizeof(T), smooth,       resid,        ss, rs, sl, sz, restrict0,   galerkin0,   galerkin,   coarse_smooth,
-                     coarse_resid, coarse_pre_resid, restrict_, prolong_add, coarse_tail,
+                     coarse_resid, coarse_pre_resid, restrict_, coarse_tail,
                      line_search};
   }
 };

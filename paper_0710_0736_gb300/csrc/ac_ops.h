@@ -96,9 +96,11 @@ struct SolverOps {
   // `sweeps` (even) smoothing sweeps in fused pairs starting from v, using v
   // and tmp in turn; *out returns the buffer holding the result.  zero_start:
   // v = 0 on entry (it is then neither read nor needs clearing).  gs:
-  // 3-colour Gauss-Seidel on shared-memory tiles, else l1-Jacobi
+  // 3-colour Gauss-Seidel on shared-memory tiles, else l1-Jacobi.  vc
+  // (nullable; not with zero_start): the correction of the coarser grid gc,
+  // prolonged and added to v by the first pair
   int (*coarse_smooth)(const void *op, const void *r, void *v, void *tmp, const Geo &g, int sweeps, bool zero_start,
-                       void **out, const LevelLists *L, bool gs, cudaStream_t s);
+                       const void *vc, const Geo &gc, void **out, const LevelLists *L, bool gs, cudaStream_t s);
   int (*coarse_resid)(const void *op, const void *r, const void *v, const Geo &g, void *t, const LevelLists *L,
                       cudaStream_t s);
   // one pair of smoothing sweeps from v = 0, then t = r - S v
@@ -106,8 +108,6 @@ struct SolverOps {
                           bool gs, cudaStream_t s);
   int (*restrict_)(const void *t, const Geo &gf, const Geo &gc, const void *opc, void *rc, const LevelLists *Lc,
                    cudaStream_t s);
-  int (*prolong_add)(const void *vc, const Geo &gf, const Geo &gc, const void *opf, void *vf, const LevelLists *Lf,
-                     cudaStream_t s);
   // v of level k0 from r of level k0 by the whole cycle below it (see
   // TailArgs); smem bytes of dynamic shared memory per block
   int (*coarse_tail)(const TailArgs &a, const void *r0, void *v0, int coarse_sweeps, int coarsest_sweeps,
