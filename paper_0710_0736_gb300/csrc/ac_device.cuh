@@ -644,9 +644,16 @@ __device__ __forceinline__ T warp_sum(T v) {
   return v;
 }
 
-// max that propagates a NaN held in either argument.
+// max of non-negative values that propagates a NaN held in either argument.
+// Binary64 ones compare as unsigned bit patterns (a NaN of either sign is
+// above infinity): the ten comparisons of a warp's maximum were about half of
+// the binary64 instructions of the FP64 residual.
 template <typename T>
 __device__ __forceinline__ T nanmax(T a, T b) { return (a != a || b <= a) ? a : b; }
+template <>
+__device__ __forceinline__ double nanmax<double>(double a, double b) {
+  return (unsigned long long)__double_as_longlong(a) >= (unsigned long long)__double_as_longlong(b) ? a : b;
+}
 
 template <typename T>
 __device__ __forceinline__ T warp_nanmax(T v) {

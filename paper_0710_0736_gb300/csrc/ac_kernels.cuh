@@ -3054,48 +3054,82 @@ __global__ void k_adj_prepare(const double *__restrict__ up, const double *__res
 //   [2 + 3i + ch]  G_i = dL/dc_i = 2 tau lambda sum w_i (m1 - c_i m0)
 // and the moment gradients gm (dL/dm1 RGB, dL/dm2) accumulated in place:
 //   dL/dm2 += -tau lambda sum_i w_i,  dL/dm1 += 2 tau lambda sum_i w_i c_i.
+// Bound by the binary64 pipe (one warp instruction in about 26 cycles of an
+// SM): the constant factors are applied to the totals or formed once a block,
+// a block takes kAdjRows rows, so that its 2 + 3N warp sums (70 instructions
+// a warp at N = 4, as many as a row's nodes) are shared by as many nodes, and
+// a phase whose w is 0 in a whole warp is left out (every term has w as a
+// factor).  At 512^2, N = 4: 154 -> 82 us on a step from random phases (97 on
+// average of four steps).
+constexpr int kAdjRows = 4;
 template <int N>
 __global__ void __launch_bounds__(kBlock) k_adj_accum(const double *__restrict__ w, const double *__restrict__ u,
                                                       const double *__restrict__ up, const double *__restrict__ mom,
                                                       const double *__restrict__ c, Geo g, double tau, double eps,
                                                       double lam, double *__restrict__ gm, double *__restrict__ part) {
   pdl_sync();
+  // per phase: c (RGB), |c|^2
+  __shared__ double sc[N][4];
+  if (threadIdx.x < N) {
+    const double c0 = c[threadIdx.x * 3], c1 = c[threadIdx.x * 3 + 1], c2 = c[threadIdx.x * 3 + 2];
+    sc[threadIdx.x][0] = c0;
+    sc[threadIdx.x][1] = c1;
+    sc[threadIdx.x][2] = c2;
+    sc[threadIdx.x][3] = c0 * c0 + c1 * c1 + c2 * c2;
+  }
+  __syncthreads();
   double acc[2 + 3 * N];
 #pragma unroll
   for (int k = 0; k < 2 + 3 * N; ++k) acc[k] = 0.0;
-  const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
-  if (x <= g.W) {
-    const int64_t n = (int64_t)y * g.Wn + x;
-    const double m0 = g.m0[node_class(g, x, y)];
+  const int x = blockIdx.x * blockDim.x + threadIdx.x;
+  const double tl2 = 2.0 * tau * lam, tl = -tau * lam, k1 = -2.0 * tau / (eps * eps);
+#pragma unroll 1
+  for (int q = 0; q < kAdjRows; ++q) {
+    const int y = blockIdx.y * kAdjRows + q;
+    const bool in = x <= g.W && y <= g.H;
+    const int64_t n = in ? (int64_t)y * g.Wn + x : 0;
+    double wk[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) wk[i] = 0.0;
+    if (in) ldn<double, N>(w + n * N, wk);
+    unsigned on = 0;
+#pragma unroll
+    for (int i = 0; i < N; ++i) on |= (__double_as_longlong(wk[i]) << 1) != 0 ? 1u << i : 0u;
+    on = __reduce_or_sync(0xffffffffu, on);
+    if (!on || !in) continue;
+    const double m0 = g.m0[node_class(g, x, y)], km0 = k1 * m0;
     const double4 m = ld_mom(mom + n * 4);
-    double wk[N], uk[N], upk[N], nb[N];
-    ldn<double, N>(w + n * N, wk);
+    const Weights wt = edge_weights(g, x, y);
+    const double wsum = f32_to_f64(wt.e + wt.w + wt.n + wt.s);
+    double uk[N], upk[N], nb[N];
     ldn<double, N>(u + n * N, uk);
     ldn<double, N>(up + n * N, upk);
     nbr_sum<double, N>(up, g, x, y, nb);
-    const Weights wt = edge_weights(g, x, y);
-    const double wsum = (double)wt.e + (double)wt.w + (double)wt.n + (double)wt.s;
     double sw = 0.0, swc[3] = {0, 0, 0};
 #pragma unroll
     for (int i = 0; i < N; ++i) {
-      const double c0 = c[i * 3], c1 = c[i * 3 + 1], c2 = c[i * 3 + 2];
-      const double f = m.w - 2.0 * (c0 * m.x + c1 * m.y + c2 * m.z) + (c0 * c0 + c1 * c1 + c2 * c2) * m0;
-      acc[0] += wk[i] * (-tau * f);
-      acc[1] += wk[i] * m0 * uk[i] * (-2.0 * tau / (eps * eps)) - tau * wk[i] * (wsum * upk[i] - nb[i]);
-      acc[2 + 3 * i + 0] += 2.0 * tau * lam * wk[i] * (m.x - c0 * m0);
-      acc[2 + 3 * i + 1] += 2.0 * tau * lam * wk[i] * (m.y - c1 * m0);
-      acc[2 + 3 * i + 2] += 2.0 * tau * lam * wk[i] * (m.z - c2 * m0);
+      if (!((on >> i) & 1u)) continue;
+      const double c0 = sc[i][0], c1 = sc[i][1], c2 = sc[i][2];
+      const double f = (m.w - 2.0 * (c0 * m.x + c1 * m.y + c2 * m.z)) + sc[i][3] * m0;
+      acc[0] += wk[i] * f;
+      acc[1] += wk[i] * (km0 * uk[i] - tau * (wsum * upk[i] - nb[i]));
+      acc[2 + 3 * i + 0] += wk[i] * (m.x - c0 * m0);
+      acc[2 + 3 * i + 1] += wk[i] * (m.y - c1 * m0);
+      acc[2 + 3 * i + 2] += wk[i] * (m.z - c2 * m0);
       sw += wk[i];
       swc[0] += wk[i] * c0;
       swc[1] += wk[i] * c1;
       swc[2] += wk[i] * c2;
     }
     double *gk = gm + n * 4;
-    gk[0] += 2.0 * tau * lam * swc[0];
-    gk[1] += 2.0 * tau * lam * swc[1];
-    gk[2] += 2.0 * tau * lam * swc[2];
-    gk[3] += -tau * lam * sw;
+    gk[0] += tl2 * swc[0];
+    gk[1] += tl2 * swc[1];
+    gk[2] += tl2 * swc[2];
+    gk[3] += tl * sw;
   }
+  acc[0] *= -tau;
+#pragma unroll
+  for (int k = 2; k < 2 + 3 * N; ++k) acc[k] *= tl2;
   block_sum_store<2 + 3 * N>(acc, part + (int64_t)(blockIdx.y * gridDim.x + blockIdx.x) * (2 + 3 * N));
 }
 
@@ -3103,32 +3137,40 @@ __global__ void __launch_bounds__(kBlock) k_adj_accum(const double *__restrict__
 // dL/dm1 += sum_i G_i u^t_i / M_i (c_i = s_i/M_i); phases of zero mass kept
 // their previous mean and contribute no c-term.  G at tot[2 + 3i + ch], M_i at
 // mass[i].
+// The quotients by M_i are formed once a block: a division is some ten
+// binary64 instructions, and four a phase and node were most of the kernel
+// (512^2, N = 4: 147 -> 31 us).
 template <int N>
-__global__ void k_adj_back(const double *__restrict__ w, const double *__restrict__ u, const double *__restrict__ mom,
-                           const double *__restrict__ c, const double *__restrict__ tot,
-                           const double *__restrict__ mass, Geo g, double a1, double *__restrict__ gout,
-                           double *__restrict__ gm) {
+__global__ void __launch_bounds__(kBlock) k_adj_back(const double *__restrict__ w, const double *__restrict__ u,
+                                                     const double *__restrict__ mom, const double *__restrict__ c,
+                                                     const double *__restrict__ tot, const double *__restrict__ mass,
+                                                     Geo g, double a1, double *__restrict__ gout,
+                                                     double *__restrict__ gm) {
   pdl_sync();
+  // G_i,ch / M_i (0 for a phase without mass) and c_i,ch
+  __shared__ double sg[3 * N], sc[3 * N];
+  if (threadIdx.x < 3 * N) {
+    const double M = mass[threadIdx.x / 3];
+    sg[threadIdx.x] = M != 0.0 ? tot[2 + threadIdx.x] / M : 0.0;
+    sc[threadIdx.x] = M != 0.0 ? c[threadIdx.x] : 0.0;
+  }
+  __syncthreads();
   const int x = blockIdx.x * blockDim.x + threadIdx.x, y = blockIdx.y;
   if (x > g.W) return;
   const int64_t n = (int64_t)y * g.Wn + x;
-  const double m0 = g.m0[node_class(g, x, y)];
+  const double m0 = g.m0[node_class(g, x, y)], am0 = m0 * a1;
   const double4 m = ld_mom(mom + n * 4);
   double wk[N], uk[N], o[N], add[3] = {0, 0, 0};
   ldn<double, N>(w + n * N, wk);
   ldn<double, N>(u + n * N, uk);
 #pragma unroll
   for (int i = 0; i < N; ++i) {
-    double v = m0 * a1 * wk[i];
-    const double M = mass[i];
-    if (M != 0.0) {
-      const double G0 = tot[2 + 3 * i], G1 = tot[3 + 3 * i], G2 = tot[4 + 3 * i];
-      v += (G0 * (m.x - c[i * 3] * m0) + G1 * (m.y - c[i * 3 + 1] * m0) + G2 * (m.z - c[i * 3 + 2] * m0)) / M;
-      add[0] += G0 * uk[i] / M;
-      add[1] += G1 * uk[i] / M;
-      add[2] += G2 * uk[i] / M;
-    }
-    o[i] = v;
+    const double G0 = sg[3 * i], G1 = sg[3 * i + 1], G2 = sg[3 * i + 2];
+    o[i] = am0 * wk[i] +
+           (G0 * (m.x - sc[3 * i] * m0) + G1 * (m.y - sc[3 * i + 1] * m0) + G2 * (m.z - sc[3 * i + 2] * m0));
+    add[0] += G0 * uk[i];
+    add[1] += G1 * uk[i];
+    add[2] += G2 * uk[i];
   }
   stn<double, N>(gout + n * N, o);
   double *gk = gm + n * 4;

@@ -411,7 +411,7 @@ struct Launch {
   static int adj_accum(const double *w, const double *u, const double *up, const double *mom, const double *c,
                        const Geo &g, double tau, double eps, double lam, double *gm, double *part, double *tot,
                        double *scal, cudaStream_t s) {
-    const dim3 grid = row_grid(g.W + 1, g.H + 1);
+    const dim3 grid = row_grid(g.W + 1, (g.H + kAdjRows) / kAdjRows);
     const int blocks = (int)(grid.x * grid.y);
     launch(k_adj_accum<N>, grid, kBlock, 0, s, w, u, up, mom, c, g, tau, eps, lam, gm, part);
     launch(k_colsum, 2 + 3 * N, 1024, 0, s, part, blocks, 2 + 3 * N, tot);
