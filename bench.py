@@ -180,10 +180,11 @@ def job_rate(local_ms, local_units, world, device):
     ms_max = float(t.item())
     return float(u.item()) / (ms_max / 1e3), ms_max
 
-SMOOTH_TRAFFIC = {"sha256": "a0467499a47d6f0029c4ad9328b3cf2a61457a4359bf305310fac607d20c5941",
-                  "bytes_per_node": (201.543936e6 + 47.308032e6) / 4198401, "n_phases": 8, "precision": "mixed"}
+SMOOTH_TRAFFIC = {"sha256": "627a2a0ed9816f16703474bf13155d22f0973b4537cada4671a777f897cc310e",
+                  "bytes_per_node": (201.545728e6 + 47.035648e6) / 4198401, "n_phases": 8, "precision": "mixed"}
 SMOOTH_HELPERS = ("node_class", "edge_weights", "fslot", "geo_te", "geo_invD", "omega_t", "rcp_small", "proj_box",
-                  "nbr_sum", "ldn", "ldn_rw", "stn", "mark_dirty")
+                  "nbr_sum", "ldn", "ldn_rw", "stn", "mark_dirty", "fma_rn", "mul_rn")
+SMOOTH_KERNEL = ("k_smooth_fine", "smooth_node", "free_mask", "store_mask")
 
 
 def _function_text(src, name):
@@ -202,7 +203,8 @@ def smooth_source_digest():
         kern = f.read()
     with open(os.path.join(csrc, "ac_device.cuh")) as f:
         dev = f.read()
-    text = _function_text(kern, "k_smooth_fine") + "".join(_function_text(dev, n) for n in SMOOTH_HELPERS)
+    text = "".join(_function_text(kern, n) for n in SMOOTH_KERNEL) + "".join(_function_text(dev, n)
+                                                                            for n in SMOOTH_HELPERS)
     return hashlib.sha256(text.encode()).hexdigest()
 
 
