@@ -248,9 +248,11 @@ AC_HD T rcp_count(int k) {
 // with FP64_ONLY, the binary64 iteration runs.
 // any_or(m) returns the OR of m over the lanes that run together (the
 // identity on the host): a binary64 operation on component i is skipped
-// when no lane needs it.  Returns 0 (float set accepted), 1 (binary64
-// iteration) or 2 (no kept component, which a feasible correction cannot
-// give: u is then zero and the caller projects it).
+// when no lane needs it.  Every lane reaches every any_or (a lane that left
+// early while the others wait for it in a loop over tiles would be
+// undefined).  Returns 0 (float set accepted), 1 (binary64 iteration) or 2 (no
+// kept component, which a feasible correction cannot give: u is then zero and
+// the caller projects it).
 template <int N, bool FP64_ONLY = false, typename AnyOr>
 AC_HD int outer_update_node(double (&uk)[N], const float (&dk)[N], AnyOr any_or) {
   unsigned keep0 = 0;
@@ -270,7 +272,6 @@ AC_HD int outer_update_node(double (&uk)[N], const float (&dk)[N], AnyOr any_or)
       uk[i] = 0.0;
     }
   }
-  if (cnt == 0) return 2;
   unsigned keep = keep0;
   double theta = 0.0;
   bool ok = !FP64_ONLY;
@@ -334,7 +335,7 @@ AC_HD int outer_update_node(double (&uk)[N], const float (&dk)[N], AnyOr any_or)
 #pragma unroll
   for (int i = 0; i < N; ++i)
     uk[i] = (((anyf >> i) & 1u) && ((keep >> i) & 1u)) ? uk[i] - theta : 0.0;
-  return ok ? 0 : 1;
+  return cnt == 0 ? 2 : ok ? 0 : 1;
 }
 
 // ---- 64-bit fixed point -------------------------------------------------------
