@@ -1,0 +1,45 @@
+"""The coarsest level of the GPU path's grid hierarchy."""
+import numpy as np
+import pytest
+
+from paper_0710_0736_gb300 import synth
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def ac():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_0710_0736_gb300 import build
+    build.build()
+    from paper_0710_0736_gb300 import ac as mod
+    return mod
+
+
+def _step(ac, W, H, N, eps, tau, precision, smoother, **kw):
+    seg = ac.Segmenter(W, H, N, eps, 1.0, tau, tol=1e-10, max_cycles=500,
+                       precision=ac.AC_MIXED if precision == "mixed" else ac.AC_FP64, **kw)
+    ac.ac_set_coarse_smoother(seg.ctx, smoother)
+    seg.set_image(synth.shapes_image(W + N, W, H, rect_side=(1, max(1, W // 3)), disk_r=(1, max(1.5, H / 5))))
+    seg.set_phase(synth.dirichlet_init(3, (W + 1) * (H + 1), N))
+    st = seg.step(1)
+    u = seg.phase()
+    seg.close()
+    return u, st
+
+
+# one coarse level, above the size that the one-block tail takes: ended by
+# coarse_min, and by the mass (8 tau eps = 4 h^2 on its cells of side 2)
+@pytest.mark.parametrize("W,H,N,eps,tau,coarse_min", [(256, 256, 2, 5.0, 25.0, 100), (255, 200, 3, 5.0, 25.0, 60),
+                                                      (600, 401, 4, 1.0, 2.0, 4)])
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_coarsest_level_takes_gauss_seidel(ac, W, H, N, eps, tau, coarse_min, precision):
+    """The coarsest level is solved by Gauss-Seidel with either smoother, so
+    with no other coarse level the choice changes nothing."""
+    (u, st), (v, sv) = (_step(ac, W, H, N, eps, tau, precision, s, coarse_min=coarse_min)
+                        for s in (ac.AC_SMOOTH_GS3, ac.AC_SMOOTH_JACOBI))
+    assert st.converged and sv.converged
+    assert st.total_cycles == sv.total_cycles
+    assert np.array_equal(u, v)
