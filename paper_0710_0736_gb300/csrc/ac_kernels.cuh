@@ -2583,13 +2583,14 @@ __device__ __forceinline__ T tail_offdiag(const TailLevel<T> &L, const T *v, int
 // `sweeps` Gauss-Seidel sweeps on v in place, the colours forward (0, 1, 2)
 // in even sweeps and backward in odd ones (as the tiles of k_coarse_pair).
 // The colour that ends one sweep starts the next: its second pass would
-// repeat the first one's values, and is left out.
+// repeat the first one's values, and is left out.  forward: the colours
+// forward in every sweep, three passes that all count.
 template <typename T>
-__device__ __forceinline__ void tail_sgs(const TailLevel<T> &L, int sweeps) {
+__device__ __forceinline__ void tail_sgs(const TailLevel<T> &L, int sweeps, bool forward = false) {
   const TailWalk w(L.W);
   for (int s = 0; s < sweeps; ++s)
-    for (int q = s > 0 ? 1 : 0; q < 3; ++q) {
-      tail_colour(L, w, (s & 1) ? 2 - q : q,
+    for (int q = s > 0 && !forward ? 1 : 0; q < 3; ++q) {
+      tail_colour(L, w, (s & 1) && !forward ? 2 - q : q,
                   [&](int k) { L.v[k] = (L.r[k] - tail_offdiag(L, L.v, k)) * L.I[k]; });
       __syncthreads();
     }
@@ -2768,7 +2769,7 @@ __global__ void __launch_bounds__(kTailThreads) k_coarse_tail(TailArgs a, const 
   }
   {
     const TailLevel<T> L = level(last);
-    tail_sgs(L, coarsest_sweeps);
+    tail_sgs(L, coarsest_sweeps, a.forward);
   }
   for (int l = last - 1; l >= 0; --l) {
     const TailLevel<T> L = level(l), Cc = level(l + 1);

@@ -27,6 +27,7 @@ struct TailArgs {
   int levels;
   int W[kTailMaxLevels], H[kTailMaxLevels];
   const void *op[kTailMaxLevels];  // phase-major C, E, N, NE planes of each level
+  bool forward;  // the coarsest level's sweeps run the colours forward in each (else forward and backward in turn)
 };
 
 // The live-tile state of a tiled coarse level (see kLiveNow in
