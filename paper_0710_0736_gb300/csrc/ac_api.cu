@@ -1359,14 +1359,14 @@ int step_device(ac_ctx *ctx, int n_steps, ac_stats *out) {
   if (out) AC_CUDA(cudaMemcpyAsync(ctx->h_scalars + 1, ctx->energy, sizeof(double), cudaMemcpyDeviceToHost, ctx->s));
   AC_CUDA(cudaMemcpyAsync(ctx->h_scalars + 2, ctx->rho + 1, sizeof(double), cudaMemcpyDeviceToHost, ctx->s));
   AC_CUDA(cudaStreamSynchronize(ctx->s));
-  {
+  ac_stats st{};
+  int rc = loop_stats(ctx, ctx->step_graph[0], n_steps, &st);
+  if (st.total_cycles > 0) {
     // the free nodes of the last cycle (one colour) choose the next call's loop
     unsigned long long c = 0;
     std::memcpy(&c, ctx->h_scalars + 2, sizeof c);
-    if (ctx->p.nu1 + ctx->p.nu2 > 0) ctx->sv.free_frac = 2.0 * (double)c / (double)ctx->sv.lv[0].n;
+    ctx->sv.free_frac = 2.0 * (double)c / (double)ctx->sv.lv[0].n;
   }
-  ac_stats st{};
-  int rc = loop_stats(ctx, ctx->step_graph[0], n_steps, &st);
   if (out) {
     st.energy = std::ldexp(ctx->h_scalars[1], -ctx->r);  // pixel units: E = 2^-r E(eps', lambda')
     *out = st;
@@ -1695,6 +1695,7 @@ int ac_create(ac_ctx **out, const ac_params *p) {
     // rho, the free-node count of the fine residual, and the settled tiles'
     // list counters (read back together)
     AC_ALLOC(ctx->rho, 2 * sizeof(double) + sizeof(ac::SettledCtl));
+    AC_CUDA(cudaMemsetAsync(ctx->rho, 0, 2 * sizeof(double) + sizeof(ac::SettledCtl), ctx->s));
     S.settled.ctl = reinterpret_cast<ac::SettledCtl *>(ctx->rho + 2);
     AC_ALLOC(ctx->omega, 2 * sizeof(double));  // omega and its float rounding
     AC_ALLOC(ctx->ls_part, (size_t)2 * ls_blocks * sizeof(double));
