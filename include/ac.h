@@ -285,14 +285,16 @@ int ac_set_coarse_smoother(ac_ctx *ctx, int mode);
  *     (ac_set_coarse_tiling; with AC_TILES_AUTO that is every image whose
  *     coarse levels are too small for tiles, e.g. 1024^2 and below at N <= 8),
  *     and on the host otherwise, as it is for an image of at least 3 M
- *     unknowns (0.5 M in AC_FP64) whose last cycle found few free nodes: the
- *     host loop then visits only the fine tiles that can change
- *     (ac_set_coarse_tiling);
+ *     unknowns (0.5 M in AC_FP64) with few free nodes -- as the last cycle
+ *     found them, or, after ac_set_phase, as a sample of the new field's nodes
+ *     has two phases or more: the host loop then visits only the fine tiles that
+ *     can change (ac_set_coarse_tiling);
  *   AC_LOOP_HOST: always on the host.
  * If the graph cannot be captured or instantiated (a driver without
  * conditional nodes), the context switches itself to AC_LOOP_HOST and the
  * step runs on the host loop.  ac_get_cycle_loop sets *on_device to 1 if the
- * next ac_step runs the loop on the device.  AC_ERR_ARG for a NULL context or
+ * next ac_step runs the loop on the device (after ac_set_phase it may wait for
+ * the stream to see the field).  AC_ERR_ARG for a NULL context or
  * an unknown mode. */
 enum { AC_LOOP_AUTO = 0, AC_LOOP_HOST = 1 };
 int ac_set_cycle_loop(ac_ctx *ctx, int mode);

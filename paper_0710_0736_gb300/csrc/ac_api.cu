@@ -13,6 +13,7 @@
 #include <cstring>
 #include <map>
 #include <new>
+#include <numeric>
 #include <string>
 #include <thread>
 #include <tuple>
@@ -193,10 +194,12 @@ struct Solve {
   int depth = 0;          // levels in use (<= lv.size()); a schedule can cut the hierarchy short
   ac::Galerkin0Table tab0{};
   // the settled fine tiles' record (changed null: none, the adjoint's solves);
-  // whether the last cycle kept it, and the free fraction it found
+  // whether the last cycle kept it; the free fraction that the last cycle found,
+  // unless a field has been set since, and sampled (field_set)
   ac::SettledTiles settled{};
   bool record = false;
   double free_frac = 1.0;
+  bool sampled = false;
   // graphs [profiling][variant]: smoothing + residual (SmoothVariant), and
   // the coarse correction with its line search [profiling][form: dense levels
   // / tiled levels with live flags and work lists]
@@ -325,6 +328,8 @@ struct ac_ctx {
   AdjState adj;
   bool adj_pre32 = true;           // the adjoint's FCG preconditioned by the FP32 V-cycle (else FP64)
   double *h_scalars = nullptr;     // pinned: rho, energy
+  unsigned *h_undecided = nullptr;  // behind it: the undecided nodes in a field's sample (field_set)
+  cudaEvent_t sample_done = nullptr;
   bool have_image = false, have_rhs = false;
   std::vector<void *> allocs;
   // instrumentation
@@ -791,11 +796,57 @@ int enqueue_correction(ac_ctx *ctx, Solve &S) {
   return AC_OK;
 }
 
-// Whether the next cycle smooths only the tiles that can change.
-bool settled_form(const ac_ctx *ctx, const Solve &S, int64_t min_unknowns) {
+// u is replaced by the field at u (device): the next step's loop and form
+// follow it.  Its undecided nodes (two phases or more) are counted on a sample --
+// the choice needs no more, and the numbers do not depend on it -- or taken to
+// be all of them on grids that have no such choice.  Left at what the last step
+// found, a random field after a formed one took the host loop and the record of
+// all tiles, and a formed field in a new context the plain form (first pass at
+// 1024^2, N = 4 FP64 4.7 -> 3.2 ms, at 4096^2, N = 8 mixed 13.0 -> 11.4).
+// Called before the copy of a field on the device: the copy then covers the way
+// of the count to the host.
+int field_set(ac_ctx *ctx, const double *u) {
+  Solve &S = ctx->sv;
+  S.free_frac = 1.0;
+  S.sampled = false;
+  if (ctx->n * ctx->N < settled_min_unknowns(S.o->elem) || ctx->n < ac::kSampleNodes) return AC_OK;
+  if (ctx->s) {
+    // in a caller's capture the count would come with the replay
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    AC_CUDA(cudaStreamIsCapturing(ctx->s, &cap));
+    if (cap != cudaStreamCaptureStatusNone) return AC_OK;
+  }
+  AC_RUN(AC_PROF_SETUP, ctx->ops->undecided(u, ctx->n, ctx->h_undecided, ctx->s));
+  AC_CUDA(cudaEventRecord(ctx->sample_done, ctx->s));
+  S.sampled = true;
+  return AC_OK;
+}
+
+// Whether a kernel may read doubles at p as this device's memory (a copy takes
+// more: other devices' memory, any alignment).
+bool device_doubles(const double *p) {
+  cudaPointerAttributes a{};
+  int dev = 0;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return a.type == cudaMemoryTypeDevice && a.device == dev && reinterpret_cast<uintptr_t>(p) % sizeof(double) == 0;
+}
+
+// Whether the next cycle smooths only the tiles that can change.  Waits for
+// the count of a field set since the last step, if that decides.
+bool settled_form(ac_ctx *ctx, Solve &S, int64_t min_unknowns) {
   // a cycle's passes must not reach past a tile (k_smooth_settled)
   if (!S.settled.changed || 2 * (ctx->p.nu1 + ctx->p.nu2) > ac::kSetT || S.tiling == AC_TILES_NEVER) return false;
-  return S.tiling == AC_TILES_ALWAYS || (S.lv[0].n * ctx->N >= min_unknowns && S.free_frac < kSettledFreeFraction);
+  if (S.tiling == AC_TILES_ALWAYS) return true;
+  if (S.lv[0].n * ctx->N < min_unknowns) return false;
+  if (S.sampled) {
+    if (cudaEventSynchronize(ctx->sample_done) != cudaSuccess) return false;  // the call that follows reports it
+    S.free_frac = std::accumulate(ctx->h_undecided, ctx->h_undecided + ac::kSampleBlocks, 0u) / (double)ac::kSampleNodes;
+    S.sampled = false;
+  }
+  return S.free_frac < kSettledFreeFraction;
 }
 
 // Multigrid solve of one step problem.  Cycle structure:
@@ -863,6 +914,7 @@ int solve_mg(ac_ctx *ctx, Solve &S, double tol, int max_cycles, int *cycles_out,
     // free nodes: only one colour is counted after a smoothing sequence, about
     // half of them
     S.free_frac = (double)nfree * (nsw >= 1 ? 2.0 : 1.0) / (double)S.lv[0].n;
+    S.sampled = false;
     if (rho <= tol) {
       status = AC_OK;
       break;
@@ -1173,7 +1225,7 @@ void release_step_graphs(ac_ctx *ctx) {
 }
 
 // Whether ac_step runs the device-side loop (see above).
-bool loop_on_device(const ac_ctx *ctx) {
+bool loop_on_device(ac_ctx *ctx) {
   return ctx->loop_mode == AC_LOOP_AUTO && ctx->use_graphs && !ctx->profiling && tiled_end(ctx->sv) <= 1 &&
          !settled_form(ctx, ctx->sv, settled_host_unknowns(ctx->sv.o->elem));
 }
@@ -1333,6 +1385,7 @@ int loop_stats(ac_ctx *ctx, const StepGraph &sg, int n_steps, ac_stats *out) {
   ctx->delta_warm = c.warm != 0;
   ctx->have_rhs = true;
   ctx->sv.record = false;  // the device-side loop keeps no record of its tiles
+  ctx->sv.sampled = false;  // a field set before is not the one at hand any more
   if (out) {
     out->residual = c.last_rho;
     out->cycles = c.last_cycles;
@@ -1719,7 +1772,9 @@ int ac_create(ac_ctx **out, const ac_params *p) {
       L.lists.sms = ctx->sms;
       AC_CUDA(cudaMemsetAsync(L.lists.flags, ac::kLiveNow, nt * N, ctx->s));  // the first cycle writes all tiles
     }
-    AC_CUDA(cudaMallocHost(&ctx->h_scalars, 4 * sizeof(double)));
+    AC_CUDA(cudaMallocHost(&ctx->h_scalars, 4 * sizeof(double) + ac::kSampleBlocks * sizeof(unsigned)));
+    ctx->h_undecided = reinterpret_cast<unsigned *>(ctx->h_scalars + 4);
+    AC_CUDA(cudaEventCreateWithFlags(&ctx->sample_done, cudaEventDisableTiming));
     AC_CUDA(cudaMemsetAsync(ctx->c, 0, (size_t)3 * N * sizeof(double), ctx->s));
     AC_CUDA(cudaMemsetAsync(ctx->omega, 0, 2 * sizeof(double), ctx->s));
     AC_CUDA(cudaMemsetAsync(ctx->ls_done, 0, sizeof(unsigned), ctx->s));
@@ -1761,6 +1816,7 @@ void ac_destroy(ac_ctx *ctx) {
   if (ctx->lab) cudaFree(ctx->lab);
   if (ctx->img16) cudaFree(ctx->img16);
   if (ctx->h_scalars) cudaFreeHost(ctx->h_scalars);
+  if (ctx->sample_done) cudaEventDestroy(ctx->sample_done);
   delete ctx;
 }
 
@@ -1865,6 +1921,8 @@ static int set_image_impl(ac_ctx *ctx, const void *rgb, int is_device, bool f64)
   ctx->have_image = true;
   ctx->have_rhs = false;
   ctx->delta_warm = false;
+  ctx->sv.free_frac = 1.0;  // every node of the random start is undecided
+  ctx->sv.sampled = false;
   return AC_OK;
 }
 
@@ -1960,10 +2018,15 @@ int ac_segment(ac_ctx *ctx, int n_steps, int8_t *pixel_labels, int is_device, ac
 
 int ac_set_phase(ac_ctx *ctx, const double *u, int is_device) {
   if (!ctx || !u) return fail(AC_ERR_ARG, "NULL argument");
+  const bool early = is_device && device_doubles(u);
+  int rc = early ? field_set(ctx, u) : AC_OK;
+  if (rc) return rc;
   AC_CUDA(cudaMemcpyAsync(ctx->u, u, (size_t)ctx->n * ctx->N * sizeof(double),
                           is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, ctx->s));
   AC_CUDA(cudaMemsetAsync(ctx->c, 0, (size_t)3 * ctx->N * sizeof(double), ctx->s));
   ctx->delta_warm = false;  // a new state: the next step's correction starts from zero
+  if (!early) rc = field_set(ctx, ctx->u);
+  if (rc) return rc;
   if (!is_device) AC_CUDA(cudaStreamSynchronize(ctx->s));
   return AC_OK;
 }
@@ -2452,6 +2515,7 @@ int ac_adjoint_backward(ac_ctx *ctx, const double *grad_u, double *grad_lambda, 
     // arithmetic: like the forward, the segment's first step starts its
     // correction from zero (AC_MIXED), and the later ones from the previous
     // step's, which the recomputation has just produced
+    if (int rc = field_set(ctx, A.cp_u + (size_t)j * nN)) return rc;
     AC_CUDA(cudaMemcpyAsync(ctx->u, A.cp_u + (size_t)j * nN, fN, cudaMemcpyDeviceToDevice, ctx->s));
     AC_CUDA(cudaMemcpyAsync(ctx->c, A.cp_c + (size_t)j * N * 3, cN, cudaMemcpyDeviceToDevice, ctx->s));
     AC_CUDA(cudaMemcpyAsync(A.seg_u, ctx->u, fN, cudaMemcpyDeviceToDevice, ctx->s));
@@ -2526,6 +2590,7 @@ int ac_adjoint_backward(ac_ctx *ctx, const double *grad_u, double *grad_lambda, 
   }
   AC_CUDA(cudaMemcpyAsync(ctx->h_scalars + 2, A.scal, 2 * sizeof(double), cudaMemcpyDeviceToHost, ctx->s));
   AC_CUDA(cudaMemcpyAsync(ctx->h_scalars + 1, A.ndiff, sizeof(unsigned long long), cudaMemcpyDeviceToHost, ctx->s));
+  if (int rc = field_set(ctx, A.uT)) return rc;
   AC_CUDA(cudaMemcpyAsync(ctx->u, A.uT, fN, cudaMemcpyDeviceToDevice, ctx->s));  // leave u = u^T
   AC_CUDA(cudaStreamSynchronize(ctx->s));
   *grad_lambda = std::ldexp(ctx->h_scalars[2], -ctx->r);

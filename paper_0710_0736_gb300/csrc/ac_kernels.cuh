@@ -3378,6 +3378,23 @@ __global__ void k_composite(const double *__restrict__ u, const double *__restri
   for (int ch = 0; ch < 3; ++ch) o[ch] = (float)(rounded ? c[best * 3 + ch] : rgb[ch]);
 }
 
+// Undecided nodes (two phases or more other than 0) among the sample nodes, one
+// a thread, drawn each from its own equal part of the grid's n >= gridDim.x *
+// kBlock nodes; out[block] in page-locked host memory.  u may be a caller's
+// buffer, aligned to its doubles only: no vector loads.
+template <int N>
+__global__ void __launch_bounds__(kBlock) k_undecided(const double *__restrict__ u, int64_t n,
+                                                      unsigned *__restrict__ out) {
+  pdl_sync();
+  const int64_t k = (int64_t)blockIdx.x * kBlock + threadIdx.x, part = n / ((int64_t)gridDim.x * kBlock);
+  const double *const p = u + (k * part + (int64_t)(splitmix64((uint64_t)k) % (uint64_t)part)) * N;
+  int on = 0;
+#pragma unroll
+  for (int i = 0; i < N; ++i) on += p[i] != 0.0;
+  const int c = __syncthreads_count(on >= 2);
+  if (threadIdx.x == 0) out[blockIdx.x] = (unsigned)c;
+}
+
 // Node label = argmax_i u_n,i (lowest index on ties), on the solve grid.
 template <int N>
 __global__ void k_labels(const double *__restrict__ u, Geo g, int8_t *__restrict__ node_lab) {

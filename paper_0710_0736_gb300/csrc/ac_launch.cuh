@@ -384,6 +384,10 @@ struct Launch {
     launch(k_composite<N>, row_grid(g.W >> r, g.H >> r), kBlock, 0, s, u, c, g, r, rounded, out);
     return 1;
   }
+  static int undecided(const double *u, int64_t n, unsigned *out, cudaStream_t s) {
+    launch(k_undecided<N>, kSampleBlocks, kBlock, 0, s, u, n, out);
+    return 1;
+  }
   static int labels(const double *u, const Geo &g, int r, int8_t *node_lab, int8_t *pix_lab, cudaStream_t s) {
     int k = 0;
     if (node_lab) {
@@ -468,6 +472,7 @@ struct Launch {
                           outer_update,
                           outer_resid_tiles,
                           outer_update_tiles,
+                          undecided,
                           labels,
                           composite,
                           project,

@@ -15,6 +15,10 @@ struct SettledTiles;
 // Scratch of the block-partial reductions: at most kMaxPartBlocks rows.
 constexpr int kMaxPartBlocks = 1024;
 
+// Sample of a field's nodes (undecided): blocks of 256 threads, one node each.
+// A share of 0.2 comes out within 0.007 (three standard deviations).
+constexpr int kSampleBlocks = 112, kSampleNodes = kSampleBlocks * 256;
+
 // The bottom levels k0 .. k0 + levels - 1 of a coarse V-cycle, run by one
 // block per phase in shared memory (kTailArrays values per node: C, 1/C, E,
 // N, NE, r, v, t, each array framed by zeros: one node west and south, two
@@ -148,6 +152,9 @@ struct Ops {
   int (*outer_resid_tiles)(const double *u, const float *b, const Geo &g, float *r32, float *u32, double *rho,
                            const SettledTiles &st, cudaStream_t s);
   int (*outer_update_tiles)(double *u, const float *delta, const Geo &g, const SettledTiles &st, cudaStream_t s);
+  // nodes with two phases or more among kSampleNodes sample nodes of n >=
+  // kSampleNodes (out: kSampleBlocks parts of the count, page-locked host memory)
+  int (*undecided)(const double *u, int64_t n, unsigned *out, cudaStream_t s);
   // pixel outputs are on the image's pixels: the solve grid g coarsened r times
   int (*labels)(const double *u, const Geo &g, int r, int8_t *node_lab, int8_t *pix_lab, cudaStream_t s);
   int (*composite)(const double *u, const double *c, const Geo &g, int r, int rounded, float *out, cudaStream_t s);
