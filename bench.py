@@ -209,14 +209,18 @@ def smooth_source_digest():
 
 
 def smooth_bytes(prof):
-    """Algorithmic bytes of all timed smoother launches: each launch moves the
-    library's per-launch bytes (one colour's right-hand side and obstacle and
-    the other colour's iterate read, its own colour written); a launch that
-    also applies the pending coarse correction reads the other colour's
-    correction d as well."""
+    """Algorithmic bytes of all timed smoother launches: those the library
+    booked to the class (launches on settled tiles count the visited part).
+    Without class bytes, each launch moves the library's per-launch bytes (one
+    colour's right-hand side and obstacle and the other colour's iterate read,
+    its own colour written); a launch that also applies the pending coarse
+    correction reads the other colour's correction d as well."""
     from paper_0710_0736_gb300 import ac
-    return (prof.launches[ac.PROF_CLASSES.index("smooth")] * prof.smooth_bytes_per_launch
-            + prof.smooth_corr_launches * prof.smooth_corr_extra_bytes)
+    k = ac.PROF_CLASSES.index("smooth")
+    booked = getattr(prof, "bytes", None)
+    if booked is not None:
+        return booked[k]
+    return prof.launches[k] * prof.smooth_bytes_per_launch + prof.smooth_corr_launches * prof.smooth_corr_extra_bytes
 
 
 def smooth_traffic(n_nodes, n_phases, precision):

@@ -129,8 +129,8 @@ enum {
 typedef struct {
   double ms[AC_PROF_COUNT];        /* summed device time per class (CUDA events on the context's stream) */
   int64_t launches[AC_PROF_COUNT]; /* kernel launches per class while profiling was on */
-  double smooth_bytes_per_launch;  /* algorithmic HBM bytes of one smoother launch (one colour), on average where
-                                      cycles visited part of the nodes: AC_FP64
+  double smooth_bytes_per_launch;  /* algorithmic HBM bytes of one smoother launch (one colour) that visits every
+                                      node of it (bytes[AC_PROF_SMOOTH] has what the launches visited): AC_FP64
                                       1.5 n N 8 (b of the colour, u of the other colour read, u of the
                                       colour written), AC_MIXED 2 n N 4 (r and obstacle of the colour,
                                       delta of the other colour read, delta of the colour written) */

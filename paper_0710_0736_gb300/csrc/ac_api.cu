@@ -349,7 +349,6 @@ struct ac_ctx {
   double prof_bytes[AC_PROF_COUNT] = {};
   int64_t prof_corr_launches = 0;  // smoother launches that applied a pending correction
   double settled_bytes[2][AC_PROF_COUNT] = {};  // a first / later cycle's smoothing and residual over all nodes
-  bool prof_settled = false;                 // the profile holds cycles that did not visit all nodes
   // CUDA graphs (off on the legacy default stream, which cannot be captured)
   bool use_graphs = false;
   GraphSlot *capturing = nullptr;
@@ -895,7 +894,6 @@ int solve_mg(ac_ctx *ctx, Solve &S, double tol, int max_cycles, int *cycles_out,
         // the graph books every node: take the nodes not visited off again
         for (int cls : {(int)AC_PROF_SMOOTH, (int)AC_PROF_RESID})
           ctx->prof_bytes[cls] -= (1.0 - listed) * ctx->settled_bytes[later][cls];
-        ctx->prof_settled = true;
       }
     }
 #ifdef AC_TRACE_CYCLES
@@ -2160,7 +2158,6 @@ int ac_set_profiling_mask(ac_ctx *ctx, unsigned class_mask) {
     ctx->prof_bytes[k] = 0;
   }
   ctx->prof_corr_launches = 0;
-  ctx->prof_settled = false;
   class_mask &= (1u << AC_PROF_COUNT) - 1u;
   ctx->profiling = class_mask != 0;
   ctx->prof_mask = class_mask ? class_mask : (1u << AC_PROF_COUNT) - 1u;
@@ -2243,13 +2240,10 @@ int ac_get_profile(ac_ctx *ctx, ac_profile *out) {
   }
   out->smooth_bytes_per_launch = ctx->p.precision == AC_MIXED ? 2.0 * (double)ctx->n * ctx->N * sizeof(float)
                                                                : 1.5 * (double)ctx->n * ctx->N * sizeof(double);
-  const double corr_extra = 0.5 * (double)ctx->n * ctx->N * (ctx->p.precision == AC_MIXED ? sizeof(float) : sizeof(double));
-  if (ctx->prof_settled && ctx->prof_launches[AC_PROF_SMOOTH] > 0)
-    out->smooth_bytes_per_launch = (ctx->prof_bytes[AC_PROF_SMOOTH] - corr_extra * (double)ctx->prof_corr_launches) /
-                                   (double)ctx->prof_launches[AC_PROF_SMOOTH];
   out->total_launches = ctx->total_launches;
   out->smooth_corr_launches = ctx->prof_corr_launches;
-  out->smooth_corr_extra_bytes = corr_extra;
+  out->smooth_corr_extra_bytes = 0.5 * (double)ctx->n * ctx->N * (ctx->p.precision == AC_MIXED ? sizeof(float)
+                                                                                                 : sizeof(double));
   return AC_OK;
 }
 
