@@ -117,7 +117,7 @@ typedef struct {
 /* Kernel classes of the profile (no counterpart in the paper: instrumentation). */
 enum {
   AC_PROF_SMOOTH = 0,  /* fine red-black projected Gauss-Seidel, one launch per colour */
-  AC_PROF_RESID,       /* fine residual, natural residual, mask, tangent projection */
+  AC_PROF_RESID,       /* fine residual, natural residual, mask, tangent projection; lists of the fine tiles to visit */
   AC_PROF_COARSE,      /* coarse-level smoothing, residuals and coarsest solve */
   AC_PROF_TRANSFER,    /* truncated Galerkin operators, restriction */
   AC_PROF_LINESEARCH,  /* coarse-correction direction, line search, update */

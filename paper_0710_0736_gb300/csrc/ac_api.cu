@@ -712,9 +712,7 @@ int coarse_vcycle(ac_ctx *ctx, Solve &S, int k, void **res) {
 int enqueue_smooth_resid(ac_ctx *ctx, Solve &S, SmoothVariant variant) {
   const bool later = variant == kLater || variant == kLaterSettledAll || variant == kLaterSettled;
   const bool settled = variant >= kFirstSettledAll;
-  const ac::SettledCycle which = variant == kFirstSettled   ? ac::kSettledStart
-                                 : variant == kLaterSettled ? ac::kSettledCycle
-                                                            : ac::kSettledAll;
+  const bool all = variant != kFirstSettled && variant != kLaterSettled;
   const ac::SolverOps *o = S.o;
   const ac::Geo &g0 = S.lv[0].g;
   const ByteModel bm = byte_model(ctx, S);
@@ -736,14 +734,18 @@ int enqueue_smooth_resid(ac_ctx *ctx, Solve &S, SmoothVariant variant) {
                                   ? ac::MaskDirty{S.lv[1].lists.dirty, ac::tiles_x(S.lv[1].g), ac::tiles_y(S.lv[1].g)}
                                   : ac::MaskDirty{nullptr, 0, 0};
   if (settled) {
-    if (which != ac::kSettledAll) {
+    const double rs_bytes = 0.5 * bm.n * (bm.ns * (4 + bm.ob) + 1);
+    if (!all) {
       ctx->settled_bytes[later ? 1 : 0][AC_PROF_SMOOTH] = sm_bytes;
-      ctx->settled_bytes[later ? 1 : 0][AC_PROF_RESID] = 0.5 * bm.n * (bm.ns * (4 + bm.ob) + 1);
+      ctx->settled_bytes[later ? 1 : 0][AC_PROF_RESID] = rs_bytes;
+      // (counted with the residual, whose marks it reads)
+      AC_RUN(AC_PROF_RESID, o->settled_list(S.settled, later ? ac::kSetCycle : ac::kSetCycle | ac::kSetSeed | ac::kSetX,
+                                            true, !later, ctx->s));
     }
     AC_RUNB(AC_PROF_SMOOTH, sm_bytes, o->smooth_settled(S.x, S.rhs, S.ob, corr, ctx->omega, g0, nsw, rt_zero, S.mask,
-                                                        dirty, ctx->rho, S.settled, which, ctx->s));
-    AC_RUNB(AC_PROF_RESID, 0.5 * bm.n * (bm.ns * (4 + bm.ob) + 1),
-            o->resid_settled(S.x, S.rhs, S.ob, g0, S.rt, S.mask, ctx->rho, dirty, S.settled, which, ctx->s));
+                                                        dirty, ctx->rho, S.settled, all, ctx->s));
+    AC_RUNB(AC_PROF_RESID, rs_bytes,
+            o->resid_settled(S.x, S.rhs, S.ob, g0, S.rt, S.mask, ctx->rho, dirty, S.settled, all, ctx->s));
     return AC_OK;
   }
   AC_RUNB(AC_PROF_SMOOTH, sm_bytes, o->smooth(S.x, S.rhs, S.ob, corr, ctx->omega, g0, nsw, rt_zero,

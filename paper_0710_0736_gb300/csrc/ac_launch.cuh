@@ -101,10 +101,7 @@ struct SolverLaunch {
   }
   static int smooth_settled(void *x, const void *rhs, const void *ob, const void *corr, const double *omega,
                             const Geo &g, int sweeps, void *rt, uint8_t *mask, const MaskDirty &dirty, double *rho,
-                            const SettledTiles &st, SettledCycle which, cudaStream_t s) {
-    const bool all = which == kSettledAll;
-    if (which == kSettledCycle) settled_list(st, kSetCycle, true, false, s);
-    if (which == kSettledStart) settled_list(st, kSetCycle | kSetSeed | kSetX, true, true, s);
+                            const SettledTiles &st, bool all, cudaStream_t s) {
     for (int p = 0; p < 2 * sweeps; ++p) {
       const T *cr = p == 0 ? (const T *)corr : nullptr;
       if (p == 2 * sweeps - 1)
@@ -118,12 +115,10 @@ struct SolverLaunch {
                s, (T *)x, (const T *)rhs, (const T *)ob, cr, omega, g, p & 1, nullptr, mask,
                MaskDirty{nullptr, 0, 0}, nullptr, st, all);
     }
-    return 2 * sweeps + (all ? 0 : 1);
+    return 2 * sweeps;
   }
   static int resid_settled(const void *x, const void *rhs, const void *ob, const Geo &g, void *rt, uint8_t *mask,
-                           double *rho, const MaskDirty &dirty, const SettledTiles &st, SettledCycle which,
-                           cudaStream_t s) {
-    const bool all = which == kSettledAll;
+                           double *rho, const MaskDirty &dirty, const SettledTiles &st, bool all, cudaStream_t s) {
     launch(k_resid_settled<T, N, FORM>, settled_grid(st, k_resid_settled<T, N, FORM>), kBlock, 0, s, (const T *)x,
            (const T *)rhs, (const T *)ob, g, (T *)rt, mask, rho, dirty, st, all);
     return 1;
@@ -283,11 +278,9 @@ struct SolverLaunch {
     if constexpr (FORM != kTangent) {
       ss = smooth_settled;
       rs = resid_settled;
-    }
-    if constexpr (FORM == kShifted) {
       sl = settled_list;
-      sz = settled_zero;
     }
+    if constexpr (FORM == kShifted) sz = settled_zero;
     return SolverOps{(int)sizeof(T), smooth,       resid,        ss, rs, sl, sz, restrict0,   galerkin0,   galerkin,   coarse_smooth,
                      coarse_resid, coarse_pre_resid, restrict_, coarse_tail,
                      line_search};

@@ -53,11 +53,6 @@ struct LevelLists {
   int sms;
 };
 
-// The tiles a cycle visits: all, which starts their record; those that the
-// record of the last cycle leaves; or, at the start of a solve, those and the
-// ones that the outer residual marked.
-enum SettledCycle { kSettledAll, kSettledCycle, kSettledStart };
-
 // One multigrid solve instantiation (scalar type and constraint form); array
 // arguments are typed by that instantiation (double or float).
 struct SolverOps {
@@ -73,15 +68,14 @@ struct SolverOps {
   int (*resid)(const void *x, const void *rhs, const void *ob, const Geo &g, void *rt, uint8_t *mask, double *rho,
                int color, const MaskDirty &dirty, cudaStream_t s);
   // the same two (smooth with a mask, resid of the first colour) on the tiles
-  // that can change in the cycle, or on all of them to start their record
+  // of the cycle's list, or on all of them to start their record
   int (*smooth_settled)(void *x, const void *rhs, const void *ob, const void *corr, const double *omega, const Geo &g,
                         int sweeps, void *rt, uint8_t *mask, const MaskDirty &dirty, double *rho,
-                        const SettledTiles &st, SettledCycle which, cudaStream_t s);
+                        const SettledTiles &st, bool all, cudaStream_t s);
   int (*resid_settled)(const void *x, const void *rhs, const void *ob, const Geo &g, void *rt, uint8_t *mask,
-                       double *rho, const MaskDirty &dirty, const SettledTiles &st, SettledCycle which,
-                       cudaStream_t s);
-  // mixed form: the list of the tiles with a mark in `what` (and those around
-  // them), and x = 0 on a list
+                       double *rho, const MaskDirty &dirty, const SettledTiles &st, bool all, cudaStream_t s);
+  // the list of the tiles with a mark in `what` (and those around them), and
+  // (mixed form) x = 0 on a list
   int (*settled_list)(const SettledTiles &st, unsigned what, bool around, bool restart, cudaStream_t s);
   int (*settled_zero)(void *x, const Geo &g, const SettledTiles &st, cudaStream_t s);
   // transfers skip the rows whose diagonal in the (coarse or fine) level's

@@ -52,3 +52,12 @@ def test_plain_launch_bytes_do_not_depend_on_the_tiles(ac, precision):
     for p in _profiles(ac, precision):
         assert p.smooth_bytes_per_launch == (8.0 * n if precision == "mixed" else 12.0 * n)
         assert p.smooth_corr_extra_bytes == (2.0 * n if precision == "mixed" else 4.0 * n)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_list_launches_are_not_smoother_launches(ac, precision):
+    """The same cycles run as many smoother launches, whatever they visit."""
+    k = ac.PROF_CLASSES.index("smooth")
+    dense, settled = _profiles(ac, precision)
+    assert settled.launches[k] == dense.launches[k]
+    assert 0 < settled.bytes[k] < dense.bytes[k]
