@@ -891,11 +891,13 @@ int solve_mg(ac_ctx *ctx, Solve &S, double tol, int max_cycles, int *cycles_out,
     if (variant == kFirstSettled || variant == kLaterSettled) {
       ac::SettledCtl sc;
       std::memcpy(&sc, ctx->h_scalars + 2, sizeof sc);
-      listed = (double)sc.count / ((double)S.settled.tx * S.settled.ty);
+      const double tiles = (double)S.settled.tx * S.settled.ty;
+      listed = (double)sc.count / tiles;
       if (ctx->profiling) {
-        // the graph books every node: take the nodes not visited off again
-        for (int cls : {(int)AC_PROF_SMOOTH, (int)AC_PROF_RESID})
-          ctx->prof_bytes[cls] -= (1.0 - listed) * ctx->settled_bytes[later][cls];
+        // the graph books every node: take the nodes not visited off again (the
+        // residual visits the tiles that joined the list too)
+        ctx->prof_bytes[AC_PROF_SMOOTH] -= (1.0 - listed) * ctx->settled_bytes[later][AC_PROF_SMOOTH];
+        ctx->prof_bytes[AC_PROF_RESID] -= (1.0 - listed - sc.joined / tiles) * ctx->settled_bytes[later][AC_PROF_RESID];
       }
     }
 #ifdef AC_TRACE_CYCLES
@@ -971,17 +973,32 @@ int solve_mixed(ac_ctx *ctx, int *cycles_out, double *rho_out, int64_t *sweeps_o
   // another 1.3 ms less.
   bool listed = false;  // the marks describe u and b
   int rc = AC_OK;
+  // a list of S.settled's tiles; while profiling, the unknowns on them (a read back)
+  const double all_unknowns = (double)ctx->n * ctx->N;
+  double visited = 0;
+  auto make_list = [&](unsigned what, bool around) -> int {
+    AC_RUN(AC_PROF_OUTER, S.o->settled_list(S.settled, what, around, false, ctx->s));
+    if (!ctx->profiling) return AC_OK;
+    double r = 0;
+    int rc_read = read_rho(ctx, &r);
+    if (rc_read) return rc_read;
+    ac::SettledCtl sc;
+    std::memcpy(&sc, ctx->h_scalars + 2, sizeof sc);
+    visited = all_unknowns * sc.count / ((double)S.settled.tx * S.settled.ty);
+    return AC_OK;
+  };
   for (;;) {
     AC_CUDA(cudaMemsetAsync(ctx->rho, 0, sizeof(double), ctx->s));
     if (outer > 0 && listed && S.record) {
-      AC_RUN(AC_PROF_OUTER, S.o->settled_list(S.settled, ac::kSetSeed | ac::kSetX, true, false, ctx->s));
-      AC_RUN(AC_PROF_OUTER, o->outer_resid_tiles(ctx->u, (const float *)ctx->b, ctx->g0, ctx->r32, ctx->u32, ctx->rho,
-                                                 S.settled, ctx->s));
+      rc = make_list(ac::kSetSeed | ac::kSetX, true);
+      if (rc) return rc;
+      AC_RUNB(AC_PROF_OUTER, visited * 24, o->outer_resid_tiles(ctx->u, (const float *)ctx->b, ctx->g0, ctx->r32,
+                                                                ctx->u32, ctx->rho, S.settled, ctx->s));
     } else {
       listed = S.record && settled_form(ctx, S, settled_min_unknowns(S.o->elem));
       if (listed) AC_CUDA(cudaMemsetAsync(S.settled.seed, 0, (size_t)S.settled.tx * S.settled.ty, ctx->s));
       // u (binary64) and b (double-float pairs) read, r32 and u32 written
-      AC_RUNB(AC_PROF_OUTER, (double)ctx->n * ctx->N * 24,
+      AC_RUNB(AC_PROF_OUTER, all_unknowns * 24,
               o->outer_resid(ctx->u, (const float *)ctx->b, ctx->g0, ctx->r32, ctx->u32, ctx->rho, rho32,
                              listed ? S.settled.seed : nullptr, S.settled.tx, ctx->s));
     }
@@ -1008,8 +1025,9 @@ int solve_mixed(ac_ctx *ctx, int *cycles_out, double *rho_out, int64_t *sweeps_o
     const bool warm = outer == 0 && ctx->delta_warm && ctx->p.nu1 >= 1;
     ctx->delta_warm = false;
     if (!warm && listed) {
-      AC_RUN(AC_PROF_OUTER, S.o->settled_list(S.settled, ac::kSetX, false, false, ctx->s));
-      AC_RUN(AC_PROF_OUTER, S.o->settled_zero(S.x, ctx->g0, S.settled, ctx->s));
+      rc = make_list(ac::kSetX, false);
+      if (rc) return rc;
+      AC_RUNB(AC_PROF_OUTER, visited * 4, S.o->settled_zero(S.x, ctx->g0, S.settled, ctx->s));
     } else if (!warm) {
       AC_CUDA(cudaMemsetAsync(S.x, 0, (size_t)fine_slots(ctx->n) * ctx->N * sizeof(float), ctx->s));
     }
@@ -1023,11 +1041,13 @@ int solve_mixed(ac_ctx *ctx, int *cycles_out, double *rho_out, int64_t *sweeps_o
     if (rc && rc != AC_ERR_NOT_CONVERGED) return rc;
     const int solved = rc;
     if (listed && S.record) {
-      AC_RUN(AC_PROF_OUTER, S.o->settled_list(S.settled, ac::kSetSeed | ac::kSetX, false, false, ctx->s));
-      AC_RUN(AC_PROF_OUTER, o->outer_update_tiles(ctx->u, (const float *)S.x, ctx->g0, S.settled, ctx->s));
+      rc = make_list(ac::kSetSeed | ac::kSetX, false);
+      if (rc) return rc;
+      AC_RUNB(AC_PROF_OUTER, visited * 20,
+              o->outer_update_tiles(ctx->u, (const float *)S.x, ctx->g0, S.settled, ctx->s));
     } else {
       // u read and written, delta read
-      AC_RUNB(AC_PROF_OUTER, (double)ctx->n * ctx->N * 20,
+      AC_RUNB(AC_PROF_OUTER, all_unknowns * 20,
               o->outer_update(ctx->u, (const float *)S.x, ctx->g0, ctx->s));
     }
     ++outer;

@@ -21,9 +21,9 @@ def ac():
 W, H, N = 320, 260, 4
 
 
-def _profiles(ac, precision):
-    """Profiles of the same steps from a formed field with every tile visited
-    and with the settled ones left out."""
+def _profiles(ac, precision, before=0):
+    """Profiles of the same steps (after `before` others) from a formed field
+    with every tile visited and with the settled ones left out."""
     rng = np.random.default_rng(2)
     y, x = np.mgrid[0:H + 1, 0:W + 1]
     z = -np.stack([np.hypot(x - rng.uniform(0, W), y - rng.uniform(0, H)) for _ in range(N)], -1) / 2.0
@@ -38,6 +38,8 @@ def _profiles(ac, precision):
         seg.set_cycle_loop(ac.AC_LOOP_HOST)
         seg.set_image(synth.shapes_image(W, W, H, rect_side=(20, 80), disk_r=(10, 40)))
         seg.set_phase(u0 / u0.sum(1, keepdims=True))
+        if before:
+            seg.step(before)
         ac.ac_set_profiling(seg.ctx, True)
         st = seg.step(4)
         out.append((st, ac.ac_get_profile(seg.ctx)))
@@ -61,3 +63,13 @@ def test_list_launches_are_not_smoother_launches(ac, precision):
     dense, settled = _profiles(ac, precision)
     assert settled.launches[k] == dense.launches[k]
     assert 0 < settled.bytes[k] < dense.bytes[k]
+
+
+def test_outer_passes_on_tiles_book_what_they_visit(ac):
+    """Of a mixed step only the first outer residual visits every node (24
+    bytes an unknown) once the record stands; the update and the other
+    residuals visit the listed tiles."""
+    k = ac.PROF_CLASSES.index("outer")
+    dense, settled = _profiles(ac, "mixed", before=1)
+    first = 4 * 24.0 * (W + 1) * (H + 1) * N
+    assert first < settled.bytes[k] < dense.bytes[k]
