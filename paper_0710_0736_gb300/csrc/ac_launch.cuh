@@ -2,6 +2,7 @@
 #pragma once
 #include <algorithm>
 #include "ac_kernels.cuh"
+#include "ac_resident.h"
 
 namespace ac {
 
@@ -40,15 +41,14 @@ inline int resident_blocks(K k, int threads) {
 }
 // The grid of a launch of kernel k over a level's lists: every block
 // resident at once, no more blocks than list entries can exist.
-template <class K>
-inline dim3 list_grid(const LevelLists *L, int64_t entries, K k, int threads) {
-  static const int per_sm = resident_blocks(k, threads);
-  const int64_t b = (int64_t)L->sms * per_sm;
+template <auto K, int THREADS>
+inline dim3 list_grid(const LevelLists *L, int64_t entries) {
+  const int64_t b = (int64_t)L->sms * once_per_kernel<K, THREADS>(resident_blocks<decltype(K)>);
   return dim3((unsigned)(b < entries ? b : (entries > 0 ? entries : 1)));
 }
-template <class K>
-inline dim3 tile_grid(const Geo &g, const LevelLists *L, int N, K k, int threads) {
-  return L ? list_grid(L, L->cap, k, threads) : dim3((unsigned)tiles_x(g), (unsigned)tiles_y(g), (unsigned)N);
+template <auto K, int THREADS>
+inline dim3 tile_grid(const Geo &g, const LevelLists *L, int N) {
+  return L ? list_grid<K, THREADS>(L, L->cap) : dim3((unsigned)tiles_x(g), (unsigned)tiles_y(g), (unsigned)N);
 }
 
 template <typename T, int N, int FORM>
@@ -84,10 +84,10 @@ struct SolverLaunch {
   }
   // the same two on the tiles that have work (see k_smooth_settled): every
   // block resident at once, its warps striding over the cycle's tiles
-  template <class K>
-  static dim3 settled_grid(const SettledTiles &st, K k) {
-    static const int per_sm = resident_blocks(k, kBlock);
+  template <auto K>
+  static dim3 settled_grid(const SettledTiles &st) {
     constexpr int W = kBlock / 32;
+    const int per_sm = once_per_kernel<K, kBlock>(resident_blocks<decltype(K)>);
     return dim3((unsigned)std::min((st.tx * st.ty + W - 1) / W, st.sms * per_sm));
   }
   static int settled_list(const SettledTiles &st, unsigned what, bool around, bool restart, cudaStream_t s) {
@@ -96,7 +96,7 @@ struct SolverLaunch {
     return 1;
   }
   static int settled_zero(void *x, const Geo &g, const SettledTiles &st, cudaStream_t s) {
-    launch(k_settled_zero<T, N>, settled_grid(st, k_settled_zero<T, N>), kBlock, 0, s, (T *)x, g, st);
+    launch(k_settled_zero<T, N>, settled_grid<k_settled_zero<T, N>>(st), kBlock, 0, s, (T *)x, g, st);
     return 1;
   }
   static int smooth_settled(void *x, const void *rhs, const void *ob, const void *corr, const double *omega,
@@ -105,13 +105,13 @@ struct SolverLaunch {
     for (int p = 0; p < 2 * sweeps; ++p) {
       const T *cr = p == 0 ? (const T *)corr : nullptr;
       if (p == 2 * sweeps - 1)
-        launch(k_smooth_settled<T, N, FORM, true>, settled_grid(st, k_smooth_settled<T, N, FORM, true>), kBlock, 0, s,
+        launch(k_smooth_settled<T, N, FORM, true>, settled_grid<k_smooth_settled<T, N, FORM, true>>(st), kBlock, 0, s,
                (T *)x, (const T *)rhs, (const T *)ob, cr, omega, g, p & 1, (T *)rt, mask, dirty, rho, st, all);
       else if (all)
         launch(k_smooth_fine<T, N, FORM, false>, row_grid((g.W + 2) / 2, g.H + 1), kBlock, 0, s, (T *)x,
                (const T *)rhs, (const T *)ob, cr, omega, g, p & 1, nullptr, mask, MaskDirty{nullptr, 0, 0}, nullptr);
       else
-        launch(k_smooth_settled<T, N, FORM, false>, settled_grid(st, k_smooth_settled<T, N, FORM, false>), kBlock, 0,
+        launch(k_smooth_settled<T, N, FORM, false>, settled_grid<k_smooth_settled<T, N, FORM, false>>(st), kBlock, 0,
                s, (T *)x, (const T *)rhs, (const T *)ob, cr, omega, g, p & 1, nullptr, mask,
                MaskDirty{nullptr, 0, 0}, nullptr, st, all);
     }
@@ -119,13 +119,13 @@ struct SolverLaunch {
   }
   static int resid_settled(const void *x, const void *rhs, const void *ob, const Geo &g, void *rt, uint8_t *mask,
                            double *rho, const MaskDirty &dirty, const SettledTiles &st, bool all, cudaStream_t s) {
-    launch(k_resid_settled<T, N, FORM>, settled_grid(st, k_resid_settled<T, N, FORM>), kBlock, 0, s, (const T *)x,
+    launch(k_resid_settled<T, N, FORM>, settled_grid<k_resid_settled<T, N, FORM>>(st), kBlock, 0, s, (const T *)x,
            (const T *)rhs, (const T *)ob, g, (T *)rt, mask, rho, dirty, st, all);
     return 1;
   }
   static int restrict0(const void *rt, const Geo &gf, const Geo &gc, const void *op1, void *r1, const LevelLists *L1,
                        cudaStream_t s) {
-    const dim3 grid = L1 ? list_grid(L1, L1->cap / N, k_restrict0<T, N>, kTileThreads)
+    const dim3 grid = L1 ? list_grid<k_restrict0<T, N>, kTileThreads>(L1, L1->cap / N)
                          : dim3((unsigned)tiles_x(gc), (unsigned)tiles_y(gc));
     launch(k_restrict0<T, N>, grid, kTileThreads, 0, s, (const T *)rt, gf, gc, (const T *)op1, (T *)r1,
                                                   L1 ? L1->tiles : nullptr, L1 ? L1->count + 1 : nullptr);
@@ -164,13 +164,13 @@ struct SolverLaunch {
       if (p == 0 && zero_start) {
         // v is not read: the pair can write it
         constexpr int th = GS ? kGsThreads : kJ2Threads;
-        const dim3 grid = tile_grid(g, L, N, k_coarse_pair<T, N, true, GS>, th);
+        const dim3 grid = tile_grid<k_coarse_pair<T, N, true, GS>, th>(g, L, N);
         launch(k_coarse_pair<T, N, true, GS>, grid, th, 0, s, (const T *)op, (const T *)r, (const T *)v, (T *)v,
                (const T *)nullptr, g, g, tf);
       } else {
         void *nxt = cur == v ? tmp : v;
         constexpr int th = GS ? kGsThreads : kJ2Threads;
-        const dim3 grid = tile_grid(g, L, N, k_coarse_pair<T, N, false, GS>, th);
+        const dim3 grid = tile_grid<k_coarse_pair<T, N, false, GS>, th>(g, L, N);
         launch(k_coarse_pair<T, N, false, GS>, grid, th, 0, s, (const T *)op, (const T *)r, (const T *)cur, (T *)nxt,
                corr, g, gc, tf);
         corr = nullptr;
@@ -195,12 +195,12 @@ struct SolverLaunch {
     const TileList tf = item_list(L);
     if constexpr (sizeof(T) == 4) {
       constexpr int th = GS ? kGsThreads : kJ2Threads;
-      const dim3 grid = tile_grid(g, L, N, k_coarse_pair_resid<T, N, GS>, th);
+      const dim3 grid = tile_grid<k_coarse_pair_resid<T, N, GS>, th>(g, L, N);
       launch(k_coarse_pair_resid<T, N, GS>, grid, th, 0, s, (const T *)op, (const T *)r, (T *)v, (T *)t, g, tf);
       return 1;
     } else {
       constexpr int th = GS ? kGsThreads : kJ2Threads;
-      const dim3 grid = tile_grid(g, L, N, k_coarse_pair<T, N, true, GS>, th);
+      const dim3 grid = tile_grid<k_coarse_pair<T, N, true, GS>, th>(g, L, N);
       launch(k_coarse_pair<T, N, true, GS>, grid, th, 0, s, (const T *)op, (const T *)r, (const T *)v, (T *)v,
              (const T *)nullptr, g, g, tf);
       return 1 + coarse_resid(op, r, v, g, t, L, s);
@@ -213,7 +213,7 @@ struct SolverLaunch {
   static int coarse_resid(const void *op, const void *r, const void *v, const Geo &g, void *t, const LevelLists *Lv,
                           cudaStream_t s) {
     if (Lv) {
-      launch(k_coarse_resid_tiled<T, N>, list_grid(Lv, Lv->cap, k_coarse_resid_tiled<T, N>, kTileThreads), kTileThreads, 0,
+      launch(k_coarse_resid_tiled<T, N>, list_grid<k_coarse_resid_tiled<T, N>, kTileThreads>(Lv, Lv->cap), kTileThreads, 0,
                                    s, (const T *)op, (const T *)r, (const T *)v, g,
                                                                     (T *)t, item_list(Lv));
     } else {
@@ -225,7 +225,7 @@ struct SolverLaunch {
   static int restrict_(const void *t, const Geo &gf, const Geo &gc, const void *opc, void *rc, const LevelLists *Lc,
                        cudaStream_t s) {
     if (Lc) {
-      launch(k_restrict_tiled<T, N>, list_grid(Lc, Lc->cap, k_restrict_tiled<T, N>, kTileThreads), kTileThreads, 0, s, (const T *)t, gf, gc, (const T *)opc, (T *)rc,
+      launch(k_restrict_tiled<T, N>, list_grid<k_restrict_tiled<T, N>, kTileThreads>(Lc, Lc->cap), kTileThreads, 0, s, (const T *)t, gf, gc, (const T *)opc, (T *)rc,
                                                                item_list(Lc));
     } else {
       const PhaseLaunch L = phase_grid(gc.W + 1, gc.H + 1, N);
@@ -363,12 +363,12 @@ struct Launch {
   }
   static int outer_resid_tiles(const double *u, const float *b, const Geo &g, float *r32, float *u32, double *rho,
                                const SettledTiles &st, cudaStream_t s) {
-    launch(k_outer_resid_tiles<N>, SolverLaunch<float, N, kShifted>::settled_grid(st, k_outer_resid_tiles<N>), kBlock, 0,
+    launch(k_outer_resid_tiles<N>, SolverLaunch<float, N, kShifted>::template settled_grid<k_outer_resid_tiles<N>>(st), kBlock, 0,
            s, u, b, g, r32, u32, rho, st);
     return 1;
   }
   static int outer_update_tiles(double *u, const float *delta, const Geo &g, const SettledTiles &st, cudaStream_t s) {
-    launch(k_outer_update_tiles<N>, SolverLaunch<float, N, kShifted>::settled_grid(st, k_outer_update_tiles<N>), kBlock,
+    launch(k_outer_update_tiles<N>, SolverLaunch<float, N, kShifted>::template settled_grid<k_outer_update_tiles<N>>(st), kBlock,
            0, s, u, delta, g, st);
     return 1;
   }
