@@ -79,7 +79,8 @@ typedef struct {
   int nu1, nu2;        /* pre/post projected smoothing sweeps of the V-cycle, >= 0, nu1+nu2 >= 1 */
   int max_cycles;      /* V-cycle cap per step, >= 1 */
   int coarse_min;      /* coarsen (W, H) to ((W + 1)/2, (H + 1)/2) while the smaller of the two stays >= coarse_min
-                          (>= 1) and the level is not yet mass-dominated (8 tau eps > 4 h^2 on its cells of side h) */
+                          (>= 1) and, at the default 4 and above, the level is not yet mass-dominated (8 tau eps >
+                          4 h^2 on its cells of side h); 1 to 3 give every level */
   int precision;       /* AC_FP64: every array and operation of the solve in FP64.
                           AC_MIXED: FP64 state u and its update; right-hand side, colour
                           means, energy and residual r = b - S u of the defect correction in

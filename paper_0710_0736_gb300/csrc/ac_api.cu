@@ -241,6 +241,7 @@ int64_t settled_host_unknowns(int elem) { return elem == 4 ? 3 << 20 : 1 << 19; 
 #endif
 constexpr int kCoarseSweeps = AC_COARSE_SWEEPS;
 static_assert(kCoarseSweeps >= 2 && kCoarseSweeps % 2 == 0, "coarse sweeps: an even count >= 2");
+constexpr int kDefaultCoarseMin = 4;
 // Level k (cell side h = 2^k) is mass-dominated when 8 tau eps <= kMassRatio
 // h^2.  On cells of side h the Galerkin operator is about h^2 (consistent
 // mass) + tau eps A with A <= 8, so its condition number is at most a small
@@ -250,6 +251,10 @@ static_assert(kCoarseSweeps >= 2 && kCoarseSweeps % 2 == 0, "coarse sweeps: an e
 // 1001 x 751 13 / 12; one level less (8 tau eps = 16 h^2) takes 22, 25 and 28.
 // The levels below cost launches and the serial one-block tail: 1024^2, N = 4
 // 3.73 ms a step with all levels, 2.21 ms with two coarse levels (eps 2).
+// tau and eps enter by their product only.  Over 260 steps (64 x 48 to 2048 x
+// 1024, tau eps 0.01 to 216, lambda 1 and 50, both precisions) against all levels:
+// time 0.87 (64 x 48, tau eps 80: 23 cycles for 21) to 2 times better, 1.16 in
+// the median; a caller can ask for all of them (coarse_min).
 constexpr double kMassRatio = 4.0;
 bool mass_dominated(double te, int level) { return 8.0 * te <= kMassRatio * std::ldexp(1.0, 2 * level); }
 // Sweeps on the coarsest level, in the tail and in tile launches (a pair
@@ -1649,7 +1654,7 @@ int ac_default_params(ac_params *p) {
   p->nu1 = 2;
   p->nu2 = 2;
   p->max_cycles = 200;
-  p->coarse_min = 4;
+  p->coarse_min = kDefaultCoarseMin;
   p->precision = AC_FP64;
   p->projection = AC_PROJ_SIMPLEX;
   return AC_OK;
@@ -1702,9 +1707,11 @@ int ac_create(ac_ctx **out, const ac_params *p) {
   // sides only left 1001 x 751, N = 5 without a coarse level: 90 cycles of
   // plain sweeps to 1e-12 in 6.08 ms, against 13 cycles in 3.68 ms.
   // Coarsening stops at the first level whose system the mass dominates
-  // (kMassRatio): a few sweeps solve that one.
+  // (kMassRatio): a few sweeps solve that one.  A caller who asks for more
+  // levels than the default's gets them all.
+  const bool all_levels = p->coarse_min < kDefaultCoarseMin;
   while ((W < H ? W : H) >= 2 && ((W < H ? W : H) + 1) / 2 >= p->coarse_min &&
-         !mass_dominated(te, (int)S.lv.size() - 1)) {
+         (all_levels || !mass_dominated(te, (int)S.lv.size() - 1))) {
     W = (W + 1) / 2;
     H = (H + 1) / 2;
     Level L;

@@ -57,3 +57,28 @@ def test_early_coarsest_level_is_solved(ac, W, H, N, eps, tau, coarse_min, preci
     for smoother in (ac.AC_SMOOTH_GS3, ac.AC_SMOOTH_JACOBI):
         st = _step(ac, W, H, N, eps, tau, precision, smoother, coarse_min=coarse_min)[1]
         assert st.converged and st.total_cycles <= 18, (smoother, st.total_cycles)
+
+
+@pytest.mark.parametrize("W,H,coarse_min,depths", [(128, 128, 4, (3,)), (128, 128, 1, (5, 8)), (200, 70, 2, (5, 7)),
+                                                   (200, 70, 64, (1,))])
+def test_coarse_min_below_the_default_gives_every_level(ac, W, H, coarse_min, depths):
+    """coarse_min 1 to 3 alone decides the depth; at the default the hierarchy
+    ends where the mass dominates (eps 2, tau 4: on cells of side 4).  The
+    tuner reports the depth: all levels, or 5.  Either way the step is the
+    same minimiser: two solves to 1e-13 differ by at most twice (1 + 4 tau eps)
+    = 33 residuals."""
+    N, img = 3, synth.shapes_image(5, W, H, rect_side=(8, 60), disk_r=(4, 30))
+    b = ac.Batch([dict(W=W, H=H, N=N, eps=2.0, tau=4.0, lam=1.0, tol=1e-10, max_cycles=500, coarse_min=coarse_min)],
+                 n_streams=1)
+    b.set_image(0, img)
+    assert b.tune()[0][2] in depths
+    b.close()
+    u0, out = synth.dirichlet_init(1, (W + 1) * (H + 1), N), []
+    for cm in (4, coarse_min):
+        seg = ac.Segmenter(W, H, N, 2.0, 1.0, 4.0, tol=1e-13, max_cycles=500, coarse_min=cm)
+        seg.set_image(img.astype(np.float64))
+        seg.set_phase(u0)
+        assert seg.step(1).converged
+        out.append(seg.phase())
+        seg.close()
+    assert np.abs(out[0] - out[1]).max() <= 2 * 33 * 1e-13
