@@ -81,7 +81,14 @@ typedef struct {
   int coarse_min;      /* coarsen (W, H) to ((W + 1)/2, (H + 1)/2) while the smaller of the two stays >= coarse_min
                           (>= 1) and, at the default 4 and above, the level is not yet mass-dominated (8 tau eps >
                           4 h^2 on its cells of side h); 1 to 3 give every level */
-  int precision;       /* AC_FP64: every array and operation of the solve in FP64.
+  int precision;       /* AC_FP64: every array of the solve in FP64, and every operation but those of the fine
+                          level's nodal problem that fit 64-bit fixed point (the neighbours' sum, the projection,
+                          the natural residual, the line search's direction).  They are then closer to exact than
+                          the FP64 chain, whose roundings near 1 are 2^-53: z is held in multiples of 2^-57, its
+                          projection too (a phase below 2^-58 is 0 and not free), and neighbours enter the sum in
+                          multiples of 2^-60 (below 2^-7 with fewer relative bits than FP64; an edge of weight 1/2
+                          drops the last bit).  A node with |z| >= 4, a value >= 2 or one that is not finite runs in
+                          FP64 throughout.
                           AC_MIXED: FP64 state u and its update; right-hand side, colour
                           means, energy and residual r = b - S u of the defect correction in
                           double-float arithmetic (about 2^-46 of the terms: GB300 runs FP64

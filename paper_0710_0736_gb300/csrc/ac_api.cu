@@ -253,8 +253,8 @@ constexpr int kDefaultCoarseMin = 4;
 // 3.73 ms a step with all levels, 2.21 ms with two coarse levels (eps 2).
 // tau and eps enter by their product only.  Over 260 steps (64 x 48 to 2048 x
 // 1024, tau eps 0.01 to 216, lambda 1 and 50, both precisions) against all levels:
-// time 0.87 (64 x 48, tau eps 80: 23 cycles for 21) to 2 times better, 1.16 in
-// the median; a caller can ask for all of them (coarse_min).
+// 1.16 times faster in the median, 0.87 at worst (64 x 48, tau eps 80: 23 cycles
+// for 21); a caller can ask for all of them (coarse_min).
 constexpr double kMassRatio = 4.0;
 bool mass_dominated(double te, int level) { return 8.0 * te <= kMassRatio * std::ldexp(1.0, 2 * level); }
 // Sweeps on the coarsest level, in the tail and in tile launches (a pair
@@ -798,7 +798,8 @@ int enqueue_correction(ac_ctx *ctx, Solve &S) {
   // written; curvature: d and the mask read
   const double ls_bytes = bm.n * (bm.ns * (3 + bm.ob) + 1) + l1 + bm.n * (bm.ns + 1);
   AC_RUNB(AC_PROF_LINESEARCH, ls_bytes,
-          o->line_search(S.x, S.ob, S.rt, v1, S.mask, g0, L1.g, S.d, S.d_live, ctx->ls_part, ctx->ls_done, ctx->omega, ctx->s));
+          o->line_search(S.x, S.ob, S.rt, v1, S.mask, g0, L1.g, S.d, S.d_live, ctx->ls_part, ctx->ls_done, ctx->omega,
+                         ctx->s));
   return AC_OK;
 }
 
@@ -849,7 +850,8 @@ bool settled_form(ac_ctx *ctx, Solve &S, int64_t min_unknowns) {
   if (S.lv[0].n * ctx->N < min_unknowns) return false;
   if (S.sampled) {
     if (cudaEventSynchronize(ctx->sample_done) != cudaSuccess) return false;  // the call that follows reports it
-    S.free_frac = std::accumulate(ctx->h_undecided, ctx->h_undecided + ac::kSampleBlocks, 0u) / (double)ac::kSampleNodes;
+    const unsigned *const c = ctx->h_undecided;
+    S.free_frac = std::accumulate(c, c + ac::kSampleBlocks, 0u) / (double)ac::kSampleNodes;
     S.sampled = false;
   }
   return S.free_frac < kSettledFreeFraction;
@@ -1334,8 +1336,8 @@ int enqueue_step_loop(ac_ctx *ctx, cudaGraph_t top, bool energy, StepGraph &sg) 
               o->outer_resid(ctx->u, (const float *)ctx->b, ctx->g0, ctx->r32, ctx->u32, ctx->rho, true, nullptr, 0,
                              ctx->s));
       AC_RUN(AC_PROF_OUTER,
-             (ac::launch(k_ctl_outer, 1, 1, 0, ctx->s, ctx->ctl, ctx->rho, accept, ctx->p.tol, kInnerTolFrac, kInnerReduction,
-                                               ctx->p.max_cycles, kInnerMaxCycles, ctx->p.nu1, h_out),
+             (ac::launch(k_ctl_outer, 1, 1, 0, ctx->s, ctx->ctl, ctx->rho, accept, ctx->p.tol, kInnerTolFrac,
+                         kInnerReduction, ctx->p.max_cycles, kInnerMaxCycles, ctx->p.nu1, h_out),
               1));
       return AC_OK;
     };
@@ -1346,9 +1348,8 @@ int enqueue_step_loop(ac_ctx *ctx, cudaGraph_t top, bool energy, StepGraph &sg) 
     ctx->s = ctx->body_s[0];
     ctx->capturing = &cnt_pass;
     const int64_t xs = fine_slots(ctx->n) * ctx->N;
-    AC_RUN(AC_PROF_OUTER, (ac::launch(k_zero_unless_warm, (unsigned)std::min<int64_t>((xs + 255) / 256, 8 * ctx->sms), 256, 0,
-                                                ctx->s, ctx->ctl, (float *)S.x, xs),
-                           1));
+    const unsigned zero_blocks = (unsigned)std::min<int64_t>((xs + 255) / 256, 8 * ctx->sms);
+    AC_RUN(AC_PROF_OUTER, (ac::launch(k_zero_unless_warm, zero_blocks, 256, 0, ctx->s, ctx->ctl, (float *)S.x, xs), 1));
     rc = solve(1);
     if (rc) return rc;
     AC_RUNB(AC_PROF_OUTER, (double)ctx->n * ctx->N * 20,
@@ -1744,7 +1745,7 @@ int ac_create(ac_ctx **out, const ac_params *p) {
     }
     AC_ALLOC(S.rt, fNs);
     AC_ALLOC(S.mask, (size_t)ctx->n);
-    AC_CUDA(cudaMemsetAsync(S.mask, 0, (size_t)ctx->n, ctx->s));  // read as a hint before the first cycle sets it
+    AC_CUDA(cudaMemsetAsync(S.mask, 0, (size_t)ctx->n, ctx->s));  // the first cycle compares with what it replaces
     if (S.lv.size() > 1) AC_ALLOC(S.d, fNs);
     AC_ALLOC(S.d_live, (size_t)(ctx->n + 31) / 32);
     AC_CUDA(cudaMemsetAsync(S.d_live, 1, (size_t)(ctx->n + 31) / 32, ctx->s));

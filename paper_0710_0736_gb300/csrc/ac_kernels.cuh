@@ -2360,9 +2360,9 @@ constexpr int pair_min_blocks(int elem, bool gs) { return gs ? (elem == 4 ? AC_G
 // (GS) or l1-Jacobi.  vc (nullable, grid gc): the coarser level's correction,
 // added to vin first.
 template <typename T, int N, bool ZERO_IN, bool GS>
-__global__ void __launch_bounds__(GS ? kGsThreads : kJ2Threads, pair_min_blocks(sizeof(T), GS)) k_coarse_pair(const T *__restrict__ op, const T *__restrict__ r,
-                                                                  const T *vin, T *vout, const T *vc, Geo g, Geo gc,
-                                                                  TileList L) {
+__global__ void __launch_bounds__(GS ? kGsThreads : kJ2Threads, pair_min_blocks(sizeof(T), GS))
+    k_coarse_pair(const T *__restrict__ op, const T *__restrict__ r, const T *vin, T *vout, const T *vc, Geo g, Geo gc,
+                  TileList L) {
   pdl_sync();
   for_each_tile(L, g, [&](int tx, int ty, int i, bool dying) {
     const int64_t nc = (int64_t)g.Wn * (g.H + 1);
@@ -2476,9 +2476,9 @@ __device__ __forceinline__ void jacobi2_resid_tile(const T *__restrict__ op, con
 }
 
 template <typename T, int N, bool GS>
-__global__ void __launch_bounds__(GS ? kGsThreads : kJ2Threads, pair_min_blocks(sizeof(T), GS)) k_coarse_pair_resid(const T *__restrict__ op,
-                                                                        const T *__restrict__ r, T *__restrict__ vout,
-                                                                        T *__restrict__ tout, Geo g, TileList L) {
+__global__ void __launch_bounds__(GS ? kGsThreads : kJ2Threads, pair_min_blocks(sizeof(T), GS))
+    k_coarse_pair_resid(const T *__restrict__ op, const T *__restrict__ r, T *__restrict__ vout, T *__restrict__ tout,
+                        Geo g, TileList L) {
   pdl_sync();
   for_each_tile(L, g, [&](int tx, int ty, int i, bool dying) {
     const int64_t nc = (int64_t)g.Wn * (g.H + 1);
@@ -2903,11 +2903,10 @@ struct NodeSum {
 };
 
 template <typename T, int N, int FORM>
-__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 6 : 4) k_ls_dir(const T *__restrict__ x, const T *__restrict__ ob,
-                                                   const T *__restrict__ rt, const T *__restrict__ v1,
-                                                   const uint8_t *__restrict__ mask, Geo gf, Geo gc, int chunks,
-                                                   T *__restrict__ d, uint8_t *__restrict__ live,
-                                                   double *__restrict__ part) {
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 6 : 4)
+    k_ls_dir(const T *__restrict__ x, const T *__restrict__ ob, const T *__restrict__ rt, const T *__restrict__ v1,
+             const uint8_t *__restrict__ mask, Geo gf, Geo gc, int chunks, T *__restrict__ d,
+             uint8_t *__restrict__ live, double *__restrict__ part) {
   pdl_sync();
   NodeSum<T> dot;
   const int64_t nodes = (int64_t)gf.Wn * (gf.H + 1);
@@ -2987,9 +2986,9 @@ __global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 6 : 4) k_ls_dir(const
 // kernel's; *done counts the blocks that have stored theirs (0 between
 // launches).
 template <typename T, int N>
-__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 6 : 5) k_ls_curv(const T *__restrict__ d, const uint8_t *__restrict__ mask, Geo g,
-                                                    int chunks, double *part, unsigned *done,
-                                                    double *__restrict__ omega) {
+__global__ void __launch_bounds__(kBlock, sizeof(T) == 4 ? 6 : 5)
+    k_ls_curv(const T *__restrict__ d, const uint8_t *__restrict__ mask, Geo g, int chunks, double *part, unsigned *done,
+              double *__restrict__ omega) {
   pdl_sync();
   const int blocks = (int)gridDim.x;
   NodeSum<T> dot;

@@ -66,11 +66,10 @@ struct SolverLaunch {
         const T *cr = k == 0 && c == 0 ? (const T *)corr : nullptr;
         if (mask && k == sweeps - 1 && c == 1)
           launch(k_smooth_fine<T, N, FORM, true>, grid, kBlock, 0, s, (T *)x, (const T *)rhs, (const T *)ob, cr, omega,
-                                                                g, c, (T *)rt, mask, dirty, rho);
+                 g, c, (T *)rt, mask, dirty, rho);
         else
           launch(k_smooth_fine<T, N, FORM, false>, grid, kBlock, 0, s, (T *)x, (const T *)rhs, (const T *)ob, cr, omega,
-                                                                 g, c, nullptr, mask, MaskDirty{nullptr, 0, 0},
-                                                                 nullptr);
+                 g, c, nullptr, nullptr, MaskDirty{nullptr, 0, 0}, nullptr);
       }
     return 2 * sweeps;
   }
@@ -79,7 +78,7 @@ struct SolverLaunch {
                    double *rho, int color, const MaskDirty &dirty, cudaStream_t s) {
     const dim3 grid = color < 0 ? row_grid(g.W + 1, g.H + 1) : row_grid((g.W + 2) / 2, g.H + 1);
     launch(k_fine_resid<T, N, FORM>, grid, kBlock, 0, s, (const T *)x, (const T *)rhs, (const T *)ob, g, (T *)rt, mask,
-                                                   rho, color, dirty);
+           rho, color, dirty);
     return 1;
   }
   // the same two on the tiles that have work (see k_smooth_settled): every
@@ -108,12 +107,12 @@ struct SolverLaunch {
         launch(k_smooth_settled<T, N, FORM, true>, settled_grid<k_smooth_settled<T, N, FORM, true>>(st), kBlock, 0, s,
                (T *)x, (const T *)rhs, (const T *)ob, cr, omega, g, p & 1, (T *)rt, mask, dirty, rho, st, all);
       else if (all)
-        launch(k_smooth_fine<T, N, FORM, false>, row_grid((g.W + 2) / 2, g.H + 1), kBlock, 0, s, (T *)x,
-               (const T *)rhs, (const T *)ob, cr, omega, g, p & 1, nullptr, mask, MaskDirty{nullptr, 0, 0}, nullptr);
+        launch(k_smooth_fine<T, N, FORM, false>, row_grid((g.W + 2) / 2, g.H + 1), kBlock, 0, s, (T *)x, (const T *)rhs,
+               (const T *)ob, cr, omega, g, p & 1, nullptr, nullptr, MaskDirty{nullptr, 0, 0}, nullptr);
       else
-        launch(k_smooth_settled<T, N, FORM, false>, settled_grid<k_smooth_settled<T, N, FORM, false>>(st), kBlock, 0,
-               s, (T *)x, (const T *)rhs, (const T *)ob, cr, omega, g, p & 1, nullptr, mask,
-               MaskDirty{nullptr, 0, 0}, nullptr, st, all);
+        launch(k_smooth_settled<T, N, FORM, false>, settled_grid<k_smooth_settled<T, N, FORM, false>>(st), kBlock, 0, s,
+               (T *)x, (const T *)rhs, (const T *)ob, cr, omega, g, p & 1, nullptr, nullptr, MaskDirty{nullptr, 0, 0},
+               nullptr, st, all);
     }
     return 2 * sweeps;
   }
@@ -128,16 +127,15 @@ struct SolverLaunch {
     const dim3 grid = L1 ? list_grid<k_restrict0<T, N>, kTileThreads>(L1, L1->cap / N)
                          : dim3((unsigned)tiles_x(gc), (unsigned)tiles_y(gc));
     launch(k_restrict0<T, N>, grid, kTileThreads, 0, s, (const T *)rt, gf, gc, (const T *)op1, (T *)r1,
-                                                  L1 ? L1->tiles : nullptr, L1 ? L1->count + 1 : nullptr);
+           L1 ? L1->tiles : nullptr, L1 ? L1->count + 1 : nullptr);
     return 1;
   }
   static int galerkin0(const uint8_t *mask, const Geo &gf, const Geo &gc, const Galerkin0Table &tab, void *op,
                        const LevelLists *L1, uint8_t *dirty, cudaStream_t s) {
     const dim3 grid((unsigned)tiles_x(gc), (unsigned)tiles_y(gc));
     launch(k_galerkin0<T, N>, grid, kTileThreads, 0, s, mask, gf, gc, tab, (T *)op, L1 ? L1->flags : nullptr,
-                                                  L1 ? L1->items : nullptr, L1 ? L1->tiles : nullptr,
-                                                  L1 ? L1->count : nullptr, L1 ? L1->dirty : dirty,
-                                                  L1 ? L1->changed : nullptr);
+           L1 ? L1->items : nullptr, L1 ? L1->tiles : nullptr, L1 ? L1->count : nullptr, L1 ? L1->dirty : dirty,
+           L1 ? L1->changed : nullptr);
     return 1;
   }
   static int galerkin(const void *opf, const Geo &gf, const Geo &gc, void *opc, const LevelLists *Lf,
@@ -145,7 +143,7 @@ struct SolverLaunch {
     if (Lc) {
       const dim3 grid((unsigned)tiles_x(gc), (unsigned)tiles_y(gc), (unsigned)N);
       launch(k_galerkin_tiled<T, N>, grid, kTileThreads, 0, s, (const T *)opf, gf, gc, (T *)opc, Lf->flags, Lc->flags,
-                                                         Lc->items, Lc->count, Lf->changed, Lc->changed);
+             Lc->items, Lc->count, Lf->changed, Lc->changed);
     } else {
       const PhaseLaunch L = phase_grid(gc.W + 1, gc.H + 1, N);
       launch(k_galerkin<T, N>, L.grid, L.block, 0, s, (const T *)opf, gf, gc, (T *)opc);
@@ -213,9 +211,8 @@ struct SolverLaunch {
   static int coarse_resid(const void *op, const void *r, const void *v, const Geo &g, void *t, const LevelLists *Lv,
                           cudaStream_t s) {
     if (Lv) {
-      launch(k_coarse_resid_tiled<T, N>, list_grid<k_coarse_resid_tiled<T, N>, kTileThreads>(Lv, Lv->cap), kTileThreads, 0,
-                                   s, (const T *)op, (const T *)r, (const T *)v, g,
-                                                                    (T *)t, item_list(Lv));
+      launch(k_coarse_resid_tiled<T, N>, list_grid<k_coarse_resid_tiled<T, N>, kTileThreads>(Lv, Lv->cap), kTileThreads,
+             0, s, (const T *)op, (const T *)r, (const T *)v, g, (T *)t, item_list(Lv));
     } else {
       const PhaseLaunch L = phase_grid(g.W + 1, g.H + 1, N);
       launch(k_coarse_resid<T, N>, L.grid, L.block, 0, s, (const T *)op, (const T *)r, (const T *)v, g, (T *)t);
@@ -225,8 +222,8 @@ struct SolverLaunch {
   static int restrict_(const void *t, const Geo &gf, const Geo &gc, const void *opc, void *rc, const LevelLists *Lc,
                        cudaStream_t s) {
     if (Lc) {
-      launch(k_restrict_tiled<T, N>, list_grid<k_restrict_tiled<T, N>, kTileThreads>(Lc, Lc->cap), kTileThreads, 0, s, (const T *)t, gf, gc, (const T *)opc, (T *)rc,
-                                                               item_list(Lc));
+      launch(k_restrict_tiled<T, N>, list_grid<k_restrict_tiled<T, N>, kTileThreads>(Lc, Lc->cap), kTileThreads, 0, s,
+             (const T *)t, gf, gc, (const T *)opc, (T *)rc, item_list(Lc));
     } else {
       const PhaseLaunch L = phase_grid(gc.W + 1, gc.H + 1, N);
       launch(k_restrict<T, N>, L.grid, L.block, 0, s, (const T *)t, gf, gc, (const T *)opc, (T *)rc);
@@ -254,19 +251,22 @@ struct SolverLaunch {
               : coarse_tail_t<false>(a, r0, v0, coarse_sweeps, coarsest_sweeps, smem, s);
   }
   static int line_search(const void *x, const void *ob, const void *rt, const void *v1, const uint8_t *mask,
-                         const Geo &gf, const Geo &gc, void *d, uint8_t *live, double *part, unsigned *done, double *omega,
-                         cudaStream_t s) {
-    // one resident set of blocks while a block then takes at most eight
-    // chunks, so that the closing sum of the last block stays near 1 us
-    // (1024^2: 821 blocks); four sets on larger grids, whose blocks differ in
-    // their share of free nodes
-    constexpr int64_t kSet = 152 * 6;
+                         const Geo &gf, const Geo &gc, void *d, uint8_t *live, double *part, unsigned *done,
+                         double *omega, cudaStream_t s) {
+    // a fixed number of blocks, so that the sums are grouped alike on every
+    // device: kLsBlocks while a block then takes at most eight chunks, so that
+    // the closing sum of the last block stays near 1 us (1024^2: 821 blocks);
+    // four times as many on larger grids, whose blocks differ in their share of
+    // free nodes.  kLsBlocks are the float kernels' resident blocks on 152
+    // multiprocessors (6 each); of the FP64 kernels 4 and 5 fit, and 912 blocks
+    // are 1.5 and 1.2 sets.
+    constexpr int64_t kLsBlocks = 912;
     const int64_t all = ((int64_t)(gf.W + 1) * (gf.H + 1) + kBlock - 1) / kBlock;
-    const int64_t want = all <= 8 * kSet ? kSet : 4 * kSet;
+    const int64_t want = all <= 8 * kLsBlocks ? kLsBlocks : 4 * kLsBlocks;
     const int chunks = (int)((all + want - 1) / want);
     const unsigned grid = (unsigned)((all + chunks - 1) / chunks);
-    launch(k_ls_dir<T, N, FORM>, grid, kBlock, 0, s, (const T *)x, (const T *)ob, (const T *)rt, (const T *)v1, mask, gf,
-                                               gc, chunks, (T *)d, live, part);
+    launch(k_ls_dir<T, N, FORM>, grid, kBlock, 0, s, (const T *)x, (const T *)ob, (const T *)rt, (const T *)v1, mask,
+           gf, gc, chunks, (T *)d, live, part);
     launch(k_ls_curv<T, N>, grid, kBlock, 0, s, (const T *)d, mask, gf, chunks, part, done, omega);
     return 2;
   }
@@ -281,9 +281,9 @@ struct SolverLaunch {
       sl = settled_list;
     }
     if constexpr (FORM == kShifted) sz = settled_zero;
-    return SolverOps{(int)sizeof(T), smooth,       resid,        ss, rs, sl, sz, restrict0,   galerkin0,   galerkin,   coarse_smooth,
-                     coarse_resid, coarse_pre_resid, restrict_, coarse_tail,
-                     line_search};
+    return SolverOps{(int)sizeof(T), smooth,       resid,            ss,        rs,          sl,         sz, restrict0,
+                     galerkin0,      galerkin,     coarse_smooth,    coarse_resid, coarse_pre_resid, restrict_,
+                     coarse_tail,    line_search};
   }
 };
 
@@ -350,8 +350,7 @@ struct Launch {
           k_outer_resid_df<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)outer_resid_smem<N>());
       (void)attr;
       launch(k_outer_resid_df<N>, dim3((g.W + 1 + kOrThreads - 3) / (kOrThreads - 2), (g.H + kOrRows) / kOrRows),
-                            kOrThreads, outer_resid_smem<N>(), s, u, b, g, r32, u32, rho, seeds,
-             seeds_x);
+             kOrThreads, outer_resid_smem<N>(), s, u, b, g, r32, u32, rho, seeds, seeds_x);
     }
     else
       launch(k_outer_resid<N>, row_grid(g.W + 1, g.H + 1), kBlock, 0, s, u, b, g, r32, u32, rho);
@@ -363,13 +362,14 @@ struct Launch {
   }
   static int outer_resid_tiles(const double *u, const float *b, const Geo &g, float *r32, float *u32, double *rho,
                                const SettledTiles &st, cudaStream_t s) {
-    launch(k_outer_resid_tiles<N>, SolverLaunch<float, N, kShifted>::template settled_grid<k_outer_resid_tiles<N>>(st), kBlock, 0,
-           s, u, b, g, r32, u32, rho, st);
+    launch(k_outer_resid_tiles<N>, SolverLaunch<float, N, kShifted>::template settled_grid<k_outer_resid_tiles<N>>(st),
+           kBlock, 0, s, u, b, g, r32, u32, rho, st);
     return 1;
   }
   static int outer_update_tiles(double *u, const float *delta, const Geo &g, const SettledTiles &st, cudaStream_t s) {
-    launch(k_outer_update_tiles<N>, SolverLaunch<float, N, kShifted>::template settled_grid<k_outer_update_tiles<N>>(st), kBlock,
-           0, s, u, delta, g, st);
+    launch(k_outer_update_tiles<N>,
+           SolverLaunch<float, N, kShifted>::template settled_grid<k_outer_update_tiles<N>>(st), kBlock, 0, s, u, delta,
+           g, st);
     return 1;
   }
   static int composite(const double *u, const double *c, const Geo &g, int r, int rounded, float *out,
