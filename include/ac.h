@@ -149,8 +149,9 @@ typedef struct {
                                       0.5 n N 4 (AC_MIXED) */
   double bytes[AC_PROF_COUNT];     /* algorithmic HBM bytes of the class's launches while profiling was on:
                                       every array element a launch is defined on read once and written once
-                                      (dense counts: rows the coarse kernels skip are still counted; fine
-                                      tiles that a cycle does not visit are not) */
+                                      (dense counts: rows the coarse kernels skip, and nodes without a free
+                                      phase that the line search skips, are still counted; fine tiles that a
+                                      cycle or an outer pass does not visit are not) */
 } ac_profile;
 
 /* Defaults: tol 1e-10, nu1 = nu2 = 2, max_cycles 200, coarse_min 4, AC_FP64,
