@@ -256,13 +256,18 @@ constexpr int kDefaultCoarseMin = 4;
 // 1.16 times faster in the median, 0.87 at worst (64 x 48, tau eps 80: 23 cycles
 // for 21); a caller can ask for all of them (coarse_min).
 constexpr double kMassRatio = 4.0;
-bool mass_dominated(double te, int level) { return 8.0 * te <= kMassRatio * std::ldexp(1.0, 2 * level); }
+bool mass_ratio_below(double ratio, double te, int level) { return 8.0 * te <= ratio * std::ldexp(1.0, 2 * level); }
+bool mass_dominated(double te, int level) { return mass_ratio_below(kMassRatio, te, level); }
 // Sweeps on the coarsest level, in the tail and in tile launches (a pair
 // each); a hierarchy that ends early (a small picture, coarse_min, a tuned
-// depth) leaves a system that is not mass-dominated.  The tail then runs the
-// colours forward in every sweep: 60 passes that count, against 41 forward and
-// backward in turn, which left it half solved (48 x 40, N = 3, eps 8, tau 64
-// mixed: 14 cycles a step against 47).
+// depth) leaves a system that is not mass-dominated.  The more it lacks mass,
+// the more colour passes the tail needs: forward and backward in turn 20 sweeps
+// are 41 passes that count, all forward 60.  Over 70 small systems with r = 8
+// tau eps / h^2 on the last level, cycles a step in turn / forward: r <= 40 the
+// same within two either way (10 / 10 at 13.5, 16 / 17 at 25, 20 / 21 at 40) and
+// a tenth of the time less in turn; from r = 50 on forward is needed (mixed 46 / 12 at
+// 50, 47 / 14 at 64, 133 / 84 at 500).
+constexpr double kForwardRatio = 45.0;
 constexpr int kDominatedTailSweeps = 6, kDominatedSweeps = 4, kCoarsestSweeps = 20;
 bool ends_dominated(const Solve &S) { return mass_dominated(S.lv[0].g.te, S.depth - 1); }
 // AC_MIXED: inner FP32 solve to max(0.9 tol, 1e-5 rho_outer) ...  The inner
@@ -662,7 +667,7 @@ int coarse_vcycle(ac_ctx *ctx, Solve &S, int k, void **res) {
       ops += 4.0 * (double)S.lv[k + l].n * ns;
     }
     const int sweeps = ends_dominated(S) ? kDominatedTailSweeps : kCoarsestSweeps;
-    a.forward = !ends_dominated(S);
+    a.forward = !mass_ratio_below(kForwardRatio, S.lv[0].g.te, S.depth - 1);
     AC_RUNB(AC_PROF_COARSE, ops + 2 * lk,
             o->coarse_tail(a, L.r, L.v, kCoarseSweeps, sweeps, smem, S.coarse_gs, ctx->s));
     *res = L.v;
