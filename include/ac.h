@@ -294,10 +294,11 @@ int ac_set_coarse_smoother(ac_ctx *ctx, int mode);
  *     (ac_set_coarse_tiling; with AC_TILES_AUTO that is every image whose
  *     coarse levels are too small for tiles, e.g. 1024^2 and below at N <= 8),
  *     and on the host otherwise, as it is for an image of at least 3 M
- *     unknowns (0.5 M in AC_FP64) with few free nodes -- as the last cycle
- *     found them, or, after ac_set_phase, as a sample of the new field's nodes
- *     has two phases or more: the host loop then visits only the fine tiles that
- *     can change (ac_set_coarse_tiling);
+ *     unknowns (0.5 M in AC_FP64) with few free nodes -- below a fifth in the
+ *     last cycle, or, after ac_set_phase, below 0.6 of a sample of the new
+ *     field's nodes with two phases or more (a solve leaves a third of them):
+ *     the host loop then visits only the fine tiles that can change
+ *     (ac_set_coarse_tiling);
  *   AC_LOOP_HOST: always on the host.
  * If the graph cannot be captured or instantiated (a driver without
  * conditional nodes), the context switches itself to AC_LOOP_HOST and the
